@@ -155,7 +155,8 @@ typedef struct {
   int res_cluster;   /* resident solver: CTAs per thread-block cluster, 1..16 */
                      /* (0 = 4)                                              */
   int res_cta_octs;  /* resident solver: a level of at most this many octs is */
-                     /* solved by one CTA alone (0 = 2048, < 0 = never)      */
+                     /* solved by one CTA alone (0 = 2048 for ATS_PREC_MIXED, */
+                     /* 128 for ATS_PREC_FP64; < 0 = never)                  */
   int res_max_octs;  /* ATS_SCHED_AUTO: levels above this many octs take the  */
                      /* whole-GPU form or the tick path (see ATS_SCHED_AUTO) */
                      /* (0 = 16384 for ATS_PREC_MIXED, 2048 for              */
@@ -171,7 +172,8 @@ typedef struct {
                      /* memory (L2).  The FP64 bulk always uses global.      */
   int res_cluster_big; /* resident solver: CTAs per cluster for the levels    */
                      /* whose runs on res_cluster_mid CTAs would not fit     */
-                     /* their shared memory, or whose estimated work         */
+                     /* their shared memory (ATS_PREC_FP64: would exceed     */
+                     /* 128 octs per CTA), or whose estimated work         */
                      /* exceeds res_big_work (0 = 16; < 0 = none)           */
   int res_big_work;  /* resident solver: a level of more than res_cta_octs   */
                      /* octs also takes the larger clusters when its        */
@@ -179,7 +181,8 @@ typedef struct {
                      /* h = dt / (2 dx^2), exceeds this (0 = no work rule)   */
   int res_cluster_mid; /* resident solver: CTAs per cluster for the levels    */
                      /* whose runs on res_cluster CTAs would not fit their   */
-                     /* shared memory but whose runs on this many would     */
+                     /* shared memory (ATS_PREC_FP64: 128 octs per CTA)      */
+                     /* but whose runs on this many would     */
                      /* (0 = 8; < 0 = none: they take res_cluster_big);     */
                      /* used only between res_cluster and res_cluster_big   */
   int cg_form;       /* resident solver, mixed precision: how each CG step    */
@@ -214,15 +217,15 @@ typedef struct {
  *   estimated work (after a completed run, their measured SM-time).  Not for the paper stopping rule (ATS_STOP_PAPER
  *   takes the tick path). */
 #define ATS_SCHED_AUTO 0     /* resident solver for levels up to res_max_octs octs; */
-        /* above it, FP32 bulk: the whole-GPU form (see ATS_SCHED_GRID) for a level */
-        /* of at most 1 100 octs per CTA of that form (167 200 octs on 152 SMs),    */
-        /* the tick path for larger levels and for FP64                             */
+        /* above it the whole-GPU form (see ATS_SCHED_GRID): FP64 for every level,   */
+        /* FP32 bulk for a level of at most 1 100 octs per CTA of that form (167 200 */
+        /* octs on 152 SMs) and the tick path for larger ones                        */
 #define ATS_SCHED_TICK 1     /* the tick path for every level                    */
 #define ATS_SCHED_RESIDENT 2 /* the resident solver for every level              */
-#define ATS_SCHED_GRID 3     /* as AUTO, and every level above res_max_octs (FP32  */
-        /* bulk) on the whole-GPU form of the resident solver: one cooperative     */
-        /* launch, one CTA per SM, each CTA's run of octs with its CG arrays in     */
-        /* shared memory, the faces across runs and the per-step sums through       */
+#define ATS_SCHED_GRID 3     /* as AUTO, and every level above res_max_octs on the   */
+        /* whole-GPU form of the resident solver: one cooperative launch, one CTA    */
+        /* per SM, each CTA's run of octs with its CG arrays in shared memory (FP64: */
+        /* in global memory), the faces across runs and the per-step sums through   */
         /* global memory, steps ordered by a grid barrier whose waits give up after */
         /* a bounded number of polls (the solve then ends with ATS_ERR_TIMEOUT);    */
         /* such levels run one after another, after the other resident solves.     */

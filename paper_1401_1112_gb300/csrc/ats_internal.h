@@ -212,12 +212,12 @@ struct ResArgs {
   // whole-GPU form (launch_resident_grid): every CTA of one cooperative
   // launch works on gq[0], gq[1], ... in turn; gbar[0] = the arrivals at
   // its grid barriers so far (zeroed before the launch; gbar[1] unused),
-  // gpart = [2][grid + 1][3] (hi, lo) pairs: per buffer, each CTA's partial
+  // gpart = [2][grid + 1][3] sums (FP32 bulk: (hi, lo) pairs): per buffer, each CTA's partial
   // sums (the last row unused); *gerr set when a barrier wait gave up
   const int32_t *gq;
   int n_gq;
   unsigned *gbar;
-  float *gpart;
+  double *gpart;
   int *gerr;
   int g_expect;  // arrivals a grid barrier waits for (0: every CTA of the launch)
   // FP32-bulk kernels: where each solve's result goes (x, or 2 x' - E^n for
@@ -230,14 +230,13 @@ struct ResArgs {
 // One resident launch on st of the FP64 solver (CG state in global memory):
 // clusters of `cluster` CTAs of `threads` threads (256 or 512), `grid` CTAs
 // in all (a multiple of `cluster`) when the cluster queue is not empty, else
-// `grid` single CTAs.  fp64 = false: cudaErrorInvalidValue (the FP32-bulk
-// solver is launch_resident_smem).
-cudaError_t launch_resident(bool fp64, int threads, int cluster, int grid, const ResArgs &a, cudaStream_t st,
+// `grid` single CTAs.
+cudaError_t launch_resident(int threads, int cluster, int grid, const ResArgs &a, cudaStream_t st,
                             bool cta_only = false);
 // Clusters of that shape resident at once on the current device (0: none).
-int resident_max_clusters(bool fp64, int threads, int cluster);
+int resident_max_clusters(int threads, int cluster);
 // CTAs of the single-CTA kernel resident per SM.
-int resident_cta_blocks(bool fp64, int threads);
+int resident_cta_blocks(int threads);
 // The resident solver of FP32-bulk solves with each CTA's K, z, p in shared
 // memory: a.cap octs per CTA (resident_smem_cap gives the largest that fits;
 // 0 keeps every array in global memory, with the same arithmetic), one CTA
@@ -249,19 +248,18 @@ cudaError_t launch_resident_smem(int threads, int cluster, int grid, const ResAr
                                  bool cta_only = false, int priority = 0);
 int resident_smem_clusters(int threads, int cluster, int cap);
 int resident_smem_cap(int threads, int device);
-// The whole-GPU form of the shared-memory solver (FP32 bulk, 512-thread CTAs
-// only): one cooperative launch of `grid` CTAs (at most resident_grid_ctas,
-// 0 for other CTA sizes) solves gq[0, n_gq) one
-// level at a time, each level split into `grid` contiguous runs; sums and
+// The whole-GPU form of the resident solver of either bulk precision
+// (512-thread CTAs): one cooperative launch of `grid` CTAs (at most
+// resident_grid_ctas) solves gq[0, n_gq) one level at a time, each level split into `grid` contiguous runs; sums and
 // steps go through global memory and a grid barrier whose waits end after a
 // bounded number of polls (then *gerr is set and the solve ends with
 // ATS_ERR_TIMEOUT).
-cudaError_t launch_resident_grid(int threads, int grid, const ResArgs &a, cudaStream_t st);
+cudaError_t launch_resident_grid(bool fp64, int grid, const ResArgs &a, cudaStream_t st);
 // A one-thread kernel on st that returns after about ns nanoseconds (bounded
 // by a fixed number of clock reads): the work queued behind it on st starts
 // that much later.
 cudaError_t launch_hold(unsigned long long ns, cudaStream_t st);
-int resident_grid_ctas(int threads, int device);
+int resident_grid_ctas(bool fp64, int device);
 // Octs per CTA up to which the shared-memory solver keeps all six CG arrays
 // (K, z, p, D, q, e) of a CTA's run in shared memory.
 int resident_six_cap();

@@ -330,7 +330,7 @@ __device__ __forceinline__ void in_oct_faces(const T (&K)[8], const T (&v)[8], T
 
 // k_op, CG phase, out-of-oct face DIR: p_new of the neighbour's facing cells
 // is formed on the fly from its z and p_old.
-template <int DIR, typename T, bool kCoh = false>
+template <int DIR, typename T>
 __device__ __forceinline__ void op_face(int n, const T *__restrict__ KT, const T *__restrict__ z,
                                         const T *__restrict__ pold, bool first, T beta, T h,
                                         const T (&K)[8], T (&off)[8]) {
@@ -338,8 +338,8 @@ __device__ __forceinline__ void op_face(int n, const T *__restrict__ KT, const T
   if (n < 0) return;
   T Kn[8], Zn[8], Pn[8];
   ld_face<A, NB>(KT + 8 * n, Kn);
-  ldvf<A, NB, kCoh>(z + 8 * n, Zn);
-  if (!first) ldvf<A, NB, kCoh>(pold + 8 * n, Pn);
+  ld_face<A, NB>(z + 8 * n, Zn);
+  if (!first) ld_face<A, NB>(pold + 8 * n, Pn);
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     if (((c >> A) & 1) != S) continue;
@@ -480,11 +480,11 @@ __device__ __forceinline__ void ref_oct_values(const SolveDev &sd, int o, bool w
   }
 }
 
-template <typename T, bool kCoh = false>
+template <typename T>
 __device__ __forceinline__ void op_refine_oct(const SolveDev &sd, int o, bool want_x, Acc<T> &rr,
                                               Acc<T> &xx, Acc<T> &rz) {
   T zo[8], dv[8];
-  ref_oct_values<T, kCoh>(sd, o, want_x, rr, xx, rz, zo, dv);
+  ref_oct_values<T>(sd, o, want_x, rr, xx, rz, zo, dv);
   st8((T *)sd.z + 8 * o, zo);
   st8((T *)sd.dg + 8 * o, dv);
 }
@@ -531,6 +531,13 @@ struct Slot<float> {
     float2 v = make_float2(a.s, a.c);
     *reinterpret_cast<float2 *>(p) = v;
   }
+  static __device__ __forceinline__ Acc<float> load(const double *p) {
+    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+    Acc<float> a;
+    a.s = v.x;
+    a.c = v.y;
+    return a;
+  }
   static __device__ __forceinline__ void load_add(const double *p, Acc<float> &a) {
     const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
     float s, e;
@@ -542,6 +549,11 @@ struct Slot<float> {
 template <>
 struct Slot<double> {
   static __device__ __forceinline__ void store(double *p, const Acc<double> &a) { *p = a.s; }
+  static __device__ __forceinline__ Acc<double> load(const double *p) {
+    Acc<double> a;
+    a.s = __ldcg(p);
+    return a;
+  }
   static __device__ __forceinline__ void load_add(const double *p, Acc<double> &a) { a.s += __ldcg(p); }
 };
 
@@ -642,20 +654,20 @@ struct OpOwn {
   T K[8], z[8], pp[8], d[8];
 };
 
-template <typename T, bool kCoh = false>
+template <typename T>
 __device__ __forceinline__ void op_load_own(const SolveDev &sd, int o, bool first, const T *__restrict__ pold,
                                             OpOwn<T> &w) {
   load_nbr6(sd.nbr, o, w.nb);
   check_nbr6(w.nb, sd.n_oct);
   ld8_ro((const T *)sd.KT + 8 * o, w.K);
-  ldv8<kCoh>((const T *)sd.z + 8 * o, w.z);
-  ldv8<kCoh>((const T *)sd.dg + 8 * o, w.d);
-  if (!first) ldv8<kCoh>(pold + 8 * o, w.pp);
+  ld8_ro((const T *)sd.z + 8 * o, w.z);
+  ld8_ro((const T *)sd.dg + 8 * o, w.d);
+  if (!first) ld8_ro(pold + 8 * o, w.pp);
 }
 
 // k_op, CG phase: p_new = z + beta p_old (first: z), q = (I + dt A) p_new,
 // partial p_new . q (per-oct FP32 sum, carried error-free across octs).
-template <typename T, bool kCoh = false>
+template <typename T>
 __device__ __forceinline__ void op_compute(const SolveDev &sd, int o, const OpOwn<T> &w, T h, T beta, bool first,
                                            const T *__restrict__ pold, T *__restrict__ pnew, Acc<T> &pq) {
   const T *__restrict__ KT = (const T *)sd.KT;
@@ -667,12 +679,12 @@ __device__ __forceinline__ void op_compute(const SolveDev &sd, int o, const OpOw
 #pragma unroll
   for (int c = 0; c < 8; ++c) off[c] = T(0);
   in_oct_faces(w.K, pv, h, off);
-  op_face<0, T, kCoh>(w.nb[0], KT, z, pold, first, beta, h, w.K, off);
-  op_face<1, T, kCoh>(w.nb[1], KT, z, pold, first, beta, h, w.K, off);
-  op_face<2, T, kCoh>(w.nb[2], KT, z, pold, first, beta, h, w.K, off);
-  op_face<3, T, kCoh>(w.nb[3], KT, z, pold, first, beta, h, w.K, off);
-  op_face<4, T, kCoh>(w.nb[4], KT, z, pold, first, beta, h, w.K, off);
-  op_face<5, T, kCoh>(w.nb[5], KT, z, pold, first, beta, h, w.K, off);
+  op_face<0, T>(w.nb[0], KT, z, pold, first, beta, h, w.K, off);
+  op_face<1, T>(w.nb[1], KT, z, pold, first, beta, h, w.K, off);
+  op_face<2, T>(w.nb[2], KT, z, pold, first, beta, h, w.K, off);
+  op_face<3, T>(w.nb[3], KT, z, pold, first, beta, h, w.K, off);
+  op_face<4, T>(w.nb[4], KT, z, pold, first, beta, h, w.K, off);
+  op_face<5, T>(w.nb[5], KT, z, pold, first, beta, h, w.K, off);
   T local = T(0), qv[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
@@ -693,16 +705,8 @@ struct UpdOwn {
   T p[8], q[8], d[8], z[8], e[8];
 };
 
-template <typename T, bool kCoh = false>
+template <typename T>
 __device__ __forceinline__ void upd_load_own(const SolveDev &sd, int o, const T *__restrict__ p, UpdOwn<T> &w) {
-  if (kCoh) {  // every vector is rewritten within a resident launch
-    ldc8(p + 8 * o, w.p);
-    ldc8((const T *)sd.q + 8 * o, w.q);
-    ldc8((const T *)sd.dg + 8 * o, w.d);
-    ldc8((const T *)sd.z + 8 * o, w.z);
-    ldc8((const T *)sd.e + 8 * o, w.e);
-    return;
-  }
   // p, q (this tick's k_op) and D (a refinement pass) are read-only here
   ld8_ro(p + 8 * o, w.p);
   ld8_ro((const T *)sd.q + 8 * o, w.q);
@@ -1701,7 +1705,8 @@ int tick_blocks_per_sm(bool fp64, bool paper) {
 // later one (z, p, D, x) is read with ld.global.cg after the step's cluster
 // barrier (release / acquire at cluster scope); arrays no step writes (K, the
 // neighbour table, face coefficients, b, diagonal extras) take the read-only
-// path.
+// path.  The FP32 bulk keeps its CG state in shared memory, the FP64 bulk in
+// global memory (L2); each has its own section below.
 
 namespace {
 
@@ -1815,6 +1820,99 @@ __device__ __forceinline__ bool cg_beta(ResState &st, const Acc<T> &rz_tot, cons
   return rr <= st.inner_target * st.inner_target || rz_new == 0.0;
 }
 
+// Decisions after a true-residual pass, from its sums r.r, x.x and r.z (FP64).
+__device__ __forceinline__ void refine_decision(ResState &st, const SolveDev &sd, double rr, double xx, double rz) {
+  const double rnorm = sqrt(rr), xnorm = sqrt(xx);
+  if (st.refines == 0) st.r0 = rnorm;
+  st.refines += 1;
+  st.rnorm = rnorm;
+  st.xnorm = xnorm;
+  const double target = sd.tol * (sd.stop_rule == ATS_STOP_CERTIFIED ? xnorm : st.r0);
+  if (st.final_pass) {
+    st.phase = kDone;
+  } else if (!isfinite(rnorm)) {
+    st.status = ATS_ERR_BREAKDOWN;
+    st.phase = kDone;
+  } else if (rnorm <= target) {
+    st.phase = kDone;
+  } else if (st.refines > sd.max_refine) {
+    st.status = ATS_ERR_NOT_CONVERGED;
+    st.phase = kDone;
+  } else if (!(rz > 0.0)) {
+    st.status = ATS_ERR_BREAKDOWN;
+    st.phase = kDone;
+  } else {
+    st.phase = kInner;
+    st.rz = rz;
+    st.rzf = (float)rz;
+    st.first = 1;
+    st.inner_iters = 0;
+    st.inner_target = fmax(sd.inner_rtol * rnorm, sd.final_safety * target);
+    st.t2f = (float)(st.inner_target * st.inner_target);
+  }
+}
+
+// Decisions after a CG step (conv: the inner solve has converged).
+__device__ __forceinline__ void step_decision(ResState &st, const SolveDev &sd, bool conv) {
+  st.iters += 1;
+  st.inner_iters += 1;
+  st.first = 0;
+  if (conv) {
+    st.phase = kRefine;
+  } else if (st.iters >= sd.max_iter) {
+    st.status = ATS_ERR_NOT_CONVERGED;
+    st.final_pass = 1;
+    st.phase = kRefine;
+  } else if (st.inner_iters >= sd.inner_max) {
+    st.phase = kRefine;  // restart from the true residual
+  }
+  if (st.phase == kRefine) st.n_xpe += 1;
+}
+
+// A whole-GPU barrier gave up (thread 0): the solve ends with ATS_ERR_TIMEOUT.
+__device__ __forceinline__ void res2_timeout(ResState &st) {
+  st.status = ATS_ERR_TIMEOUT;
+  st.phase = kDone;
+}
+
+// The final state of solve s of n octs (thread 0 of the group's first CTA).
+__device__ void res_finish(const ResArgs &a, int s, const ResState &st, int n) {
+  SolveScalars f;
+  memset(&f, 0, sizeof(f));
+  f.phase = kDone;
+  f.iters = st.iters;
+  f.inner_iters = st.inner_iters;
+  f.refines = st.refines;
+  f.status = st.status;
+  f.final_pass = st.final_pass;
+  f.ticks = st.n_op + st.iters + st.refines;  // group steps taken
+  f.rz = st.rz;
+  f.r0 = st.r0;
+  f.inner_target = st.inner_target;
+  f.rnorm = st.rnorm;
+  f.xnorm = st.xnorm;
+  a.final_sc[s] = f;
+  if (a.t_solve) a.t_solve[2 * s + 1] = globaltimer_ns();
+  if (a.cells) {
+    const unsigned long long N = 8ull * (unsigned long long)n;
+    atomicAdd(a.cells + 0, N * (unsigned long long)(st.n_op - st.n_first));
+    atomicAdd(a.cells + 4, N * (unsigned long long)st.n_first);
+    atomicAdd(a.cells + 1, N * (unsigned long long)st.refines);
+    atomicAdd(a.cells + 2, N * (unsigned long long)st.iters);
+    atomicAdd(a.cells + 3, N * (unsigned long long)st.n_xpe);
+  }
+}
+
+// A solve of a whole-GPU launch that is not started because an earlier barrier
+// wait of the launch gave up: CTA 0 records it as timed out.
+__device__ void res_never_ran(const ResArgs &a, int s) {
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  SolveScalars f;
+  memset(&f, 0, sizeof(f));
+  f.phase = kDone;
+  f.status = ATS_ERR_TIMEOUT;
+  a.final_sc[s] = f;
+}
 
 // Sums of NA accumulators over the group: this CTA alone, or every CTA of the
 // cluster.  Thread 0 of each CTA ends with the group totals in `out`.  The
@@ -1902,216 +2000,7 @@ __device__ __forceinline__ void res_xpe_oct(const SolveDev &sd, int o) {
 // them while the group waits, and the GB300's FP64 pipe makes an FP64
 // quotient the longer wait.  A refinement pass's decisions are FP64.
 
-// One solve by one group: the refinement / inner-CG state machine of the tick
-// kernels (k_ref, k_op, k_upd), with its decisions taken right after each sum.
-template <typename T, bool kCluster>
-__device__ void res_solve(const ResArgs &a, int s, ResShared<T> &sh, int &buf) {
-  constexpr int wd = (int)(sizeof(SolveDev) / 8);
-  for (int w = threadIdx.x; w < wd; w += blockDim.x)
-    reinterpret_cast<unsigned long long *>(&sh.sd)[w] = reinterpret_cast<const unsigned long long *>(a.solves + s)[w];
-  const unsigned cs = kCluster ? cl_size() : 1u, cr = kCluster ? cl_rank() : 0u;
-  if (threadIdx.x == 0) {
-    ResState z;
-    memset(&z, 0, sizeof(z));
-    z.phase = kRefine;
-    z.status = ATS_OK;
-    sh.st = z;
-    if (a.t_solve && cr == 0) a.t_solve[2 * s] = globaltimer_ns();
-  }
-  __syncthreads();
-  const SolveDev &sd = sh.sd;
-  const int n = sd.n_oct;
-  const int chunk = (int)((n + (int)cs - 1) / (int)cs);
-  const int lo = min(n, (int)cr * chunk), hi = min(n, lo + chunk);
-  const int o0 = lo + (int)threadIdx.x, stride = (int)blockDim.x;
-  const T h = (T)sd.h;
-  const bool want_x = sd.stop_rule == ATS_STOP_CERTIFIED;
-  const bool f32 = sizeof(T) == 4 && a.cg_scalars == 0;
-  for (;;) {
-    const int phase = sh.st.phase;
-    if (phase == kDone) break;
-    if (phase == kRefine) {
-      // FP64 true residual of x, z = D^-1 r and D; sums r.r, x.x, r.z
-      Acc<T> acc[3], tot[3];
-      for (int o = o0; o < hi; o += stride) op_refine_oct<T, true>(sd, o, want_x, acc[0], acc[1], acc[2]);
-      group_sum<T, 3, kCluster>(acc, sh, buf, tot);
-      if (threadIdx.x == 0) {
-        ResState &st = sh.st;
-        const double rnorm = sqrt(tot[0].get()), xnorm = sqrt(tot[1].get()), rz = tot[2].get();
-        if (st.refines == 0) st.r0 = rnorm;
-        st.refines += 1;
-        st.rnorm = rnorm;
-        st.xnorm = xnorm;
-        const double target = sd.tol * (sd.stop_rule == ATS_STOP_CERTIFIED ? xnorm : st.r0);
-        if (st.final_pass) {
-          st.phase = kDone;
-        } else if (!isfinite(rnorm)) {
-          st.status = ATS_ERR_BREAKDOWN;
-          st.phase = kDone;
-        } else if (rnorm <= target) {
-          st.phase = kDone;
-        } else if (st.refines > sd.max_refine) {
-          st.status = ATS_ERR_NOT_CONVERGED;
-          st.phase = kDone;
-        } else if (!(rz > 0.0)) {
-          st.status = ATS_ERR_BREAKDOWN;
-          st.phase = kDone;
-        } else {
-          st.phase = kInner;
-          st.rz = rz;
-          st.rzf = (float)rz;
-          st.first = 1;
-          st.inner_iters = 0;
-          st.inner_target = fmax(sd.inner_rtol * rnorm, sd.final_safety * target);
-          st.t2f = (float)(st.inner_target * st.inner_target);
-        }
-      }
-      __syncthreads();
-      continue;
-    }
-    // inner CG iteration, step 1: p = z + beta p, q = (I + dt A) p, sum p.q
-    const bool first = sh.st.first != 0;
-    const T beta = sizeof(T) == 4 ? (T)sh.st.betaf : (T)sh.st.beta;
-    const int pcur = sh.st.pcur;
-    const T *pold = (const T *)(pcur ? sd.p1 : sd.p0);
-    T *pnew = (T *)(pcur ? sd.p0 : sd.p1);
-    {
-      Acc<T> acc[1], tot[1];
-      OpOwn<T> w;
-      for (int o = o0; o < hi; o += stride) {
-        op_load_own<T, true>(sd, o, first, pold, w);
-        op_compute<T, true>(sd, o, w, h, beta, first, pold, pnew, acc[0]);
-      }
-      group_sum<T, 1, kCluster>(acc, sh, buf, tot);
-      if (threadIdx.x == 0) {
-        ResState &st = sh.st;
-        st.n_op += 1;
-        st.n_first += first ? 1 : 0;
-        cg_alpha(st, tot[0], f32);
-      }
-      __syncthreads();
-    }
-    if (sh.st.phase == kDone) break;
-    // step 2: e += alpha p, r = D z - alpha q, z = D^-1 r; sums r.z, r.r
-    {
-      const T alpha = sizeof(T) == 4 ? (T)sh.st.alphaf : (T)sh.st.alpha;
-      Acc<T> acc[2], tot[2];
-      UpdOwn<T> w;
-      float none = 0.f;
-      for (int o = o0; o < hi; o += stride) {
-        upd_load_own<T, true>(sd, o, pnew, w);
-        upd_compute<T, false>(sd, o, w, alpha, acc[0], acc[1], none);
-      }
-      group_sum<T, 2, kCluster>(acc, sh, buf, tot);
-      if (threadIdx.x == 0) {
-        ResState &st = sh.st;
-        st.iters += 1;
-        st.inner_iters += 1;
-        st.first = 0;
-        st.pcur ^= 1;
-        const bool conv = cg_beta(st, tot[0], tot[1], f32);
-        if (conv) {
-          st.phase = kRefine;
-        } else if (st.iters >= sd.max_iter) {
-          st.status = ATS_ERR_NOT_CONVERGED;
-          st.final_pass = 1;
-          st.phase = kRefine;
-        } else if (st.inner_iters >= sd.inner_max) {
-          st.phase = kRefine;  // restart from the true residual
-        }
-        if (st.phase == kRefine) st.n_xpe += 1;
-      }
-      __syncthreads();
-    }
-    if (sh.st.phase == kRefine) {
-      // the inner solve ends: x += e, e = 0; the next residual pass reads the
-      // neighbours' x, so the whole group passes a barrier first
-      for (int o = o0; o < hi; o += stride) res_xpe_oct<T>(sd, o);
-      group_barrier<kCluster>();
-    }
-  }
-  if (threadIdx.x == 0 && cr == 0) {
-    const ResState &st = sh.st;
-    SolveScalars f;
-    memset(&f, 0, sizeof(f));
-    f.phase = kDone;
-    f.iters = st.iters;
-    f.inner_iters = st.inner_iters;
-    f.refines = st.refines;
-    f.status = st.status;
-    f.final_pass = st.final_pass;
-    f.ticks = st.n_op + st.iters + st.refines;  // group steps taken
-    f.rz = st.rz;
-    f.r0 = st.r0;
-    f.inner_target = st.inner_target;
-    f.rnorm = st.rnorm;
-    f.xnorm = st.xnorm;
-    a.final_sc[s] = f;
-    if (a.t_solve) a.t_solve[2 * s + 1] = globaltimer_ns();
-    if (a.cells) {
-      const unsigned long long N = 8ull * (unsigned long long)n;
-      atomicAdd(a.cells + 0, N * (unsigned long long)(st.n_op - st.n_first));
-      atomicAdd(a.cells + 4, N * (unsigned long long)st.n_first);
-      atomicAdd(a.cells + 1, N * (unsigned long long)st.refines);
-      atomicAdd(a.cells + 2, N * (unsigned long long)st.iters);
-      atomicAdd(a.cells + 3, N * (unsigned long long)st.n_xpe);
-    }
-  }
-}
-
-// Small solves, one CTA each, taken from the CTA queue until it is empty.
-template <typename T>
-__device__ void res_cta_loop(const ResArgs &a, ResShared<T> &sh, int &buf) {
-  for (;;) {
-    __syncthreads();  // every thread has read the previous task
-    if (threadIdx.x == 0) sh.task = atomicAdd(a.tq_head, 1);
-    __syncthreads();
-    const int t = sh.task;
-    if (t >= a.n_tq) break;
-    int s = a.tq[t];
-    if (!idx_ok(s, a.n_solves)) continue;
-    res_solve<T, false>(a, s, sh, buf);
-  }
-}
-
-template <typename T, int NT>
-struct ResMinBlocks {
-  static constexpr int value = (sizeof(T) == 4 && NT <= 256) ? 2 : 1;
-};
-
 }  // namespace
-
-// The cluster kernel: each cluster takes the large solves of the cluster
-// queue one after the other (rank 0 draws the next position and writes it
-// into every CTA's shared memory before a cluster barrier); once that queue
-// is empty its CTAs take small solves from the CTA queue independently (no
-// cluster barrier or distributed shared memory access follows).
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, ResMinBlocks<T, NT>::value) k_res_cluster(ResArgs a) {
-  __shared__ ResShared<T> sh;
-  int buf = 0;
-  const unsigned cr = cl_rank(), cs = cl_size();
-  for (;;) {
-    if (cr == 0 && threadIdx.x == 0) {
-      const int t = atomicAdd(a.cq_head, 1);
-      for (unsigned r = 0; r < cs; ++r) cl_st(cl_map(&sh.task, r), t);
-    }
-    cl_sync();
-    const int t = sh.task;
-    if (t >= a.n_cq) break;
-    const int s = a.cq[t];
-    if (idx_ok(s, a.n_solves)) res_solve<T, true>(a, s, sh, buf);
-  }
-  res_cta_loop<T>(a, sh, buf);
-}
-
-// The CTA kernel: small solves only (a plan without cluster solves).
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, ResMinBlocks<T, NT>::value) k_res_cta(ResArgs a) {
-  __shared__ ResShared<T> sh;
-  int buf = 0;
-  res_cta_loop<T>(a, sh, buf);
-}
 
 // ---------------------------------------------------------------------------
 // Resident solver with the CG state in shared memory (FP32 bulk)
@@ -2673,9 +2562,8 @@ __device__ bool grid_sync(const ResArgs &a, int *flag) {
 // up.  The slots alternate between two buffers: a buffer is written again
 // only two sums later, after a barrier that every reader has passed.
 constexpr int kGridMaxPerLane = 8;  // up to 256 CTAs in the launch
-template <int NA>
-__device__ bool grid_sum(Acc<float> (&a)[NA], ResShared<float> &sh, const ResArgs &ra, int &buf,
-                         Acc<float> (&out)[NA]) {
+template <typename T, int NA>
+__device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, int &buf, Acc<T> (&out)[NA]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < NA; ++k) warp_reduce_acc(a[k]);
@@ -2686,40 +2574,30 @@ __device__ bool grid_sum(Acc<float> (&a)[NA], ResShared<float> &sh, const ResArg
   __syncthreads();
   bool ok = true;
   if (warp == 0) {
-    Acc<float> m[NA];
+    Acc<T> m[NA];
 #pragma unroll
     for (int k = 0; k < NA; ++k) {
       if (lane < nw) m[k] = sh.red[lane][k];
       warp_reduce_acc(m[k]);
     }
     const unsigned G = gridDim.x;
-    float *slots = ra.gpart + (size_t)buf * (G + 1) * 6;  // [G] CTA slots of 3 (hi, lo) pairs
+    double *slots = ra.gpart + (size_t)buf * (G + 1) * 3;  // [G] CTA slots of 3 sums (FP32 bulk: (hi, lo) pairs)
     if (lane == 0) {
 #pragma unroll
-      for (int k = 0; k < NA; ++k) {
-        slots[blockIdx.x * 6 + 2 * k] = m[k].s;
-        slots[blockIdx.x * 6 + 2 * k + 1] = m[k].c;
-      }
+      for (int k = 0; k < NA; ++k) Slot<T>::store(slots + blockIdx.x * 3 + k, m[k]);
     }
     ok = grid_arrive_wait(ra);
     if (ok) {
 #pragma unroll
       for (int k = 0; k < NA; ++k) {
-        float vs[kGridMaxPerLane], vc[kGridMaxPerLane];
+        Acc<T> v[kGridMaxPerLane], t;
 #pragma unroll
         for (int i = 0; i < kGridMaxPerLane; ++i) {
           const unsigned r = (unsigned)lane + 32u * i;
-          vs[i] = r < G ? __ldcg(slots + r * 6 + 2 * k) : 0.f;
-          vc[i] = r < G ? __ldcg(slots + r * 6 + 2 * k + 1) : 0.f;
+          if (r < G) v[i] = Slot<T>::load(slots + r * 3 + k);
         }
-        Acc<float> t;
 #pragma unroll
-        for (int i = 0; i < kGridMaxPerLane; ++i) {
-          Acc<float> v;
-          v.s = vs[i];
-          v.c = vc[i];
-          t.merge(v);
-        }
+        for (int i = 0; i < kGridMaxPerLane; ++i) t.merge(v[i]);
         warp_reduce_acc(t);
         if (lane == 0) out[k] = t;
       }
@@ -2732,25 +2610,19 @@ __device__ bool grid_sum(Acc<float> (&a)[NA], ResShared<float> &sh, const ResArg
 // The group's sum and barrier for group kind kG (0 one CTA, 1 a cluster, 2
 // the whole GPU); only the whole-GPU forms can fail: the sum reports it to
 // thread 0 (which holds the totals), the barrier to every thread.
-template <int NA, int kG>
-__device__ __forceinline__ bool res2_sum(Acc<float> (&acc)[NA], ResShared<float> &sh, const ResArgs &a, int &buf,
-                                         Acc<float> (&tot)[NA]) {
-  if (kG == 2) return grid_sum<NA>(acc, sh, a, buf, tot);
-  group_sum<float, NA, kG == 1>(acc, sh, buf, tot);
+template <int NA, int kG, typename T>
+__device__ __forceinline__ bool res2_sum(Acc<T> (&acc)[NA], ResShared<T> &sh, const ResArgs &a, int &buf,
+                                         Acc<T> (&tot)[NA]) {
+  if (kG == 2) return grid_sum<T, NA>(acc, sh, a, buf, tot);
+  group_sum<T, NA, kG == 1>(acc, sh, buf, tot);
   return true;
 }
-template <int kG>
-__device__ __forceinline__ bool res2_barrier(const ResArgs &a, ResShared<float> &sh) {
+template <int kG, typename T>
+__device__ __forceinline__ bool res2_barrier(const ResArgs &a, ResShared<T> &sh) {
   if (kG == 2) return grid_sync(a, &sh.task);
   group_barrier<kG == 1>();
   return true;
 }
-// A whole-GPU barrier gave up (thread 0): the solve ends with ATS_ERR_TIMEOUT.
-__device__ __forceinline__ void res2_timeout(ResState &st) {
-  st.status = ATS_ERR_TIMEOUT;
-  st.phase = kDone;
-}
-
 // The result of a solve on this CTA's octs [lo, hi), as k_final writes it:
 // x (Crank-Nicolson: 2 x' - E^n) to xd, which may be device memory or host
 // memory the device can write (then the result reaches the host while other
@@ -2877,37 +2749,9 @@ __device__ bool res2_solve_l(const ResArgs &a, int s, ResShared<float> &sh, int 
       Acc<float> acc[3], tot[3];
       for (int o = o0; o < hi; o += stride) res2_ref_oct(cx, sd, o, want_x, acc[0], acc[1], acc[2]);
       const bool ok = res2_sum<3, kG>(acc, sh, a, buf, tot);
-      if (threadIdx.x == 0 && !ok) res2_timeout(sh.st);
-      if (threadIdx.x == 0 && ok) {
-        ResState &st = sh.st;
-        const double rnorm = sqrt(tot[0].get()), xnorm = sqrt(tot[1].get()), rz = tot[2].get();
-        if (st.refines == 0) st.r0 = rnorm;
-        st.refines += 1;
-        st.rnorm = rnorm;
-        st.xnorm = xnorm;
-        const double target = sd.tol * (sd.stop_rule == ATS_STOP_CERTIFIED ? xnorm : st.r0);
-        if (st.final_pass) {
-          st.phase = kDone;
-        } else if (!isfinite(rnorm)) {
-          st.status = ATS_ERR_BREAKDOWN;
-          st.phase = kDone;
-        } else if (rnorm <= target) {
-          st.phase = kDone;
-        } else if (st.refines > sd.max_refine) {
-          st.status = ATS_ERR_NOT_CONVERGED;
-          st.phase = kDone;
-        } else if (!(rz > 0.0)) {
-          st.status = ATS_ERR_BREAKDOWN;
-          st.phase = kDone;
-        } else {
-          st.phase = kInner;
-          st.rz = rz;
-          st.rzf = (float)rz;
-          st.first = 1;
-          st.inner_iters = 0;
-          st.inner_target = fmax(sd.inner_rtol * rnorm, sd.final_safety * target);
-          st.t2f = (float)(st.inner_target * st.inner_target);
-        }
+      if (threadIdx.x == 0) {
+        if (ok) refine_decision(sh.st, sd, tot[0].get(), tot[1].get(), tot[2].get());
+        else res2_timeout(sh.st);
       }
       __syncthreads();
       continue;
@@ -2954,23 +2798,7 @@ __device__ bool res2_solve_l(const ResArgs &a, int s, ResShared<float> &sh, int 
       }
       const bool ok = res2_sum<2, kG>(acc, sh, a, buf, tot);
       if (threadIdx.x == 0 && !ok) res2_timeout(sh.st);
-      if (threadIdx.x == 0 && ok) {
-        ResState &st = sh.st;
-        st.iters += 1;
-        st.inner_iters += 1;
-        st.first = 0;
-        const bool conv = cg_beta(st, tot[0], tot[1], f32);
-        if (conv) {
-          st.phase = kRefine;
-        } else if (st.iters >= sd.max_iter) {
-          st.status = ATS_ERR_NOT_CONVERGED;
-          st.final_pass = 1;
-          st.phase = kRefine;
-        } else if (st.inner_iters >= sd.inner_max) {
-          st.phase = kRefine;
-        }
-        if (st.phase == kRefine) st.n_xpe += 1;
-      }
+      if (threadIdx.x == 0 && ok) step_decision(sh.st, sd, cg_beta(sh.st, tot[0], tot[1], f32));
       __syncthreads();
     }
     if (sh.st.phase == kDone) break;
@@ -2987,33 +2815,7 @@ __device__ bool res2_solve_l(const ResArgs &a, int s, ResShared<float> &sh, int 
   // the result of the own octs (each CTA updated only its own octs' x)
   double *xd = a.x_out ? a.x_out[s] : nullptr;
   if (xd) res2_copy_out(sd, xd, cx.lo, hi, a.neg ? a.neg + s : nullptr);
-  if (threadIdx.x == 0 && cr == 0) {
-    const ResState &st = sh.st;
-    SolveScalars f;
-    memset(&f, 0, sizeof(f));
-    f.phase = kDone;
-    f.iters = st.iters;
-    f.inner_iters = st.inner_iters;
-    f.refines = st.refines;
-    f.status = st.status;
-    f.final_pass = st.final_pass;
-    f.ticks = st.n_op + st.iters + st.refines;
-    f.rz = st.rz;
-    f.r0 = st.r0;
-    f.inner_target = st.inner_target;
-    f.rnorm = st.rnorm;
-    f.xnorm = st.xnorm;
-    a.final_sc[s] = f;
-    if (a.t_solve) a.t_solve[2 * s + 1] = globaltimer_ns();
-    if (a.cells) {
-      const unsigned long long N = 8ull * (unsigned long long)n;
-      atomicAdd(a.cells + 0, N * (unsigned long long)(st.n_op - st.n_first));
-      atomicAdd(a.cells + 4, N * (unsigned long long)st.n_first);
-      atomicAdd(a.cells + 1, N * (unsigned long long)st.refines);
-      atomicAdd(a.cells + 2, N * (unsigned long long)st.iters);
-      atomicAdd(a.cells + 3, N * (unsigned long long)st.n_xpe);
-    }
-  }
+  if (threadIdx.x == 0 && cr == 0) res_finish(a, s, sh.st, n);
   return alive;
 }
 
@@ -3087,22 +2889,371 @@ __global__ void __launch_bounds__(NT, 1) k_res2_grid(ResArgs a) {
     if (!idx_ok(s, a.n_solves)) continue;
     if (alive) {
       alive = res2_solve<2, false>(a, s, sh, buf);
-    } else if (blockIdx.x == 0 && threadIdx.x == 0) {
-      SolveScalars f;
-      memset(&f, 0, sizeof(f));
-      f.phase = kDone;
-      f.status = ATS_ERR_TIMEOUT;
-      a.final_sc[s] = f;
+    } else {
+      res_never_ran(a, s);
     }
     __syncthreads();  // every thread has left the solve before the next stage-in
   }
 }
 
-template <typename T, int NT>
-static cudaError_t res_launch_t(int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only) {
+// ---------------------------------------------------------------------------
+// Resident solver, FP64 bulk
+// ---------------------------------------------------------------------------
+//
+// Bound: the FP64 pipe (1.0 TFLOP/s measured, 18 cycles per warp instruction
+// and SM, 1/67 of FP32), so a step is written for few FP64 instructions: 112
+// per oct and CG iteration against about 290 when the face coefficients are
+// formed from K and z = r / D divides.  The stencil takes the stored
+// coefficients C64; r is kept, so that D z needs no product (D z = r), and
+// 1 / D is stored, so that z = r x (1 / D); q follows the recurrence
+// q = (I + dt A) z + beta q_prev, which needs no barrier after p:
+//   1. w = r - sum C z_j, p = z + beta p, q = w + beta q, the sum p.q;
+//   2. r -= alpha q, e += alpha p, z = r x (1 / D), the sums r.z and r.r.
+// The vectors come from L1 / L2 (14 rows of 64 bytes per oct and iteration
+// against 112 x 18 / 32 = 63 cycles of the pipe), so shared memory would not
+// pay.  What counts is the octs per SM: the groups are chosen for small runs
+// (kRun64 where a plan picks them), and levels above the clusters take the
+// whole-GPU form.  z is the only array other threads read (ld.global.cg after
+// the step's barrier); p, q, r, e and 1 / D belong to the thread that owns the
+// oct.  Non-leaf cells: C = 0 on all their faces, and r = z = p = q = 0.
+// Measured, certified 5e-11, build included: 128 levels of 64..2 048 octs
+// 28.6 -> 3.1 ms (one CTA of 256 threads each before), 4 096 octs 4.51 -> 1.23
+// ms and 32 736 octs 6.49 -> 2.01 ms (tick path before).
+
+namespace {
+
+template <int A>
+__device__ __forceinline__ void resd_axis(const SolveDev &sd, int o, const int (&nb)[6], const double *z,
+                                          const double (&v)[8], double (&w)[8]) {
+  constexpr int bit = 1 << A;
+  double Cu[8];
+  ld8_ro(sd.C64 + (3 * (size_t)o + A) * 8, Cu);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    if (c & bit) continue;
+    const int d = c | bit;
+    w[c] = fma(-Cu[c], v[d], w[c]);
+    w[d] = fma(-Cu[c], v[c], w[d]);
+  }
+  int n = nb[2 * A + 1];  // +A face: C from row A of this oct
+  if (n >= 0) {
+    double Zn[8];
+    ldc_face<A, 0>(z + 8 * (size_t)n, Zn);
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (c & bit) w[c] = fma(-Cu[c], Zn[c ^ bit], w[c]);
+  }
+  n = nb[2 * A];  // -A face: C from row A of the -A neighbour
+  if (n >= 0) {
+    double Zn[8], Cn[8];
+    ldc_face<A, 1>(z + 8 * (size_t)n, Zn);
+    ld_face<A, 1>(sd.C64 + (3 * (size_t)n + A) * 8, Cn);
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (!(c & bit)) w[c] = fma(-Cn[c | bit], Zn[c | bit], w[c]);
+  }
+}
+
+// Step 1 on oct o; returns the oct's p.q in the accumulator.
+__device__ __forceinline__ void resd_op_oct(const SolveDev &sd, int o, bool first, double beta, Acc<double> &pq) {
+  int nb[6];
+  load_nbr6(sd.nbr, o, nb);
+  check_nbr6(nb, sd.n_oct);
+  const double *z = (const double *)sd.z;
+  double *p = (double *)sd.p0, *q = (double *)sd.q;
+  double v[8], w[8];
+  ldc8(z + 8 * (size_t)o, v);
+  ld8_rw((const double *)sd.p1 + 8 * (size_t)o, w);  // r
+  resd_axis<0>(sd, o, nb, z, v, w);
+  resd_axis<1>(sd, o, nb, z, v, w);
+  resd_axis<2>(sd, o, nb, z, v, w);
+  if (!first) {
+    double t[8];
+    ld8_rw(p + 8 * (size_t)o, t);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = fma(beta, t[c], v[c]);
+    ld8_rw(q + 8 * (size_t)o, t);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) w[c] = fma(beta, t[c], w[c]);
+  }
+  st8(p + 8 * (size_t)o, v);
+  st8(q + 8 * (size_t)o, w);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) pq.add(v[c], w[c]);
+}
+
+// Step 2 on oct o.
+__device__ __forceinline__ void resd_upd_oct(const SolveDev &sd, int o, double alpha, Acc<double> &rz,
+                                             Acc<double> &rr) {
+  double a[8], b[8];
+  double *r = (double *)sd.p1 + 8 * (size_t)o, *e = (double *)sd.e + 8 * (size_t)o;
+  ld8_rw(r, a);
+  ld8_rw((const double *)sd.q + 8 * (size_t)o, b);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) a[c] = fma(-alpha, b[c], a[c]);
+  st8(r, a);
+  ld8_rw((const double *)sd.dg + 8 * (size_t)o, b);  // 1 / D
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    b[c] *= a[c];
+    rr.add(a[c], a[c]);
+    rz.add(a[c], b[c]);
+  }
+  st8((double *)sd.z + 8 * (size_t)o, b);
+  ld8_rw((const double *)sd.p0 + 8 * (size_t)o, b);
+  ld8_rw(e, a);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) a[c] = fma(alpha, b[c], a[c]);
+  st8(e, a);
+}
+
+// The residual r = b - (1 + xd) x - sum C (x_i - x_j) (the form of ref_axis),
+// D = 1 + xd + sum C, z = r x (1 / D) on oct o.
+template <int A>
+__device__ __forceinline__ void resd_ref_axis(const SolveDev &sd, int o, const int (&nb)[6], const double (&xv)[8],
+                                              double (&acc)[8], double (&ds)[8]) {
+  constexpr int bit = 1 << A;
+  double Cu[8];
+  ld8_ro(sd.C64 + (3 * (size_t)o + A) * 8, Cu);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    if (c & bit) continue;
+    const int d = c | bit;
+    const double df = xv[c] - xv[d];
+    acc[c] = fma(Cu[c], df, acc[c]);
+    acc[d] = fma(-Cu[c], df, acc[d]);
+    ds[c] += Cu[c];
+    ds[d] += Cu[c];
+  }
+  int n = nb[2 * A + 1];
+  if (n >= 0) {
+    double Xn[8];
+    ldc_face<A, 0>(sd.x64 + 8 * (size_t)n, Xn);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      if (!(c & bit)) continue;
+      acc[c] = fma(Cu[c], xv[c] - Xn[c ^ bit], acc[c]);
+      ds[c] += Cu[c];
+    }
+  }
+  n = nb[2 * A];
+  if (n >= 0) {
+    double Xn[8], Cn[8];
+    ldc_face<A, 1>(sd.x64 + 8 * (size_t)n, Xn);
+    ld_face<A, 1>(sd.C64 + (3 * (size_t)n + A) * 8, Cn);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      if (c & bit) continue;
+      acc[c] = fma(Cn[c | bit], xv[c] - Xn[c | bit], acc[c]);
+      ds[c] += Cn[c | bit];
+    }
+  }
+}
+
+__device__ __forceinline__ void resd_ref_oct(const SolveDev &sd, int o, bool want_x, Acc<double> &rr, Acc<double> &xx,
+                                             Acc<double> &rz) {
+  int nb[6];
+  load_nbr6(sd.nbr, o, nb);
+  check_nbr6(nb, sd.n_oct);
+  int rec = __ldg(sd.xrec + o);
+  if (rec >= 0 && !idx_ok(rec, sd.n_xd)) rec = -1;
+  double xv[8], acc[8], ds[8];
+  ldc8(sd.x64 + 8 * (size_t)o, xv);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc[c] = ds[c] = 0.0;
+  resd_ref_axis<0>(sd, o, nb, xv, acc, ds);
+  resd_ref_axis<1>(sd, o, nb, xv, acc, ds);
+  resd_ref_axis<2>(sd, o, nb, xv, acc, ds);
+  double t[8];
+  if (rec >= 0) {
+    ld8_ro(sd.xd64 + 8 * (size_t)rec, t);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) t[c] = 0.0;
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const double m = 1.0 + t[c];
+    acc[c] = fma(m, xv[c], acc[c]);
+    ds[c] += m;
+  }
+  ld8_ro(sd.b64 + 8 * (size_t)o, t);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc[c] = t[c] - acc[c];
+  ld8_ro(sd.K64 + 8 * (size_t)o, t);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const bool leaf = t[c] >= 0.0;
+    const double r = leaf ? acc[c] : 0.0;
+    const double inv = leaf ? 1.0 / ds[c] : 1.0;
+    const double z = r * inv;
+    if (leaf) {
+      rr.add(r, r);
+      rz.add(r, z);
+      if (want_x) xx.add(xv[c], xv[c]);
+    }
+    acc[c] = r;
+    ds[c] = inv;
+    t[c] = z;
+  }
+  st8((double *)sd.p1 + 8 * (size_t)o, acc);
+  st8((double *)sd.dg + 8 * (size_t)o, ds);
+  st8((double *)sd.z + 8 * (size_t)o, t);
+}
+
+// One FP64 solve by one group (kG: 0 one CTA, 1 a cluster, 2 every CTA of a
+// cooperative launch), the state machine of res2_solve_l.  Returns false when
+// a whole-GPU barrier wait gave up (the solve then ends with ATS_ERR_TIMEOUT).
+template <int kG>
+__device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &buf) {
+  constexpr int wd = (int)(sizeof(SolveDev) / 8);
+  for (int w = threadIdx.x; w < wd; w += blockDim.x)
+    reinterpret_cast<unsigned long long *>(&sh.sd)[w] = reinterpret_cast<const unsigned long long *>(a.solves + s)[w];
+  const unsigned cs = kG == 2 ? gridDim.x : (kG == 1 ? cl_size() : 1u);
+  const unsigned cr = kG == 2 ? blockIdx.x : (kG == 1 ? cl_rank() : 0u);
+  if (threadIdx.x == 0) {
+    ResState z;
+    memset(&z, 0, sizeof(z));
+    z.phase = kRefine;
+    z.status = ATS_OK;
+    sh.st = z;
+    if (a.t_solve && cr == 0) a.t_solve[2 * s] = globaltimer_ns();
+  }
+  __syncthreads();
+  const SolveDev &sd = sh.sd;
+  const int n = sd.n_oct;
+  const int chunk = (int)((n + (int)cs - 1) / (int)cs);
+  const int lo = min(n, (int)cr * chunk), hi = min(n, lo + chunk);
+  const int o0 = lo + (int)threadIdx.x, stride = (int)blockDim.x;
+  const bool want_x = sd.stop_rule == ATS_STOP_CERTIFIED;
+  for (;;) {
+    const int phase = sh.st.phase;
+    if (phase == kDone) break;
+    if (phase == kRefine) {
+      Acc<double> acc[3], tot[3];
+      for (int o = o0; o < hi; o += stride) resd_ref_oct(sd, o, want_x, acc[0], acc[1], acc[2]);
+      const bool ok = res2_sum<3, kG>(acc, sh, a, buf, tot);
+      if (threadIdx.x == 0) {
+        if (ok) refine_decision(sh.st, sd, tot[0].get(), tot[1].get(), tot[2].get());
+        else res2_timeout(sh.st);
+      }
+      __syncthreads();
+      continue;
+    }
+    {
+      const bool first = sh.st.first != 0;
+      const double beta = sh.st.beta;
+      Acc<double> acc[1], tot[1];
+      for (int o = o0; o < hi; o += stride) resd_op_oct(sd, o, first, beta, acc[0]);
+      const bool ok = res2_sum<1, kG>(acc, sh, a, buf, tot);
+      if (threadIdx.x == 0) {
+        ResState &st = sh.st;
+        if (ok) {
+          st.n_op += 1;
+          st.n_first += st.first ? 1 : 0;
+          cg_alpha(st, tot[0], false);
+        } else {
+          res2_timeout(st);
+        }
+      }
+      __syncthreads();
+    }
+    if (sh.st.phase == kDone) break;
+    {
+      const double alpha = sh.st.alpha;
+      Acc<double> acc[2], tot[2];
+      for (int o = o0; o < hi; o += stride) resd_upd_oct(sd, o, alpha, acc[0], acc[1]);
+      const bool ok = res2_sum<2, kG>(acc, sh, a, buf, tot);
+      if (threadIdx.x == 0) {
+        if (ok) step_decision(sh.st, sd, cg_beta(sh.st, tot[0], tot[1], false));
+        else res2_timeout(sh.st);
+      }
+      __syncthreads();
+    }
+    if (sh.st.phase == kDone) break;
+    if (sh.st.phase == kRefine) {
+      // x += e, e = 0; the residual pass reads the neighbours' x
+      for (int o = o0; o < hi; o += stride) res_xpe_oct<double>(sd, o);
+      if (!res2_barrier<kG>(a, sh)) {
+        if (threadIdx.x == 0) res2_timeout(sh.st);
+        break;
+      }
+    }
+  }
+  __syncthreads();  // thread 0's last state update is seen by all
+  const bool alive = sh.st.status != ATS_ERR_TIMEOUT;
+  if (threadIdx.x == 0 && cr == 0) res_finish(a, s, sh.st, n);
+  return alive;
+}
+
+__device__ void resd_cta_loop(const ResArgs &a, ResShared<double> &sh, int &buf) {
+  for (;;) {
+    __syncthreads();  // every thread has read the previous task
+    if (threadIdx.x == 0) sh.task = atomicAdd(a.tq_head, 1);
+    __syncthreads();
+    const int t = sh.task;
+    if (t >= a.n_tq) break;
+    int s = a.tq[t];
+    if (!idx_ok(s, a.n_solves)) continue;
+    resd_solve<0>(a, s, sh, buf);
+  }
+}
+
+}  // namespace
+
+// The cluster kernel: each cluster takes the solves of the cluster queue one
+// after the other (rank 0 draws the next position and writes it into every
+// CTA's shared memory before a cluster barrier); once that queue is empty its
+// CTAs take small solves from the CTA queue independently (no cluster barrier
+// or distributed shared memory access follows).
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) k_resd_cluster(ResArgs a) {
+  __shared__ ResShared<double> sh;
+  int buf = 0;
+  const unsigned cr = cl_rank(), cs = cl_size();
+  for (;;) {
+    if (cr == 0 && threadIdx.x == 0) {
+      const int t = atomicAdd(a.cq_head, 1);
+      for (unsigned r = 0; r < cs; ++r) cl_st(cl_map(&sh.task, r), t);
+    }
+    cl_sync();
+    const int t = sh.task;
+    if (t >= a.n_cq) break;
+    const int s = a.cq[t];
+    if (idx_ok(s, a.n_solves)) resd_solve<1>(a, s, sh, buf);
+    cl_sync();  // no CTA starts the next solve while another is still in this one
+  }
+  resd_cta_loop(a, sh, buf);
+}
+
+// The CTA kernel: small solves only (a plan without cluster solves).
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) k_resd_cta(ResArgs a) {
+  __shared__ ResShared<double> sh;
+  int buf = 0;
+  resd_cta_loop(a, sh, buf);
+}
+
+// The whole-GPU form (see k_res2_grid).
+template <int NT>
+__global__ void __launch_bounds__(NT, 1) k_resd_grid(ResArgs a) {
+  __shared__ ResShared<double> sh;
+  int buf = 0;
+  bool alive = true;
+  for (int t = 0; t < a.n_gq; ++t) {
+    const int s = a.gq[t];
+    if (!idx_ok(s, a.n_solves)) continue;
+    if (alive) alive = resd_solve<2>(a, s, sh, buf);
+    else res_never_ran(a, s);
+    __syncthreads();  // every thread has left the solve before the next one starts
+  }
+}
+
+template <int NT>
+static cudaError_t resd_launch_t(int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only) {
   if (a.n_cq > 0 && !cta_only) {
     if (cluster > 8) {
-      cudaError_t e = cudaFuncSetAttribute(k_res_cluster<T, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      cudaError_t e = cudaFuncSetAttribute(k_resd_cluster<NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
@@ -3117,16 +3268,16 @@ static cudaError_t res_launch_t(int cluster, int grid, const ResArgs &a, cudaStr
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_res_cluster<T, NT>, a);
+    return cudaLaunchKernelEx(&cfg, k_resd_cluster<NT>, a);
   }
-  k_res_cta<T, NT><<<grid, NT, 0, st>>>(a);
+  k_resd_cta<NT><<<grid, NT, 0, st>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T, int NT>
-static int res_clusters_t(int cluster) {
+template <int NT>
+static int resd_clusters_t(int cluster) {
   if (cluster > 8 &&
-      cudaFuncSetAttribute(k_res_cluster<T, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaFuncSetAttribute(k_resd_cluster<NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -3141,17 +3292,17 @@ static int res_clusters_t(int cluster) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_res_cluster<T, NT>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, k_resd_cluster<NT>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   return n;
 }
 
-template <typename T, int NT>
-static int res_cta_blocks_t() {
+template <int NT>
+static int resd_cta_blocks_t() {
   int b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_res_cta<T, NT>, NT, 0) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_resd_cta<NT>, NT, 0) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -3265,10 +3416,19 @@ int resident_smem_cap(int threads, int device) {
   return threads >= 512 ? res2_cap_t<512>(device) : res2_cap_t<256>(device);
 }
 
+// The whole-GPU form of a bulk precision: its kernel and dynamic shared memory.
+using ResGridKernel = void (*)(ResArgs);
 template <int NT>
-static cudaError_t res2_grid_launch_t(int grid, const ResArgs &a, cudaStream_t st) {
-  const size_t smem = kRes2SmemBytes;
-  cudaError_t e = cudaFuncSetAttribute(k_res2_grid<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+static ResGridKernel res_grid_kernel(bool fp64, size_t *smem) {
+  *smem = fp64 ? 0 : kRes2SmemBytes;
+  return fp64 ? k_resd_grid<NT> : k_res2_grid<NT>;
+}
+
+template <int NT>
+static cudaError_t res2_grid_launch_t(bool fp64, int grid, const ResArgs &a, cudaStream_t st) {
+  size_t smem = 0;
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, &smem);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -3280,15 +3440,16 @@ static cudaError_t res2_grid_launch_t(int grid, const ResArgs &a, cudaStream_t s
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_res2_grid<NT>, a);
+  return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 template <int NT>
-static int res2_grid_ctas_t(int device) {
+static int res2_grid_ctas_t(bool fp64, int device) {
   int b = 0, sms = 0;
-  if (cudaFuncSetAttribute(k_res2_grid<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRes2SmemBytes) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_res2_grid<NT>, NT, kRes2SmemBytes) != cudaSuccess ||
+  size_t smem = 0;
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, &smem);
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, NT, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -3309,19 +3470,23 @@ cudaError_t launch_hold(unsigned long long ns, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_resident_grid(int threads, int grid, const ResArgs &a, cudaStream_t st) {
+cudaError_t launch_resident_grid(bool fp64, int grid, const ResArgs &a, cudaStream_t st) {
   if (a.n_gq <= 0) return cudaSuccess;
-  if (threads != 512 || grid <= 0 || grid > 32 * kGridMaxPerLane || a.cap != kRes2Cap3 || !a.gbar || !a.gpart ||
-      !a.gerr)
+  if (grid <= 0 || grid > 32 * kGridMaxPerLane || (!fp64 && a.cap != kRes2Cap3) || !a.gbar || !a.gpart || !a.gerr)
     return cudaErrorInvalidValue;
-  return res2_grid_launch_t<512>(grid, a, st);
+  return res2_grid_launch_t<512>(fp64, grid, a, st);
 }
 
 int resident_six_cap() { return kRes2Cap6; }
 
-int resident_grid_ctas(int threads, int device) {
-  if (threads != 512) return 0;  // compiled for 512-thread CTAs only
-  return std::min(32 * kGridMaxPerLane, res2_grid_ctas_t<512>(device));
+int resident_grid_ctas(bool fp64, int device) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  // one CTA per SM: a grid barrier costs with the CTAs that arrive
+  return std::min({32 * kGridMaxPerLane, sms, res2_grid_ctas_t<512>(fp64, device)});
 }
 
 // One grid barrier of the whole-GPU form on its own, every CTA recording
@@ -3346,24 +3511,20 @@ cudaError_t launch_grid_barrier_probe(int grid, const ResArgs &a, int *out, cuda
   return cudaLaunchKernelEx(&cfg, k_grid_barrier_probe, a, out);
 }
 
-cudaError_t launch_resident(bool fp64, int threads, int cluster, int grid, const ResArgs &a, cudaStream_t st,
-                            bool cta_only) {
+cudaError_t launch_resident(int threads, int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only) {
   if (a.n_cq + a.n_tq <= 0) return cudaSuccess;
   if (cluster < 1 || cluster > kMaxCluster || grid <= 0) return cudaErrorInvalidValue;
-  if (!fp64) return cudaErrorInvalidValue;  // FP32 bulk: launch_resident_smem
-  return threads >= 512 ? res_launch_t<double, 512>(cluster, grid, a, st, cta_only)
-                        : res_launch_t<double, 256>(cluster, grid, a, st, cta_only);
+  return threads >= 512 ? resd_launch_t<512>(cluster, grid, a, st, cta_only)
+                        : resd_launch_t<256>(cluster, grid, a, st, cta_only);
 }
 
-int resident_max_clusters(bool fp64, int threads, int cluster) {
+int resident_max_clusters(int threads, int cluster) {
   if (cluster < 1 || cluster > kMaxCluster) return 0;
-  if (!fp64) return 0;
-  return threads >= 512 ? res_clusters_t<double, 512>(cluster) : res_clusters_t<double, 256>(cluster);
+  return threads >= 512 ? resd_clusters_t<512>(cluster) : resd_clusters_t<256>(cluster);
 }
 
-int resident_cta_blocks(bool fp64, int threads) {
-  if (!fp64) return 0;
-  return threads >= 512 ? res_cta_blocks_t<double, 512>() : res_cta_blocks_t<double, 256>();
+int resident_cta_blocks(int threads) {
+  return threads >= 512 ? resd_cta_blocks_t<512>() : resd_cta_blocks_t<256>();
 }
 
 }  // namespace ats

@@ -269,7 +269,7 @@ struct Plan {
   bool queue_dirty = false;
   std::vector<int32_t> h_queue;  // the queue order last uploaded
   unsigned *d_gbar = nullptr;
-  float *d_gpart = nullptr;
+  double *d_gpart = nullptr;
   int *d_gerr = nullptr;
   int res_threads = 512, res_cluster = 8, res_cluster_big = 16, res_grid = 0, res_grid_big = 0;
   int res_cluster_mid = 8, res_grid_mid = 0;
@@ -576,6 +576,13 @@ void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
   P->res_split_measured = true;
 }
 
+// FP64 resident groups: octs per CTA up to which the next smaller group is
+// taken.  An FP64 step is bound by the SM's FP64 pipe (2 100 cycles per warp
+// of octs and CG iteration, four warps side by side), a cluster's two sums
+// cost about 3 000: runs of 128 octs keep the pipe busy most of a step and
+// spread a level over as many SMs as that allows.
+constexpr int64_t kRun64 = 128;
+
 ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const ats_solve_opts *opts_in,
                        Plan **out) {
   *out = nullptr;
@@ -691,7 +698,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     P->res_cluster_mid = 0;
   {
     const bool res_ok = o.sched != ATS_SCHED_TICK && o.stop_rule != ATS_STOP_PAPER;
-    const int64_t cta_octs = o.res_cta_octs == 0 ? 2048 : o.res_cta_octs;
+    const int64_t cta_octs = o.res_cta_octs == 0 ? (P->fp64 ? kRun64 : 2048) : o.res_cta_octs;
     // default limit: mixed precision 16384 octs (the shared-memory form
     // beats a whole-GPU tick loop up to about there for one solve alone);
     // FP64 (the global-memory form) 2048
@@ -710,14 +717,17 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     auto max_clusters = [&](int cl) {
       if (cl <= 0) return 0;
       return P->res_smem ? resident_smem_clusters(P->res_threads, cl, P->res_cap)
-                         : resident_max_clusters(P->fp64, P->res_threads, cl);
+                         : resident_max_clusters(P->res_threads, cl);
     };
-    // levels above the limit: the whole-GPU form (FP32 bulk, each CTA's run
-    // in shared memory) when asked for, and with ATS_SCHED_AUTO when the runs
-    // on its CTAs keep all six arrays in shared memory; else the tick path
-    const bool grid_ok = (o.sched == ATS_SCHED_GRID || o.sched == ATS_SCHED_AUTO) && P->res_smem && P->res_cap > 0;
-    const int grid_all = grid_ok ? resident_grid_ctas(P->res_threads, ctx->device) : 0;
-    const int64_t grid_auto_octs = (int64_t)grid_all * std::min(P->res_cap, resident_six_cap());
+    // levels above the limit: the whole-GPU form when asked for, and with
+    // ATS_SCHED_AUTO in FP64 for every level, in FP32 bulk (each CTA's run in
+    // shared memory) when the runs on its CTAs keep all six arrays in shared
+    // memory; else the tick path
+    const bool grid_ok = (o.sched == ATS_SCHED_GRID || o.sched == ATS_SCHED_AUTO) &&
+                         (P->fp64 || (P->res_cap > 0 && P->res_threads == 512));
+    const int grid_all = grid_ok ? resident_grid_ctas(P->fp64, ctx->device) : 0;
+    const int64_t grid_auto_octs =
+        P->fp64 ? INT64_MAX : (int64_t)grid_all * std::min(P->res_cap, resident_six_cap());
     P->mode.assign(n, 0);
     for (int k = 0; k < n; ++k) {
       const int64_t no = P->levels[k]->n_oct;
@@ -729,7 +739,8 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       // a level whose runs on res_cluster CTAs would not fit their shared
       // memory takes the smallest larger cluster whose runs fit (the middle
       // size, else the big one); the work rule sends it to the big clusters
-      const auto fits = [&](int cl) { return P->res_cap <= 0 || no <= (int64_t)cl * P->res_cap; };
+      const int64_t run = P->fp64 ? kRun64 : P->res_cap;
+      const auto fits = [&](int cl) { return run <= 0 || no <= cl * run; };
       if (no <= cta_octs) P->mode[k] = 2;
       else if (P->res_cluster_big > 0 && est_work(P->levels[k]) > big_work) P->mode[k] = 3;
       else if (fits(P->res_cluster)) P->mode[k] = 1;
@@ -767,7 +778,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     }
     // the first split follows the estimated work; after each completed run,
     // the measured SM-time of each class (plan_adapt_split)
-    const int cta_per_sm = P->res_smem ? 1 : std::max(1, resident_cta_blocks(P->fp64, P->res_threads));
+    const int cta_per_sm = P->res_smem ? 1 : std::max(1, resident_cta_blocks(P->res_threads));
     P->res_slots = cta_per_sm * ctx->num_sms;
     P->res_clA = clA;
     P->res_clM = clM;
@@ -789,7 +800,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       (P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq > 0 &&
        (s = dev_alloc_t(ctx, 2 * (size_t)n, &P->d_tsolve)) != ATS_OK) ||
       (P->n_gq > 0 && (s = dev_alloc_t(ctx, 2, &P->d_gbar)) != ATS_OK) ||
-      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 12 * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 6 * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
       (P->n_gq > 0 && (s = dev_alloc_t(ctx, 1, &P->d_gerr)) != ATS_OK) ||
       (s = dev_alloc_t(ctx, 4, &P->d_heads)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 4 * (size_t)P->n_items, &P->d_lists)) != ATS_OK ||
@@ -906,7 +917,7 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
                                                                                  : 2;
     const int prio = cta_only ? 0 : std::min(prio_least, prio_greatest + rank);
     return P->res_smem ? launch_resident_smem(P->res_threads, cluster, grid, a, s2, cta_only, prio)
-                       : launch_resident(P->fp64, P->res_threads, cluster, grid, a, s2, cta_only);
+                       : launch_resident(P->res_threads, cluster, grid, a, s2, cta_only);
   };
   // the launches in order: big clusters, clusters, single CTAs (the first
   // one on st, the others on the side streams, forked before the first)
@@ -975,7 +986,7 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
     a.gerr = P->d_gerr;
     CUDA_TRY(cudaMemsetAsync(P->d_gbar, 0, 2 * sizeof(unsigned), st));
     CUDA_TRY(cudaMemsetAsync(P->d_gerr, 0, sizeof(int), st));
-    CUDA_TRY(launch_resident_grid(P->res_threads, P->res_grid_all, a, st));
+    CUDA_TRY(launch_resident_grid(P->fp64, P->res_grid_all, a, st));
   }
   if (prof) CUDA_TRY(cudaEventRecord(P->res_ev[1], st));
   // the resident kernels, the hold kernels before the later ones, the whole-GPU launch
