@@ -204,6 +204,8 @@ struct ResArgs {
   int n_cq, n_tq, n_solves;
   int cg_scalars;  // FP32 bulk: 0 = step decisions in FP32 from the rounded totals, 1 = in FP64
   int q_recur;     // FP32 bulk: 1 = q = (I + dt A) z + beta q_prev (no barrier), 0 = q = (I + dt A) p
+  int regs;        // FP32 bulk, 512 threads: 1 = the CG state in registers and shared memory
+                   // (q_recur = 1, cg_scalars = 0, every run at most resident_run_cap() octs)
   int *cq_head;
   int *tq_head;
   unsigned long long *cells;
@@ -263,6 +265,8 @@ int resident_grid_ctas(bool fp64, int device);
 // Octs per CTA up to which the shared-memory solver keeps all six CG arrays
 // (K, z, p, D, q, e) of a CTA's run in shared memory.
 int resident_six_cap();
+// Octs per CTA the form with the CG state in registers and shared memory takes.
+int resident_run_cap();
 // One grid barrier of that form alone (cooperative launch of `grid` CTAs of 32
 // threads) waiting for a.g_expect arrivals: out[cta] = 1 when its wait ended
 // normally, 0 when it gave up (and *a.gerr = 1).  a.gbar, a.gerr zeroed first.

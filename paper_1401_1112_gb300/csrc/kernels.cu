@@ -147,7 +147,7 @@ struct Acc<float> {
     const float zz = __fsub_rn(t, s);
     const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, zz)), __fsub_rn(o.s, zz));
     s = t;
-    c = __fadd_rn(c, __fadd_rn(o.c, e));
+    c = __fadd_rn(__fadd_rn(c, o.c), e);  // symmetric in the two operands, to the last bit
   }
   __device__ __forceinline__ double get() const { return (double)s + (double)c; }
   // the sum rounded to FP32 (no FP64 instruction)
@@ -1734,6 +1734,15 @@ __device__ __forceinline__ unsigned cl_size() {
 __device__ __forceinline__ void cl_sync() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
+// ... in two halves, with work of the thread's own between them.  The release
+// is warp 0's alone, for callers that have just passed a CTA barrier: it is
+// cumulative, so it covers what the other warps wrote before that barrier,
+// and their own arrivals need not wait for their outstanding stores.
+__device__ __forceinline__ void cl_arrive(bool release) {
+  if (release) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  else asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // shared::cluster address of a variable of this CTA's shared memory in the
 // CTA of cluster rank `rank`
 __device__ __forceinline__ uint32_t cl_map(const void *p, unsigned rank) {
@@ -1752,12 +1761,24 @@ __device__ __forceinline__ void cl_st(uint32_t a, const Acc<double> &v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v.s) : "memory");
 }
 
-// lane 0's accumulator in every lane of the warp
-__device__ __forceinline__ void bcast_acc(const Acc<float> &a, Acc<float> &t) {
-  t.s = __shfl_sync(kFull, a.s, 0);
-  t.c = __shfl_sync(kFull, a.c, 0);
+// The sum of the 32 lanes' accumulators (kFrom = 16), or of each group of
+// 2 x kFrom lanes, in every lane: a butterfly of symmetric merges, so all
+// lanes hold the same bits.
+template <int kFrom>
+__device__ __forceinline__ void lanes_total(Acc<float> &a) {
+#pragma unroll
+  for (int off = kFrom; off > 0; off >>= 1) {
+    Acc<float> o;
+    o.s = __shfl_xor_sync(kFull, a.s, off);
+    o.c = __shfl_xor_sync(kFull, a.c, off);
+    a.merge(o);
+  }
 }
-__device__ __forceinline__ void bcast_acc(const Acc<double> &a, Acc<double> &t) { t.s = __shfl_sync(kFull, a.s, 0); }
+template <int kFrom>
+__device__ __forceinline__ void lanes_total(Acc<double> &a) {
+#pragma unroll
+  for (int off = kFrom; off > 0; off >>= 1) a.s += __shfl_xor_sync(kFull, a.s, off);
+}
 
 // State of the solve a group (a CTA or a cluster) works on; thread 0 of each
 // CTA updates its copy from the group's totals, so all copies agree.
@@ -1772,7 +1793,7 @@ template <typename T>
 struct ResShared {
   SolveDev sd;
   ResState st;
-  Acc<T> red[kResMaxWarps][3];
+  Acc<T> red[2][kResMaxWarps][3];  // [buffer][warp][sum]
   __align__(16) Acc<T> inbox[2][kMaxCluster][3];  // [buffer][sender rank][sum]
   int task;
 };
@@ -1914,58 +1935,119 @@ __device__ void res_never_ran(const ResArgs &a, int s) {
   a.final_sc[s] = f;
 }
 
+// The warp's totals of NA accumulators: ends with sum k in lanes 16 k .. 16 k
+// + 15 (NA = 2: the halves of the warp exchange a sum each at the first step
+// and then reduce one sum, half the shuffles and additions of two butterflies)
+// or, NA = 1, in every lane.
+template <typename T>
+__device__ __forceinline__ Acc<T> warp_fold(const Acc<T> &a) {
+  Acc<T> t = a;
+  lanes_total<16>(t);
+  return t;
+}
+__device__ __forceinline__ Acc<float> lane_xor16(const Acc<float> &a) {
+  Acc<float> o;
+  o.s = __shfl_xor_sync(kFull, a.s, 16);
+  o.c = __shfl_xor_sync(kFull, a.c, 16);
+  return o;
+}
+__device__ __forceinline__ Acc<double> lane_xor16(const Acc<double> &a) {
+  Acc<double> o;
+  o.s = __shfl_xor_sync(kFull, a.s, 16);
+  return o;
+}
+template <typename T>
+__device__ __forceinline__ Acc<T> warp_fold(const Acc<T> &a0, const Acc<T> &a1) {
+  const bool up = (threadIdx.x & 16) != 0;
+  Acc<T> keep = up ? a1 : a0;
+  keep.merge(lane_xor16(up ? a0 : a1));
+  lanes_total<8>(keep);
+  return keep;
+}
+__device__ __forceinline__ Acc<float> lane_get(const Acc<float> &a, int lane) {
+  Acc<float> o;
+  o.s = __shfl_sync(kFull, a.s, lane);
+  o.c = __shfl_sync(kFull, a.c, lane);
+  return o;
+}
+__device__ __forceinline__ Acc<double> lane_get(const Acc<double> &a, int lane) {
+  Acc<double> o;
+  o.s = __shfl_sync(kFull, a.s, lane);
+  return o;
+}
+
+// Pairs of a group's sums: the accumulators a[0], a[1], ... two at a time.
+// Totals of each warp into red (merge index: warp).
+template <typename T, int NA>
+__device__ __forceinline__ void warps_to_red(Acc<T> (&a)[NA], Acc<T> (*red)[3]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NA; k += 2) {
+    const int k2 = k + 1 < NA ? k + 1 : k;
+    const Acc<T> t = k2 > k ? warp_fold(a[k], a[k2]) : warp_fold(a[k]);
+    if (lane == 0) red[warp][k] = t;
+    if (k2 > k && lane == 16) red[warp][k2] = t;
+  }
+}
+// The merge of entries [0, n) of `e` (n <= 16), sums k and k2 in the two
+// halves of the warp.
+template <typename T>
+__device__ __forceinline__ Acc<T> merge_entries(const Acc<T> (*e)[3], int n, int k, int k2) {
+  const int i = threadIdx.x & 15;
+  Acc<T> m;
+  if (i < n) m = e[i][(threadIdx.x & 16) ? k2 : k];
+  lanes_total<8>(m);
+  return m;
+}
+
+struct NoWork {
+  __device__ __forceinline__ void operator()() const {}
+};
+
 // Sums of NA accumulators over the group: this CTA alone, or every CTA of the
-// cluster.  Thread 0 of each CTA ends with the group totals in `out`.  The
-// lanes of a warp, the warps of a CTA and the CTAs of a cluster are merged by
-// fixed shuffle trees (error-free TwoSum pairs in the FP32 bulk): warp 0
-// merges the warps' partials; in a cluster its lanes r < cluster size send
-// the CTA's total to CTA r's inbox (buffer `buf`, slot of this CTA's rank),
-// and after the cluster barrier warp 0 of every CTA merges its inbox, so all
-// CTAs hold bitwise the same totals.  The inbox alternates between two
-// buffers: a buffer is written again only two sums later, after a barrier
-// that every reader of its previous contents has passed.
-template <typename T, int NA, bool kCluster>
-__device__ __forceinline__ void group_sum(Acc<T> (&a)[NA], ResShared<T> &sh, int &buf, Acc<T> (&out)[NA]) {
+// cluster.  The lanes of a warp, the warps of a CTA and the CTAs of a cluster
+// are merged by butterflies of fixed order (error-free TwoSum pairs in the
+// FP32 bulk).  In a cluster, warp 0 merges the warps' partials and its lanes
+// send the CTA's totals to every CTA's inbox (slot of this CTA's rank); after
+// the cluster barrier the inbox is merged.  FP32 bulk: every warp does the
+// last merge itself, so every thread ends with the totals and takes the
+// decision that follows without a barrier (two block barriers fewer per CG
+// step); FP64: warp 0 alone (16 warps' merges would load the FP64 pipe).
+// `work` is what each thread does between its arrival and its wait.
+// Both arrays alternate between two buffers: a buffer is written again only
+// two sums later, after a barrier that every reader of its previous contents
+// has passed.
+template <typename T, int NA, bool kCluster, typename Work>
+__device__ __forceinline__ void group_sum(Acc<T> (&a)[NA], ResShared<T> &sh, int &buf, Acc<T> (&out)[NA],
+                                          const Work &work) {
+  static_assert(kResMaxWarps <= 16 && kMaxCluster <= 16, "merged within 16 lanes");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NA; ++k) warp_reduce_acc(a[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NA; ++k) sh.red[warp][k] = a[k];
-  }
+  warps_to_red<T, NA>(a, sh.red[buf]);
+  if (!kCluster) work();
   __syncthreads();
-  Acc<T> m[NA];
-  if (warp == 0) {
+  if (kCluster) {
+    const unsigned cs = cl_size(), cr = cl_rank();
+    if (warp == 0) {
 #pragma unroll
-    for (int k = 0; k < NA; ++k) {
-      if (lane < nw) m[k] = sh.red[lane][k];
-      warp_reduce_acc(m[k]);
+      for (int k = 0; k < NA; k += 2) {
+        const int k2 = k + 1 < NA ? k + 1 : k;
+        const Acc<T> m = merge_entries<T>(sh.red[buf], nw, k, k2);
+        const unsigned r = (unsigned)(lane & 15);
+        if (r < cs && (k2 > k || lane < 16)) cl_st(cl_map(&sh.inbox[buf][cr][lane < 16 ? k : k2], r), m);
+      }
     }
+    cl_arrive(warp == 0);
+    work();
+    cl_wait();
   }
-  if (!kCluster) {
-    if (threadIdx.x == 0) {
+  if (warp == 0 || sizeof(T) == 4) {
 #pragma unroll
-      for (int k = 0; k < NA; ++k) out[k] = m[k];
-    }
-    return;
-  }
-  const unsigned cs = cl_size(), cr = cl_rank();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NA; ++k) {
-      Acc<T> t;
-      bcast_acc(m[k], t);
-      if ((unsigned)lane < cs) cl_st(cl_map(&sh.inbox[buf][cr][k], (unsigned)lane), t);
-    }
-  }
-  cl_sync();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NA; ++k) {
-      Acc<T> t;
-      if ((unsigned)lane < cs) t = sh.inbox[buf][lane][k];
-      warp_reduce_acc(t);
-      if (lane == 0) out[k] = t;
+    for (int k = 0; k < NA; k += 2) {
+      const int k2 = k + 1 < NA ? k + 1 : k;
+      const Acc<T> m = kCluster ? merge_entries<T>(sh.inbox[buf], (int)cl_size(), k, k2)
+                                : merge_entries<T>(sh.red[buf], nw, k, k2);
+      out[k] = k2 > k ? lane_get(m, 0) : m;
+      if (k2 > k) out[k2] = lane_get(m, 16);
     }
   }
   buf ^= 1;
@@ -2280,17 +2362,20 @@ template <bool kRec, class Cx>
 __device__ __forceinline__ float res2_op_end(const Cx &cx, const SolveDev &sd, int o, int l, const float (&K)[8],
                                              const float (&v)[8], const float (&d)[8], const float (&off)[8],
                                              bool first, float beta) {
-  float local = 0.f, qv[8];
+  // the even and the odd cells are summed apart (the pair arithmetic of the
+  // register form); every product-sum is one explicit fused operation, so
+  // that all forms round alike
+  float local[2] = {0.f, 0.f}, qv[8];
   if (!kRec) {
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      const float q = d[c] * v[c] - off[c];
+      const float q = fmaf(d[c], v[c], -off[c]);
       const bool leaf = K[c] >= 0.f;
-      if (leaf) local = fmaf(v[c], q, local);
+      if (leaf) local[c & 1] = fmaf(v[c], q, local[c & 1]);
       qv[c] = leaf ? q : 0.f;
     }
     res2_own_store(cx, cx.sQ, cx.capD, l, (float *)sd.q, o, qv);
-    return local;
+    return __fadd_rn(local[0], local[1]);
   }
   float pp[8], pv[8];
   if (first) {
@@ -2302,17 +2387,17 @@ __device__ __forceinline__ float res2_op_end(const Cx &cx, const SolveDev &sd, i
   }
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const float w = d[c] * v[c] - off[c];
+    const float w = fmaf(d[c], v[c], -off[c]);
     const float pn = first ? v[c] : fmaf(beta, pp[c], v[c]);
     const float qn = first ? w : fmaf(beta, qv[c], w);
     const bool leaf = K[c] >= 0.f;
-    if (leaf) local = fmaf(pn, qn, local);
+    if (leaf) local[c & 1] = fmaf(pn, qn, local[c & 1]);
     qv[c] = leaf ? qn : 0.f;
     pv[c] = pn;
   }
   res2_own_store(cx, cx.sP, cx.cap, l, (float *)sd.p0, o, pv);
   res2_own_store(cx, cx.sQ, cx.capD, l, (float *)sd.q, o, qv);
-  return local;
+  return __fadd_rn(local[0], local[1]);
 }
 
 // Step 2 on own oct o: the stencil of v (p, or z with the q recurrence) from
@@ -2441,15 +2526,18 @@ __device__ __forceinline__ void res2_upd_oct(const Cx &cx, const SolveDev &sd, i
   res2_own(cx, cx.sD, cx.capD, l, (const float *)sd.dg, o, true, d);
   res2_own(cx, cx.sQ, cx.capD, l, (const float *)sd.q, o, true, q);
   res2_own(cx, cx.sE, cx.capD, l, (const float *)sd.e, o, true, e);
+  float srz[2] = {0.f, 0.f}, srr[2] = {0.f, 0.f};
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const float r = d[c] * z[c] - alpha * q[c];
-    const float zn = r * rcp_approx(d[c]);
-    lrz = fmaf(r, zn, lrz);
-    lrr = fmaf(r, r, lrr);
+    const float r = fmaf(-alpha, q[c], __fmul_rn(d[c], z[c]));
+    const float zn = __fmul_rn(r, rcp_approx(d[c]));
+    srz[c & 1] = fmaf(r, zn, srz[c & 1]);
+    srr[c & 1] = fmaf(r, r, srr[c & 1]);
     z[c] = zn;
-    e[c] += alpha * p[c];
+    e[c] = fmaf(alpha, p[c], e[c]);
   }
+  lrz = __fadd_rn(srz[0], srz[1]);
+  lrr = __fadd_rn(srr[0], srr[1]);
   res2_own_store(cx, cx.sZ, cx.cap, l, (float *)sd.z, o, z);
   if (cx.qrec && cx.grid && l < cx.cap) st8((float *)sd.z + 8 * o, z);
   res2_own_store(cx, cx.sE, cx.capD, l, (float *)sd.e, o, e);
@@ -2517,13 +2605,15 @@ __device__ __forceinline__ unsigned atom_add_acq_rel_u32(unsigned *p, unsigned v
 // other lanes read after lane 0's acquire and a warp barrier), the others
 // poll the counter with every lane's acquire loads and a short back-off.
 // Returns false, in every lane, when the wait gave up (then *gerr = 1).
-__device__ bool grid_arrive_wait(const ResArgs &a) {
-  const unsigned expect = a.g_expect > 0 ? (unsigned)a.g_expect : gridDim.x;
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ unsigned grid_arrive(const ResArgs &a) {  // lane 0's counter value before, in every lane
   unsigned old = 0;
-  if (lane == 0) old = atom_add_acq_rel_u32(a.gbar, 1u);
+  if ((threadIdx.x & 31) == 0) old = atom_add_acq_rel_u32(a.gbar, 1u);
   old = __shfl_sync(kFull, old, 0);
   __syncwarp();
+  return old;
+}
+__device__ bool grid_wait(const ResArgs &a, unsigned old) {
+  const unsigned expect = a.g_expect > 0 ? (unsigned)a.g_expect : gridDim.x;
   const unsigned target = (old / expect + 1u) * expect;
   if (old + 1u == target) return true;
   unsigned ns = 16;
@@ -2531,7 +2621,7 @@ __device__ bool grid_arrive_wait(const ResArgs &a) {
     const unsigned v = ld_acquire_u32(a.gbar);
     if (__all_sync(kFull, (int)(v - target) >= 0)) return true;
     if (it >= kGridSpinLimit) {
-      if (lane == 0) atomicOr(a.gerr, 1);
+      if ((threadIdx.x & 31) == 0) atomicOr(a.gerr, 1);
       return false;
     }
     __nanosleep(ns);
@@ -2545,7 +2635,7 @@ __device__ bool grid_arrive_wait(const ResArgs &a) {
 __device__ bool grid_sync(const ResArgs &a, int *flag) {
   __syncthreads();
   if (threadIdx.x < 32) {
-    const bool ok = grid_arrive_wait(a);
+    const bool ok = grid_wait(a, grid_arrive(a));
     if (threadIdx.x == 0) *flag = ok ? 1 : 0;
   }
   __syncthreads();
@@ -2553,40 +2643,34 @@ __device__ bool grid_sync(const ResArgs &a, int *flag) {
 }
 
 // Sums of NA accumulators over every CTA of the launch.  Each CTA's total
-// (the same shuffle trees as a cluster's) goes to its slot of gpart (buffer
-// `buf`) before the CTA arrives at the grid barrier; once the barrier is
-// complete, warp 0 of every CTA merges all slots in rank order -- lane j
-// takes ranks j, j + 32, ..., every load issued before the merges -- with a
-// shuffle tree, so all CTAs hold bitwise the same totals.  Thread 0 ends
-// with them in `out`; the return value (thread 0) is false when its wait gave
-// up.  The slots alternate between two buffers: a buffer is written again
-// only two sums later, after a barrier that every reader has passed.
+// goes to its slot of gpart (buffer `buf`) before the CTA arrives at the grid
+// barrier; once the barrier is complete, warp 0 of every CTA merges all slots
+// in rank order -- lane j takes ranks j, j + 32, ..., every load issued before
+// the merges -- with a butterfly, so all CTAs hold bitwise the same totals.
+// Every thread ends with them in `out`, and with false when the CTA's wait
+// gave up.  The slots alternate between two buffers: a buffer is written
+// again only two sums later, after a barrier that every reader has passed.
 constexpr int kGridMaxPerLane = 8;  // up to 256 CTAs in the launch
-template <typename T, int NA>
-__device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, int &buf, Acc<T> (&out)[NA]) {
+template <typename T, int NA, typename Work>
+__device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, int &buf, Acc<T> (&out)[NA],
+                         const Work &work) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NA; ++k) warp_reduce_acc(a[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NA; ++k) sh.red[warp][k] = a[k];
-  }
+  warps_to_red<T, NA>(a, sh.red[buf]);
   __syncthreads();
-  bool ok = true;
   if (warp == 0) {
-    Acc<T> m[NA];
-#pragma unroll
-    for (int k = 0; k < NA; ++k) {
-      if (lane < nw) m[k] = sh.red[lane][k];
-      warp_reduce_acc(m[k]);
-    }
     const unsigned G = gridDim.x;
     double *slots = ra.gpart + (size_t)buf * (G + 1) * 3;  // [G] CTA slots of 3 sums (FP32 bulk: (hi, lo) pairs)
-    if (lane == 0) {
 #pragma unroll
-      for (int k = 0; k < NA; ++k) Slot<T>::store(slots + blockIdx.x * 3 + k, m[k]);
+    for (int k = 0; k < NA; k += 2) {
+      const int k2 = k + 1 < NA ? k + 1 : k;
+      const Acc<T> m = merge_entries<T>(sh.red[buf], nw, k, k2);
+      if (lane == 0) Slot<T>::store(slots + blockIdx.x * 3 + k, m);
+      if (k2 > k && lane == 16) Slot<T>::store(slots + blockIdx.x * 3 + k2, m);
     }
-    ok = grid_arrive_wait(ra);
+    __syncwarp();
+    const unsigned old = grid_arrive(ra);
+    work();
+    const bool ok = grid_wait(ra, old);
     if (ok) {
 #pragma unroll
       for (int k = 0; k < NA; ++k) {
@@ -2598,23 +2682,31 @@ __device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, i
         }
 #pragma unroll
         for (int i = 0; i < kGridMaxPerLane; ++i) t.merge(v[i]);
-        warp_reduce_acc(t);
-        if (lane == 0) out[k] = t;
+        lanes_total<16>(t);
+        if (lane == 0) sh.inbox[buf][0][k] = t;
       }
     }
+    if (lane == 0) sh.task = ok ? 1 : 0;
+  } else {
+    work();
   }
+  __syncthreads();
+  const bool ok = sh.task != 0;
+#pragma unroll
+  for (int k = 0; k < NA; ++k) out[k] = sh.inbox[buf][0][k];
   buf ^= 1;
   return ok;
 }
 
 // The group's sum and barrier for group kind kG (0 one CTA, 1 a cluster, 2
-// the whole GPU); only the whole-GPU forms can fail: the sum reports it to
-// thread 0 (which holds the totals), the barrier to every thread.
-template <int NA, int kG, typename T>
+// the whole GPU); only the whole-GPU forms can fail, which every thread is told.
+// The totals: in every thread, but in thread 0 (warp 0) only for the FP64
+// sums of one CTA or a cluster.
+template <int NA, int kG, typename T, typename Work = NoWork>
 __device__ __forceinline__ bool res2_sum(Acc<T> (&acc)[NA], ResShared<T> &sh, const ResArgs &a, int &buf,
-                                         Acc<T> (&tot)[NA]) {
-  if (kG == 2) return grid_sum<T, NA>(acc, sh, a, buf, tot);
-  group_sum<T, NA, kG == 1>(acc, sh, buf, tot);
+                                         Acc<T> (&tot)[NA], const Work &work = Work()) {
+  if (kG == 2) return grid_sum<T, NA>(acc, sh, a, buf, tot, work);
+  group_sum<T, NA, kG == 1>(acc, sh, buf, tot, work);
   return true;
 }
 template <int kG, typename T>
@@ -2833,7 +2925,515 @@ __device__ bool res2_solve(const ResArgs &a, int s, ResShared<float> &sh, int &b
   return res2_solve_l<kG, Res2Three>(a, s, sh, buf);
 }
 
-template <bool kGlobal>
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// Resident solver with the CG state in registers and shared memory (FP32 bulk)
+// ---------------------------------------------------------------------------
+//
+// The default form of the FP32-bulk resident solver (512 threads, q by the
+// recurrence, decisions in FP32, state on chip), for runs of up to 2 048 octs
+// per CTA.  Bound: shared memory.  With every array in shared memory a CG
+// iteration moved 180 wavefronts per warp of octs through it, so the arrays
+// that only an oct's own thread reads stay in that thread's registers: thread
+// t owns octs t, t + 512, ... of the run, R of them at most.
+//   R = 2 (up to 1 024 octs): p, q, D and e in registers, K and z in shared
+//         memory: 102 wavefronts; a face's address is kept per oct (24 bytes).
+//   R = 4 (up to 2 048 octs): p and q in registers, K, z and D in shared
+//         memory, e in global memory (one read and one write per iteration);
+//         a face is coded as (rank, local index) in 16 bits.
+// Cells are worked on in x pairs by the packed FP32 instructions (two cells
+// per instruction: the pairs are what a 64-bit shared access holds), which cut
+// the arithmetic of the y and z faces and of the vector updates by half; each
+// lane of a packed operation rounds as the scalar one, so the results are
+// bitwise those of the other forms of this solver.
+// Measured (us per CG iteration of one level, refinement passes and call
+// included, shared-memory form -> this one): 512 octs on one CTA 4.0 -> 3.1,
+// 2 028 on one CTA 11.2 -> 8.3, 4 096 on 4 CTAs 6.8 -> 5.1, 8 000 on 8 CTAs
+// 7.3 -> 5.7, 32 768 on 16 CTAs 13.0 -> 9.3, on the whole GPU 11.2 -> 7.5.
+
+namespace {
+
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &x, float &y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float x, y;
+  unpack2(v, x, y);
+  return __fadd_rn(x, y);
+}
+template <bool kRemote>
+__device__ __forceinline__ f32x2 lds64(uint32_t a) {
+  f32x2 v;
+  if (kRemote) asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(a));
+  else asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts64(uint32_t a, f32x2 v) {
+  asm volatile("st.shared.b64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+template <bool kRemote>
+__device__ __forceinline__ float lds32(uint32_t a) {
+  return kRemote ? ldscf(a) : ldsf(a);
+}
+
+// The layout of a CTA's shared memory: pair planes (see Res2Ctx) of z, then of
+// -hK, then of D (R = 2: only handed from the residual pass to the threads'
+// registers), each cap + 1 octs (oct cap: the stand-in neighbour),
+// then the face codes, six per oct: R = 2 the shared address of the
+// neighbour's z row (its -hK row lies kToK bytes further), R = 4 16-bit codes,
+// two per word; plane d of the codes holds word d of every oct.  In a
+// whole-GPU group a neighbour owned by another CTA is coded as kFarOct + its
+// oct (R = 2) or kCodeGlobal (R = 4).
+template <int R>
+struct Res3 {
+  static constexpr int cap = 512 * R;
+  static constexpr uint32_t S = (uint32_t)(cap + 1) * 8u;  // bytes of one pair plane
+  static constexpr uint32_t kToK = 4u * S;
+  static constexpr uint32_t oD = 8u * S;
+  static constexpr uint32_t oC = 12u * S;
+  static constexpr int words = R == 2 ? 6 : 3;
+  static constexpr size_t bytes = oC + (size_t)words * 4 * cap;
+};
+static_assert(Res3<4>::bytes <= kRes2SmemBytes && Res3<2>::bytes <= kRes2SmemBytes, "fits the kernel's allocation");
+constexpr uint32_t kFarOct = 0x80000000u;
+
+// The off-diagonal part of the stencil on the cells of an oct across the face
+// in direction DIR, subtracted from w (nk: -hK of the own cells).
+template <int DIR, bool kRemote, uint32_t S, uint32_t kToK>
+__device__ __forceinline__ void res3_face(uint32_t a, const f32x2 (&nk)[4], f32x2 (&w)[4]) {
+  constexpr int A = DIR >> 1, side = DIR & 1, NB = 1 - side;
+  if constexpr (A == 0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float kn = lds32<kRemote>(a + kToK + k * S + 4u * NB), zn = lds32<kRemote>(a + k * S + 4u * NB);
+      float k0, k1, w0, w1;
+      unpack2(nk[k], k0, k1);
+      unpack2(w[k], w0, w1);
+      if (side == 0) w0 = fmaf(__fadd_rn(k0, kn), zn, w0);
+      else w1 = fmaf(__fadd_rn(k1, kn), zn, w1);
+      w[k] = pack2(w0, w1);
+    }
+  } else {
+    constexpr int bit = 1 << (A - 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (((k >> (A - 1)) & 1) != side) continue;
+      const int j = k ^ bit;
+      const f32x2 kn = lds64<kRemote>(a + kToK + j * S), zn = lds64<kRemote>(a + j * S);
+      w[k] = fma2(add2(nk[k], kn), zn, w[k]);
+    }
+  }
+}
+// ... with the neighbour's rows in global memory (a whole-GPU group).
+template <int DIR>
+__device__ __forceinline__ void res3_face_far(const SolveDev &sd, int g, float h, const f32x2 (&nk)[4],
+                                              f32x2 (&w)[4]) {
+  constexpr int A = DIR >> 1, side = DIR & 1, NB = 1 - side;
+  float Kn[8], Zn[8];
+  ld_face<A, NB>((const float *)sd.KT + 8 * (size_t)g, Kn);
+  ldc_face<A, NB>((const float *)sd.z + 8 * (size_t)g, Zn);
+  float k[8], wv[8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    unpack2(nk[i], k[2 * i], k[2 * i + 1]);
+    unpack2(w[i], wv[2 * i], wv[2 * i + 1]);
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    if (((c >> A) & 1) != side) continue;
+    const int j = c ^ (1 << A);
+    wv[c] = fmaf(__fadd_rn(k[c], -__fmul_rn(Kn[j], h)), Zn[j], wv[c]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w[i] = pack2(wv[2 * i], wv[2 * i + 1]);
+}
+
+template <int kG, int R, int DIR>
+__device__ __forceinline__ void res3_dir(const SolveDev &sd, uint32_t base, int o, uint32_t code, float h,
+                                         const f32x2 (&nk)[4], f32x2 (&w)[4]) {
+  using L = Res3<R>;
+  if (R == 2) {
+    if (kG == 2 && (code & kFarOct)) res3_face_far<DIR>(sd, (int)(code & ~kFarOct), h, nk, w);
+    else res3_face<DIR, kG == 1, L::S, L::kToK>(code, nk, w);
+  } else {
+    const uint32_t c = (code >> (16 * (DIR & 1))) & 0xFFFFu;
+    if (kG == 2 && c == kCodeGlobal) {
+      res3_face_far<DIR>(sd, __ldg(sd.nbr + 6 * (size_t)o + DIR), h, nk, w);
+    } else {
+      uint32_t at = base + (c & 0xFFFu) * 8u;
+      if (kG == 1) at = cl_map_s(at, c >> 12);
+      res3_face<DIR, kG == 1, L::S, L::kToK>(at, nk, w);
+    }
+  }
+}
+
+// Step 1+2 on own oct o (local index l): w = D z - sum C z_j, p = z + beta p,
+// q = w + beta q; returns the oct's p.q.
+template <int kG, int R>
+__device__ __forceinline__ float res3_op(const SolveDev &sd, uint32_t base, int o, int l, float h, f32x2 beta,
+                                         bool all_leaf, const f32x2 (&D)[4], f32x2 (&p)[4], f32x2 (&q)[4]) {
+  using L = Res3<R>;
+  const uint32_t row = base + (uint32_t)l * 8u;
+  uint32_t code[L::words];
+#pragma unroll
+  for (int d = 0; d < L::words; ++d)
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(code[d]) : "r"(base + L::oC + (uint32_t)(d * L::cap + l) * 4u));
+  f32x2 nk[4], v[4], w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    nk[k] = lds64<false>(row + L::kToK + k * L::S);
+    v[k] = lds64<false>(row + k * L::S);
+    w[k] = 0ull;
+  }
+  // in-oct faces: x inside a pair, y and z between pairs
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float k0, k1, v0, v1, w0, w1;
+    unpack2(nk[k], k0, k1);
+    unpack2(v[k], v0, v1);
+    const float C = __fadd_rn(k0, k1);
+    w0 = __fmul_rn(C, v1);
+    w1 = __fmul_rn(C, v0);
+    w[k] = pack2(w0, w1);
+  }
+#pragma unroll
+  for (int b = 1; b <= 2; b <<= 1) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k & b) continue;
+      const f32x2 C = add2(nk[k], nk[k | b]);
+      w[k] = fma2(C, v[k | b], w[k]);
+      w[k | b] = fma2(C, v[k], w[k | b]);
+    }
+  }
+  constexpr int dw = R == 2 ? 1 : 2;
+  res3_dir<kG, R, 0>(sd, base, o, code[0 / dw], h, nk, w);
+  res3_dir<kG, R, 1>(sd, base, o, code[1 / dw], h, nk, w);
+  res3_dir<kG, R, 2>(sd, base, o, code[2 / dw], h, nk, w);
+  res3_dir<kG, R, 3>(sd, base, o, code[3 / dw], h, nk, w);
+  res3_dir<kG, R, 4>(sd, base, o, code[4 / dw], h, nk, w);
+  res3_dir<kG, R, 5>(sd, base, o, code[5 / dw], h, nk, w);
+  f32x2 dot = 0ull;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const f32x2 d = R == 2 ? D[k] : lds64<false>(row + L::oD + k * L::S);
+    p[k] = fma2(beta, p[k], v[k]);
+    q[k] = fma2(beta, q[k], fma2(d, v[k], w[k]));
+    if (!all_leaf) {  // q = 0 off the leaves
+      float k0, k1, q0, q1;
+      unpack2(nk[k], k0, k1);
+      unpack2(q[k], q0, q1);
+      q[k] = pack2(k0 <= 0.f ? q0 : 0.f, k1 <= 0.f ? q1 : 0.f);
+    }
+    dot = fma2(p[k], q[k], dot);
+  }
+  return sum2(dot);
+}
+
+// Step 3 on own oct o: r = D z - alpha q, z = r x rcp(D), the sums.
+template <int kG, int R>
+__device__ __forceinline__ void res3_upd(const SolveDev &sd, uint32_t base, int o, int l, f32x2 nalpha,
+                                         const f32x2 (&D)[4], const f32x2 (&q)[4], float &lrz, float &lrr) {
+  using L = Res3<R>;
+  const uint32_t row = base + (uint32_t)l * 8u;
+  f32x2 srz = 0ull, srr = 0ull, zn[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const f32x2 d = R == 2 ? D[k] : lds64<false>(row + L::oD + k * L::S);
+    const f32x2 r = fma2(nalpha, q[k], mul2(d, lds64<false>(row + k * L::S)));
+    float d0, d1;
+    unpack2(d, d0, d1);
+    zn[k] = mul2(r, pack2(rcp_approx(d0), rcp_approx(d1)));
+    srz = fma2(r, zn[k], srz);
+    srr = fma2(r, r, srr);
+    sts64(row + k * L::S, zn[k]);
+  }
+  if (kG == 2)
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"((float *)sd.z + 8 * (size_t)o), "l"(zn[0]),
+                 "l"(zn[1]), "l"(zn[2]), "l"(zn[3])
+                 : "memory");
+  lrz = sum2(srz);
+  lrr = sum2(srr);
+}
+
+// Step 3's e += alpha p on own oct o, which nothing else waits for: done
+// between a thread's arrival at the sum and its wait.
+template <int R>
+__device__ __forceinline__ void res3_e(const SolveDev &sd, int o, f32x2 alpha, const f32x2 (&p)[4], f32x2 (&e)[4]) {
+  if (R == 4) {
+    float *eg = (float *)sd.e + 8 * (size_t)o;
+    f32x2 ev[4];
+    asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(ev[0]), "=l"(ev[1]), "=l"(ev[2]), "=l"(ev[3])
+                 : "l"(eg));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ev[k] = fma2(alpha, p[k], ev[k]);
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(eg), "l"(ev[0]), "l"(ev[1]), "l"(ev[2]), "l"(ev[3])
+                 : "memory");
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) e[k] = fma2(alpha, p[k], e[k]);
+  }
+}
+
+// One solve by one group (see res2_solve_l, whose state machine and decisions
+// these are).  Every thread takes the step decisions itself from the group's
+// totals, so no barrier follows them; thread 0 keeps the counters.
+template <int kG, int R>
+__device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
+  using L = Res3<R>;
+  constexpr int wd = (int)(sizeof(SolveDev) / 8);
+  for (int w = threadIdx.x; w < wd; w += blockDim.x)
+    reinterpret_cast<unsigned long long *>(&sh.sd)[w] = reinterpret_cast<const unsigned long long *>(a.solves + s)[w];
+  const unsigned cs = kG == 2 ? gridDim.x : (kG == 1 ? cl_size() : 1u);
+  const unsigned cr = kG == 2 ? blockIdx.x : (kG == 1 ? cl_rank() : 0u);
+  if (threadIdx.x == 0) {
+    ResState z;
+    memset(&z, 0, sizeof(z));
+    z.phase = kRefine;
+    z.status = ATS_OK;
+    sh.st = z;
+    if (a.t_solve && cr == 0) a.t_solve[2 * s] = globaltimer_ns();
+  }
+  __syncthreads();
+  const SolveDev &sd = sh.sd;
+  const int n = sd.n_oct;
+  const int chunk = (int)((n + (int)cs - 1) / (int)cs);
+  const int lo = min(n, (int)cr * chunk);
+  const int run = min(n, lo + chunk) - lo;
+  const float h = (float)sd.h;
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(res2_smem);
+  // stage in: -hK, the face codes, the stand-in row
+  if (threadIdx.x < 4) {
+    sts64(base + (uint32_t)L::cap * 8u + threadIdx.x * L::S, 0ull);
+    sts64(base + (uint32_t)L::cap * 8u + L::kToK + threadIdx.x * L::S, pack2(1.f, 1.f));
+  }
+  bool leafs = true;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int l = (int)threadIdx.x + 512 * r;
+    if (l >= run) continue;
+    const int o = lo + l;
+    float K[8];
+    ld8_ro((const float *)sd.KT + 8 * (size_t)o, K);
+    res2_scale_K(h, K);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      leafs = leafs && K[2 * k] >= 0.f && K[2 * k + 1] >= 0.f;
+      sts64(base + (uint32_t)l * 8u + L::kToK + k * L::S, pack2(-K[2 * k], -K[2 * k + 1]));
+    }
+    int g[6];
+    load_nbr6(sd.nbr, o, g);
+    check_nbr6(g, n);
+    uint32_t c[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      unsigned rank = kG == 1 ? cr : 0u;
+      int at = L::cap;
+      bool far = false;
+      if (g[d] >= 0) {
+        const int gr = g[d] / chunk;
+        far = kG == 2 && (unsigned)gr != cr;
+        at = g[d] - gr * chunk;
+        if (kG == 1) rank = (unsigned)gr;
+      }
+      if (R == 2) {
+        c[d] = base + (uint32_t)at * 8u;
+        if (kG == 1) c[d] = cl_map_s(c[d], rank);
+        if (far) c[d] = kFarOct | (uint32_t)g[d];
+      } else {
+        c[d] = far ? (uint32_t)kCodeGlobal : ((rank << 12) | (uint32_t)at);
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < L::words; ++d) {
+      const uint32_t v = R == 2 ? c[d] : (c[2 * d] | (c[2 * d + 1] << 16));
+      asm volatile("st.shared.u32 [%0], %1;" ::"r"(base + L::oC + (uint32_t)(d * L::cap + l) * 4u), "r"(v) : "memory");
+    }
+  }
+  const bool all_leaf = __syncthreads_and(leafs);
+  const bool want_x = sd.stop_rule == ATS_STOP_CERTIFIED;
+  bool alive = true;
+  for (;;) {
+    // FP64 residual pass: z and D of the next inner solve
+    {
+      Acc<float> acc[3];
+#pragma unroll 1
+      for (int l = (int)threadIdx.x; l < run; l += 512) {
+        float zo[8], dv[8];
+        ref_oct_values<float, true, true>(sd, lo + l, want_x, acc[0], acc[1], acc[2], zo, dv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          sts64(base + (uint32_t)l * 8u + k * L::S, pack2(zo[2 * k], zo[2 * k + 1]));
+          sts64(base + (uint32_t)l * 8u + L::oD + k * L::S, pack2(dv[2 * k], dv[2 * k + 1]));
+        }
+        if (kG == 2) st8((float *)sd.z + 8 * (size_t)(lo + l), zo);
+      }
+      Acc<float> tot[3];
+      alive = res2_sum<3, kG>(acc, sh, a, buf, tot);
+      if (threadIdx.x == 0) {
+        if (alive) refine_decision(sh.st, sd, tot[0].get(), tot[1].get(), tot[2].get());
+        else res2_timeout(sh.st);
+      }
+      __syncthreads();
+    }
+    if (sh.st.phase == kDone) break;
+    f32x2 D[R][4], p[R][4], q[R][4], e[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int l = (int)threadIdx.x + 512 * r;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        p[r][k] = q[r][k] = e[r][k] = 0ull;
+        if (R == 2) D[r][k] = l < run ? lds64<false>(base + (uint32_t)l * 8u + L::oD + k * L::S) : 0ull;
+      }
+    }
+    float rz = sh.st.rzf, beta = 0.f;  // the first step's p = z, q = w
+    const float t2 = sh.st.t2f;
+    const int left = min(sd.max_iter - sh.st.iters, sd.inner_max);
+    int it = 0;
+    bool conv = false, brk = false;
+    while (it < left && !conv) {
+      {
+        Acc<float> acc[1], tot[1];
+        const f32x2 b2 = pack2(beta, beta);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int l = (int)threadIdx.x + 512 * r;
+          if (l < run) acc[0].add_value(res3_op<kG, R>(sd, base, lo + l, l, h, b2, all_leaf, D[r], p[r], q[r]));
+        }
+        alive = res2_sum<1, kG>(acc, sh, a, buf, tot);
+        const float pq = tot[0].val();
+        brk = !(rz >= 0.f) || !isfinite(rz) || !(pq > 0.f) || !isfinite(pq);
+        if (brk || !alive) break;
+        beta = __fdiv_rn(rz, pq);  // alpha
+      }
+      {
+        Acc<float> acc[2], tot[2];
+        const f32x2 a2 = pack2(beta, beta), n2 = pack2(-beta, -beta);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int l = (int)threadIdx.x + 512 * r;
+          if (l >= run) continue;
+          float lrz, lrr;
+          res3_upd<kG, R>(sd, base, lo + l, l, n2, D[r], q[r], lrz, lrr);
+          acc[0].add_value(lrz);
+          acc[1].add_value(lrr);
+        }
+        alive = res2_sum<2, kG>(acc, sh, a, buf, tot, [&] {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int l = (int)threadIdx.x + 512 * r;
+            if (l < run) res3_e<R>(sd, lo + l, a2, p[r], e[r]);
+          }
+        });
+        if (!alive) break;
+        const float rz_new = tot[0].val();
+        beta = __fdiv_rn(rz_new, rz);
+        rz = rz_new;
+        conv = tot[1].val() <= t2 || rz_new == 0.f;
+        ++it;
+      }
+    }
+    // x += e; the next residual pass reads the neighbours' x
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int l = (int)threadIdx.x + 512 * r;
+      if (l >= run || brk || !alive) continue;
+      if (R == 4) {
+        res_xpe_oct<float>(sd, lo + l);
+      } else {
+        double xv[8];
+        double *x = sd.x64 + 8 * (size_t)(lo + l);
+        ldc8(x, xv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float e0, e1;
+          unpack2(e[r][k], e0, e1);
+          xv[2 * k] += (double)e0;
+          xv[2 * k + 1] += (double)e1;
+        }
+        st8(x, xv);
+      }
+    }
+    if (threadIdx.x == 0) {
+      ResState &st = sh.st;
+      st.n_op += it + (brk ? 1 : 0);
+      st.n_first += it + (brk ? 1 : 0) > 0 ? 1 : 0;
+      st.iters += it;
+      st.inner_iters = it;
+      st.rz = rz;
+      if (!alive) {
+        res2_timeout(st);
+      } else if (brk) {
+        st.status = ATS_ERR_BREAKDOWN;
+        st.phase = kDone;
+      } else {
+        st.n_xpe += 1;
+        if (!conv && st.iters >= sd.max_iter) {
+          st.status = ATS_ERR_NOT_CONVERGED;
+          st.final_pass = 1;
+        }
+      }
+    }
+    if (!alive) break;
+    if (!res2_barrier<kG>(a, sh)) {
+      alive = false;
+      if (threadIdx.x == 0) res2_timeout(sh.st);
+      break;
+    }
+    if (brk) break;
+  }
+  __syncthreads();  // thread 0's last state update is seen by all
+  double *xd = a.x_out ? a.x_out[s] : nullptr;
+  if (xd) res2_copy_out(sd, xd, lo, lo + run, a.neg ? a.neg + s : nullptr);
+  if (threadIdx.x == 0 && cr == 0) res_finish(a, s, sh.st, n);
+  return sh.st.status != ATS_ERR_TIMEOUT;
+}
+
+template <int kG>
+__device__ bool res3_solve(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
+  const unsigned cs = kG == 2 ? gridDim.x : (kG == 1 ? cl_size() : 1u);
+  const int chunk = (int)((a.solves[s].n_oct + (int)cs - 1) / (int)cs);
+  return chunk <= Res3<2>::cap ? res3_solve_r<kG, 2>(a, s, sh, buf) : res3_solve_r<kG, 4>(a, s, sh, buf);
+}
+
+}  // namespace
+
+namespace {
+
+// Where a kernel instance keeps a solve's CG state: shared memory planes, the
+// level's global arrays, or registers and shared memory.
+constexpr int kStateShared = 0, kStateGlobal = 1, kStateRegs = 2;
+template <int kG, int kState>
+__device__ __forceinline__ bool resf_solve(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
+  if constexpr (kState == kStateRegs) return res3_solve<kG>(a, s, sh, buf);
+  else return res2_solve<kG, kState == kStateGlobal>(a, s, sh, buf);
+}
+
+template <int kState>
 __device__ void res2_cta_loop(const ResArgs &a, ResShared<float> &sh, int &buf) {
   for (;;) {
     __syncthreads();  // every thread has read the previous task and left the previous solve
@@ -2843,13 +3443,13 @@ __device__ void res2_cta_loop(const ResArgs &a, ResShared<float> &sh, int &buf) 
     if (t >= a.n_tq) break;
     int s = a.tq[t];
     if (!idx_ok(s, a.n_solves)) continue;
-    res2_solve<0, kGlobal>(a, s, sh, buf);
+    resf_solve<0, kState>(a, s, sh, buf);
   }
 }
 
 }  // namespace
 
-template <int NT, bool kGlobal>
+template <int NT, int kState>
 __global__ void __launch_bounds__(NT, 1) k_res2_cluster(ResArgs a) {
   __shared__ ResShared<float> sh;
   int buf = 0;
@@ -2863,23 +3463,23 @@ __global__ void __launch_bounds__(NT, 1) k_res2_cluster(ResArgs a) {
     const int t = sh.task;
     if (t >= a.n_cq) break;
     const int s = a.cq[t];
-    if (idx_ok(s, a.n_solves)) res2_solve<1, kGlobal>(a, s, sh, buf);
+    if (idx_ok(s, a.n_solves)) resf_solve<1, kState>(a, s, sh, buf);
     cl_sync();  // every CTA is done with the shared rows before the next stage-in rewrites them
   }
-  res2_cta_loop<kGlobal>(a, sh, buf);
+  res2_cta_loop<kState>(a, sh, buf);
 }
 
-template <int NT, bool kGlobal>
+template <int NT, int kState>
 __global__ void __launch_bounds__(NT, 1) k_res2_cta(ResArgs a) {
   __shared__ ResShared<float> sh;
   int buf = 0;
-  res2_cta_loop<kGlobal>(a, sh, buf);
+  res2_cta_loop<kState>(a, sh, buf);
 }
 
 // The whole-GPU form: every CTA of one cooperative launch takes part in
 // every solve of the grid queue, in queue order.  After a barrier wait gave
 // up, the remaining solves are not started: CTA 0 records them as timed out.
-template <int NT>
+template <int NT, int kState>
 __global__ void __launch_bounds__(NT, 1) k_res2_grid(ResArgs a) {
   __shared__ ResShared<float> sh;
   int buf = 0;
@@ -2888,7 +3488,7 @@ __global__ void __launch_bounds__(NT, 1) k_res2_grid(ResArgs a) {
     const int s = a.gq[t];
     if (!idx_ok(s, a.n_solves)) continue;
     if (alive) {
-      alive = res2_solve<2, false>(a, s, sh, buf);
+      alive = resf_solve<2, kState>(a, s, sh, buf);
     } else {
       res_never_ran(a, s);
     }
@@ -3309,7 +3909,7 @@ static int resd_cta_blocks_t() {
   return b;
 }
 
-template <int NT, bool kG>
+template <int NT, int kState>
 static cudaError_t res2_launch_k(int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only,
                                  int priority) {
   const size_t smem = kRes2SmemBytes;
@@ -3317,9 +3917,9 @@ static cudaError_t res2_launch_k(int cluster, int grid, const ResArgs &a, cudaSt
   at[0].id = cudaLaunchAttributePriority;
   at[0].val.priority = priority;
   if (a.n_cq > 0 && !cta_only) {
-    cudaError_t e = cudaFuncSetAttribute(k_res2_cluster<NT, kG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_res2_cluster<NT, kState>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess && cluster > 8)
-      e = cudaFuncSetAttribute(k_res2_cluster<NT, kG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      e = cudaFuncSetAttribute(k_res2_cluster<NT, kState>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -3332,9 +3932,9 @@ static cudaError_t res2_launch_k(int cluster, int grid, const ResArgs &a, cudaSt
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_res2_cluster<NT, kG>, a);
+    return cudaLaunchKernelEx(&cfg, k_res2_cluster<NT, kState>, a);
   }
-  cudaError_t e = cudaFuncSetAttribute(k_res2_cta<NT, kG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_res2_cta<NT, kState>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -3343,23 +3943,24 @@ static cudaError_t res2_launch_k(int cluster, int grid, const ResArgs &a, cudaSt
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_res2_cta<NT, kG>, a);
+  return cudaLaunchKernelEx(&cfg, k_res2_cta<NT, kState>, a);
 }
 
 template <int NT>
 static cudaError_t res2_launch_t(int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only,
                                  int priority) {
-  return a.cap == 0 ? res2_launch_k<NT, true>(cluster, grid, a, st, cta_only, priority)
-                    : res2_launch_k<NT, false>(cluster, grid, a, st, cta_only, priority);
+  if (a.cap == 0) return res2_launch_k<NT, kStateGlobal>(cluster, grid, a, st, cta_only, priority);
+  if (NT == 512 && a.regs) return res2_launch_k<512, kStateRegs>(cluster, grid, a, st, cta_only, priority);
+  return res2_launch_k<NT, kStateShared>(cluster, grid, a, st, cta_only, priority);
 }
 
 template <int NT>
 static int res2_clusters_t(int cluster, int cap) {
   (void)cap;
   const size_t smem = kRes2SmemBytes;
-  if (cudaFuncSetAttribute(k_res2_cluster<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (cudaFuncSetAttribute(k_res2_cluster<NT, kStateShared>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       (cluster > 8 &&
-       cudaFuncSetAttribute(k_res2_cluster<NT, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+       cudaFuncSetAttribute(k_res2_cluster<NT, kStateShared>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
     cudaGetLastError();
     return 0;
   }
@@ -3375,7 +3976,7 @@ static int res2_clusters_t(int cluster, int cap) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_res2_cluster<NT, false>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, k_res2_cluster<NT, kStateShared>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -3389,8 +3990,8 @@ static int res2_cap_t(int device) {
   int optin = 0;
   cudaFuncAttributes fa, fb;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
-      cudaFuncGetAttributes(&fa, k_res2_cluster<NT, false>) != cudaSuccess ||
-      cudaFuncGetAttributes(&fb, k_res2_cta<NT, false>) != cudaSuccess) {
+      cudaFuncGetAttributes(&fa, k_res2_cluster<NT, kStateShared>) != cudaSuccess ||
+      cudaFuncGetAttributes(&fb, k_res2_cta<NT, kStateShared>) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -3419,15 +4020,15 @@ int resident_smem_cap(int threads, int device) {
 // The whole-GPU form of a bulk precision: its kernel and dynamic shared memory.
 using ResGridKernel = void (*)(ResArgs);
 template <int NT>
-static ResGridKernel res_grid_kernel(bool fp64, size_t *smem) {
+static ResGridKernel res_grid_kernel(bool fp64, bool regs, size_t *smem) {
   *smem = fp64 ? 0 : kRes2SmemBytes;
-  return fp64 ? k_resd_grid<NT> : k_res2_grid<NT>;
+  return fp64 ? k_resd_grid<NT> : regs ? k_res2_grid<NT, kStateRegs> : k_res2_grid<NT, kStateShared>;
 }
 
 template <int NT>
 static cudaError_t res2_grid_launch_t(bool fp64, int grid, const ResArgs &a, cudaStream_t st) {
   size_t smem = 0;
-  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, &smem);
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, a.regs != 0, &smem);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -3447,7 +4048,7 @@ template <int NT>
 static int res2_grid_ctas_t(bool fp64, int device) {
   int b = 0, sms = 0;
   size_t smem = 0;
-  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, &smem);
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, false, &smem);
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, NT, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
@@ -3478,6 +4079,8 @@ cudaError_t launch_resident_grid(bool fp64, int grid, const ResArgs &a, cudaStre
 }
 
 int resident_six_cap() { return kRes2Cap6; }
+
+int resident_run_cap() { return Res3<4>::cap; }
 
 int resident_grid_ctas(bool fp64, int device) {
   int sms = 0;

@@ -275,6 +275,7 @@ struct Plan {
   int res_cluster_mid = 8, res_grid_mid = 0;
   bool res_smem = false;  // K, z, p of each CTA's octs in shared memory (FP32 bulk)
   int res_cap = 0;        // octs per CTA kept in shared memory
+  bool res_regs = false;  // the CG state in registers and shared memory (FP32 bulk)
   int res_fill = 0;       // single CTAs launched beside the clusters on the SMs they leave
   int32_t *d_queue = nullptr;   // [n_bq + n_mq + n_cq + n_tq + n_gq]
   int *d_heads = nullptr;       // [4] next position of each queue: big, cluster, CTA, middle
@@ -764,6 +765,14 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       if (P->mode[k] == 5 && clM <= 0) P->mode[k] = 1;
       if (P->mode[k] == 1 && clB <= 0) P->mode[k] = 0;
     }
+    // the register form where the options allow it and every run fits; the
+    // other forms give the same bits
+    if (grid_all > 0) P->res_grid_all = grid_all;
+    P->res_regs = P->res_smem && P->res_cap > 0 && P->res_threads == 512 && o.cg_form != 1 && !o.cg_scalars;
+    for (int k = 0; k < n; ++k) {
+      const int64_t c = group_ctas(P, P->mode[k]);
+      if (P->mode[k] != 0 && (P->levels[k]->n_oct + c - 1) / c > resident_run_cap()) P->res_regs = false;
+    }
     double w[4] = {0.0, 0.0, 0.0, 0.0};
     for (int k = 0; k < n; ++k) {
       P->n_bq += P->mode[k] == 3;
@@ -784,7 +793,6 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     P->res_clM = clM;
     P->res_clB = clB;
     plan_split(P, w);
-    if (P->n_gq > 0) P->res_grid_all = grid_all;
   }
   const int bps = tick_blocks_per_sm(P->fp64, P->paper);
   P->grid = std::max(1, std::min(P->n_items, bps * ctx->num_sms));
@@ -894,6 +902,7 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
   ra.x_out = P->res_smem ? P->d_rdst : nullptr;
   ra.neg = neg;
   ra.q_recur = P->opts.cg_form == 1 ? 0 : 1;
+  ra.regs = P->res_regs ? 1 : 0;
   ra.cells = prof ? P->d_cells + kCellCounters : nullptr;
   // every resident solve stamps its start and end (the split of the next run
   // follows them; profiling reads the timeline)
