@@ -155,12 +155,17 @@ typedef struct {
   int res_cluster;   /* resident solver: CTAs per thread-block cluster, 1..16 */
                      /* (0 = 4)                                              */
   int res_cta_octs;  /* resident solver: a level of at most this many octs is */
-                     /* solved by one CTA alone (0 = 2048 for ATS_PREC_MIXED, */
-                     /* 128 for ATS_PREC_FP64; < 0 = never)                  */
+                     /* solved by one CTA alone (0 = 1024 for ATS_PREC_MIXED, */
+                     /* 2048 when res_max_octs is given, 128 for              */
+                     /* ATS_PREC_FP64; < 0 = never)                          */
   int res_max_octs;  /* ATS_SCHED_AUTO: levels above this many octs take the  */
                      /* whole-GPU form or the tick path (see ATS_SCHED_AUTO) */
                      /* (0 = 16384 for ATS_PREC_MIXED, 2048 for              */
-                     /* ATS_PREC_FP64)                                       */
+                     /* ATS_PREC_FP64).  Mixed precision: 0 here and in       */
+                     /* res_cta_octs sizes the groups for the shortest solve  */
+                     /* (at most 1024 octs per CTA where a cluster size       */
+                     /* allows it); a limit given in either sizes them for    */
+                     /* the most solves per SM (2048 octs per CTA)            */
   int cg_scalars;    /* resident solver, mixed precision: the CG step's alpha,  */
                      /* beta and inner convergence test from the error-free   */
                      /* dot totals, 0 = rounded to FP32 (the tick path's form, */

@@ -451,14 +451,36 @@ void plan_free(Plan *P) {
   delete P;
 }
 
-// Estimated work of a level solve, to order the resident queues (largest
-// first): octs times an iteration estimate, the square root of the stiffness
+// Estimated work of a level solve (the rule of res_big_work): octs times an
+// iteration estimate, the square root of the stiffness
 // 1 + 8 h (h = dt / (2 dx^2), K ~ 1) capped by four times the oct count's
 // cube root (about twice the level's width in cells).
 double est_work(const ats_level *L) {
   const double h = 0.5 * L->dt / (L->dx * L->dx);
   const double o = (double)L->n_oct;
   return o * std::min(std::sqrt(1.0 + 8.0 * h), 4.0 * std::cbrt(o));
+}
+
+// CTAs of each solve's group, by mode
+int group_ctas(const Plan *P, int mode) {
+  switch (mode) {
+    case 1: return P->res_cluster;
+    case 3: return P->res_cluster_big;
+    case 4: return P->res_grid_all;
+    case 5: return P->res_cluster_mid;
+    default: return 1;
+  }
+}
+
+// Estimated duration (ns) of resident solve k, for the queue order and the
+// split before a completed run has measured them: its iterations (est_work's
+// estimate scaled to the counts of stiff and of barely implicit levels) times
+// a step of its group, 2.5 us for the sums and 3.5 ns per oct of a CTA's run
+// (measured on runs of 500 .. 2 000 octs).
+double est_ns(const Plan *P, int k) {
+  const ats_level *L = P->levels[k];
+  const double its = 12.0 + 20.0 * (est_work(L) / (double)L->n_oct - 1.0);
+  return its * (2500.0 + 3.5 * (double)L->n_oct / group_ctas(P, P->mode[k]));
 }
 
 // Upload the resident queues of P in work order: big-cluster solves, cluster
@@ -476,7 +498,7 @@ ats_status plan_upload_queues(Plan *P) {
     std::vector<double> w(P->n, 0.0);
     bool meas = !P->res_meas.empty();
     for (int32_t k : q) meas = meas && P->res_meas[k] > 0.0;
-    for (int32_t k : q) w[k] = meas ? P->res_meas[k] : est_work(P->levels[k]);
+    for (int32_t k : q) w[k] = meas ? P->res_meas[k] : est_ns(P, k);
     std::stable_sort(q.begin(), q.end(), [&](int32_t a, int32_t b) { return w[a] > w[b]; });
   };
   by_work(bq);
@@ -496,39 +518,50 @@ ats_status plan_upload_queues(Plan *P) {
   return ATS_OK;
 }
 
-// The CTA slots of the device, shared by the resident launches in proportion
-// to their queues' work w[0] (big clusters), w[1] (middle clusters), w[2]
-// (clusters), w[3] (single CTAs): the single CTAs get at least their share
-// (so the largest of them start at once), the big and middle clusters theirs
-// in whole clusters, and the smallest cluster class present every remaining
-// whole cluster; what is left runs single CTAs beside them.  A cluster that
-// has emptied its queue goes on with single-CTA solves.
-void plan_split(Plan *P, const double (&w)[4]) {
+// The CTA slots of the device, shared by the resident launches by their
+// queues' work w[0] (big clusters), w[1] (middle clusters), w[2] (clusters),
+// w[3] (single CTAs) in SM-time, and by the longest solve's work in each,
+// longest[]: the counts of clusters that make the class that ends last end
+// earliest (each class ends after its work over its slots, and not before its
+// longest solve), out of every combination that fits.  The single CTAs get
+// their share first (so the largest of them start at once) and every slot
+// left over; a cluster that has emptied its queue goes on with single-CTA
+// solves.  Rounding each class's share to whole clusters, largest first, left
+// the smallest clusters 16 of 152 SMs on a batch of 512 levels: they ended
+// after 27.1 ms, the other classes after 14.4 and 11.6 ms (measured).
+void plan_split(Plan *P, const double (&w)[4], const double (&longest)[4]) {
   const int slots = P->res_slots;
   const int size[3] = {P->res_cluster_big, P->res_cluster_mid, P->res_cluster};
   const int lim[3] = {P->res_clA, P->res_clM, P->res_clB};
   const int cnt[3] = {P->n_bq, P->n_mq, P->n_cq};
   const double wsum = std::max(1e-300, w[0] + w[1] + w[2] + w[3]);
   const int c_min = P->n_tq > 0 ? std::max(1, (int)std::ceil(slots * w[3] / wsum)) : 0;
-  int k[3] = {0, 0, 0};
-  int last = -1;  // the smallest cluster class present takes the remainder
-  for (int q = 0; q < 3; ++q)
-    if (cnt[q] > 0) last = q;
-  int used = c_min;
+  int lo[3], hi[3], k[3] = {0, 0, 0};
   for (int q = 0; q < 3; ++q) {
-    if (cnt[q] <= 0 || q == last) continue;
-    k[q] = std::max(1, std::min(lim[q], (int)std::lround(slots * w[q] / wsum / size[q])));
-    used += k[q] * size[q];
+    lo[q] = cnt[q] > 0 ? 1 : 0;
+    hi[q] = cnt[q] > 0 ? std::max(1, std::min(lim[q], cnt[q])) : 0;
+    k[q] = lo[q];
   }
-  if (last >= 0) k[last] = std::max(1, std::min(lim[last], (slots - used) / size[last]));
-  auto total = [&] { return k[0] * size[0] + k[1] * size[1] + k[2] * size[2] + c_min; };
-  while (total() > slots) {
-    int q_max = -1;
-    for (int q = 0; q < 3; ++q)
-      if (k[q] > 1 && (q_max < 0 || k[q] * size[q] > k[q_max] * size[q_max])) q_max = q;
-    if (q_max < 0) break;
-    --k[q_max];
-  }
+  const auto end_of = [&](int q, int n) {
+    return cnt[q] > 0 ? std::max(w[q] / ((double)n * size[q]), longest[q] / size[q]) : 0.0;
+  };
+  // (the first combination stands when not even one cluster of each class fits)
+  double best = HUGE_VAL;
+  int best_used = 0;
+  for (int i = lo[0]; i <= hi[0]; ++i)
+    for (int j = lo[1]; j <= hi[1]; ++j)
+      for (int l = lo[2]; l <= hi[2]; ++l) {
+        const int used = i * size[0] + j * size[1] + l * size[2];
+        if (used + c_min > slots) break;
+        const double t = std::max(end_of(0, i), std::max(end_of(1, j), end_of(2, l)));
+        if (t < best || (t == best && used < best_used)) {
+          best = t;
+          best_used = used;
+          k[0] = i;
+          k[1] = j;
+          k[2] = l;
+        }
+      }
   P->res_grid_big = k[0] * size[0];
   P->res_grid_mid = k[1] * size[1];
   const bool clusters = P->n_bq + P->n_mq + P->n_cq > 0;
@@ -538,24 +571,13 @@ void plan_split(Plan *P, const double (&w)[4]) {
                     : 0;
 }
 
-// CTAs of each solve's group, by mode
-int group_ctas(const Plan *P, int mode) {
-  switch (mode) {
-    case 1: return P->res_cluster;
-    case 3: return P->res_cluster_big;
-    case 4: return P->res_grid_all;
-    case 5: return P->res_cluster_mid;
-    default: return 1;
-  }
-}
-
 // After a completed run: the SM-time each class of resident solves took
 // (each solve's duration times its group's CTAs), from the solves' start and
 // end stamps; the next run splits the slots by it and orders each queue by
 // the measured durations.  Which group and layout a solve takes does not
 // change, so neither do its results.
 void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
-  double w[4] = {0.0, 0.0, 0.0, 0.0};
+  double w[4] = {0.0, 0.0, 0.0, 0.0}, longest[4] = {0.0, 0.0, 0.0, 0.0};
   int present = 0, measured = 0;
   const int cls[4] = {P->n_bq, P->n_mq, P->n_cq, P->n_tq};
   for (int q = 0; q < 4; ++q) present += cls[q] > 0;
@@ -564,7 +586,9 @@ void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
   for (int k = 0; k < P->n; ++k) {
     const int q = class_of(P->mode[k]);
     if (q < 0 || ts[2 * k + 1] <= ts[2 * k]) continue;
-    w[q] += (double)(ts[2 * k + 1] - ts[2 * k]) * group_ctas(P, P->mode[k]);
+    const double t = (double)(ts[2 * k + 1] - ts[2 * k]) * group_ctas(P, P->mode[k]);
+    w[q] += t;
+    longest[q] = std::max(longest[q], t);
   }
   for (int q = 0; q < 4; ++q) measured += (cls[q] > 0 && w[q] > 0.0);
   // each queue in the order of the measured durations (largest first)
@@ -573,7 +597,7 @@ void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
     if (class_of(P->mode[k]) >= 0 && ts[2 * k + 1] > ts[2 * k]) P->res_meas[k] = (double)(ts[2 * k + 1] - ts[2 * k]);
   P->queue_dirty = true;
   if (measured != present) return;
-  plan_split(P, w);
+  plan_split(P, w, longest);
   P->res_split_measured = true;
 }
 
@@ -583,6 +607,14 @@ void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
 // cost about 3 000: runs of 128 octs keep the pipe busy most of a step and
 // spread a level over as many SMs as that allows.
 constexpr int64_t kRun64 = 128;
+// FP32-bulk resident groups with the default limits: runs of up to 1 024 octs
+// (the register layout that keeps every private array on chip).  A step's
+// sums cost 2 to 3 us whatever the run, so the longest runs give the most
+// solves per SM and the shorter ones the shorter solve: 5 832 octs take 1.75
+// ms on 8 CTAs and 2.61 ms on 4 (7.6 and 5.7 SM-ns per oct and iteration);
+// 512 levels of 64 .. 32 768 octs take 13.9 ms with runs of up to 2 048 and
+// 16.4 ms with the shorter ones (measured).
+constexpr int64_t kRunLatency = 1024;
 
 ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const ats_solve_opts *opts_in,
                        Plan **out) {
@@ -699,7 +731,6 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     P->res_cluster_mid = 0;
   {
     const bool res_ok = o.sched != ATS_SCHED_TICK && o.stop_rule != ATS_STOP_PAPER;
-    const int64_t cta_octs = o.res_cta_octs == 0 ? (P->fp64 ? kRun64 : 2048) : o.res_cta_octs;
     // default limit: mixed precision 16384 octs (the shared-memory form
     // beats a whole-GPU tick loop up to about there for one solve alone);
     // FP64 (the global-memory form) 2048
@@ -729,6 +760,14 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     const int grid_all = grid_ok ? resident_grid_ctas(P->fp64, ctx->device) : 0;
     const int64_t grid_auto_octs =
         P->fp64 ? INT64_MAX : (int64_t)grid_all * std::min(P->res_cap, resident_six_cap());
+    // octs per CTA up to which a smaller group is taken: FP64 kRun64; FP32 bulk
+    // with the default limits kRunLatency, with a limit given what fits the
+    // CTA (see res_max_octs)
+    const bool throughput = o.res_max_octs > 0 || o.res_cta_octs > 0;
+    // (the same groups wherever the state is kept, so that the results are the same)
+    const int64_t fit = P->res_smem ? std::max(0, resident_smem_cap(P->res_threads, ctx->device)) : 0;
+    const int64_t run = P->fp64 ? kRun64 : throughput ? fit : std::min<int64_t>(kRunLatency, fit);
+    const int64_t cta_octs = o.res_cta_octs != 0 ? o.res_cta_octs : P->fp64 ? kRun64 : throughput ? 2048 : kRunLatency;
     P->mode.assign(n, 0);
     for (int k = 0; k < n; ++k) {
       const int64_t no = P->levels[k]->n_oct;
@@ -740,7 +779,6 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       // a level whose runs on res_cluster CTAs would not fit their shared
       // memory takes the smallest larger cluster whose runs fit (the middle
       // size, else the big one); the work rule sends it to the big clusters
-      const int64_t run = P->fp64 ? kRun64 : P->res_cap;
       const auto fits = [&](int cl) { return run <= 0 || no <= cl * run; };
       if (no <= cta_octs) P->mode[k] = 2;
       else if (P->res_cluster_big > 0 && est_work(P->levels[k]) > big_work) P->mode[k] = 3;
@@ -773,7 +811,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       const int64_t c = group_ctas(P, P->mode[k]);
       if (P->mode[k] != 0 && (P->levels[k]->n_oct + c - 1) / c > resident_run_cap()) P->res_regs = false;
     }
-    double w[4] = {0.0, 0.0, 0.0, 0.0};
+    double w[4] = {0.0, 0.0, 0.0, 0.0}, longest[4] = {0.0, 0.0, 0.0, 0.0};
     for (int k = 0; k < n; ++k) {
       P->n_bq += P->mode[k] == 3;
       P->n_mq += P->mode[k] == 5;
@@ -783,7 +821,9 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       P->n_gq += P->mode[k] == 4;
       if (P->mode[k] == 0 || P->mode[k] == 4) continue;
       const int q = P->mode[k] == 3 ? 0 : P->mode[k] == 5 ? 1 : P->mode[k] == 1 ? 2 : 3;
-      w[q] += est_work(P->levels[k]);
+      const double t = est_ns(P, k) * group_ctas(P, P->mode[k]);
+      w[q] += t;
+      longest[q] = std::max(longest[q], t);
     }
     // the first split follows the estimated work; after each completed run,
     // the measured SM-time of each class (plan_adapt_split)
@@ -792,7 +832,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     P->res_clA = clA;
     P->res_clM = clM;
     P->res_clB = clB;
-    plan_split(P, w);
+    plan_split(P, w, longest);
   }
   const int bps = tick_blocks_per_sm(P->fp64, P->paper);
   P->grid = std::max(1, std::min(P->n_items, bps * ctx->num_sms));

@@ -55,10 +55,13 @@ def _solve(ats, ctx, lv, st, **kw):
     return x, stats
 
 
-@pytest.mark.parametrize("dims,kw", [((1, 1, 1), {}), ((16, 8, 8), {}), ((41, 25, 1), {}), ((16, 16, 8), {}),
-                                     ((16, 16, 16), {}), ((27, 19, 8), {}), ((16, 16, 16), dict(res_cluster=2)),
+@pytest.mark.parametrize("dims,kw", [((1, 1, 1), {}), ((16, 8, 8), {}), ((41, 25, 1), dict(res_cta_octs=2048)),
+                                     ((16, 16, 8), dict(res_cta_octs=2048)), ((41, 25, 1), {}), ((16, 16, 16), {}),
+                                     ((27, 19, 8), dict(res_max_octs=16384)), ((27, 19, 8), {}),
+                                     ((16, 16, 16), dict(res_max_octs=16384, res_cluster=2)),
                                      ((9, 9, 9), dict(res_cta_octs=-1, res_cluster=3))],
-                         ids=["1", "1024-cta", "1025-cta", "2048-cta", "1024-x4", "1026-x4", "2048-x2", "243-x3"])
+                         ids=["1", "1024-cta", "1025-cta", "2048-cta", "257-x4", "1024-x4", "1026-x4", "513-x8",
+                              "2048-x2", "243-x3"])
 def test_same_bits_as_global_state(ats, ctx, dims, kw):
     lv, st = _box(dims)
     x, stats = _solve(ats, ctx, lv, st, **kw)
