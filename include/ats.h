@@ -223,8 +223,9 @@ typedef struct {
  *   takes the tick path). */
 #define ATS_SCHED_AUTO 0     /* resident solver for levels up to res_max_octs octs; */
         /* above it the whole-GPU form (see ATS_SCHED_GRID): FP64 for every level,   */
-        /* FP32 bulk for a level of at most 1 100 octs per CTA of that form (167 200 */
-        /* octs on 152 SMs) and the tick path for larger ones                        */
+        /* FP32 bulk for a level of at most 6 144 octs per CTA of that form (933 888 */
+        /* octs on 152 SMs; 1 100 with cg_form 1 or cg_scalars 1) and the tick path  */
+        /* for larger ones                                                           */
 #define ATS_SCHED_TICK 1     /* the tick path for every level                    */
 #define ATS_SCHED_RESIDENT 2 /* the resident solver for every level              */
 #define ATS_SCHED_GRID 3     /* as AUTO, and every level above res_max_octs on the   */

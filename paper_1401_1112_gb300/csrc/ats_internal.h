@@ -205,7 +205,8 @@ struct ResArgs {
   int cg_scalars;  // FP32 bulk: 0 = step decisions in FP32 from the rounded totals, 1 = in FP64
   int q_recur;     // FP32 bulk: 1 = q = (I + dt A) z + beta q_prev (no barrier), 0 = q = (I + dt A) p
   int regs;        // FP32 bulk, 512 threads: 1 = the CG state in registers and shared memory
-                   // (q_recur = 1, cg_scalars = 0, every run at most resident_run_cap() octs)
+                   // (q_recur = 1, cg_scalars = 0, every run at most resident_run_cap() octs);
+                   // 2 (whole-GPU form): longer runs, the rest of each in global memory
   int *cq_head;
   int *tq_head;
   unsigned long long *cells;

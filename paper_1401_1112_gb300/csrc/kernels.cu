@@ -3089,6 +3089,65 @@ __device__ __forceinline__ void res3_dir(const SolveDev &sd, uint32_t base, int 
   }
 }
 
+// The in-oct faces' part of -sum C v_j: x inside a pair, y and z between pairs.
+__device__ __forceinline__ void res3_in_oct(const f32x2 (&nk)[4], const f32x2 (&v)[4], f32x2 (&w)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float k0, k1, v0, v1;
+    unpack2(nk[k], k0, k1);
+    unpack2(v[k], v0, v1);
+    const float C = __fadd_rn(k0, k1);
+    w[k] = pack2(__fmul_rn(C, v1), __fmul_rn(C, v0));
+  }
+#pragma unroll
+  for (int b = 1; b <= 2; b <<= 1) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k & b) continue;
+      const f32x2 C = add2(nk[k], nk[k | b]);
+      w[k] = fma2(C, v[k | b], w[k]);
+      w[k | b] = fma2(C, v[k], w[k | b]);
+    }
+  }
+}
+
+// The end of step 1+2: w += D v, p = v + beta p, q = w + beta q; returns p.q.
+__device__ __forceinline__ float res3_op_end(const f32x2 (&nk)[4], const f32x2 (&v)[4], const f32x2 (&w)[4],
+                                             const f32x2 (&d)[4], f32x2 beta, bool all_leaf, f32x2 (&p)[4],
+                                             f32x2 (&q)[4]) {
+  f32x2 dot = 0ull;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    p[k] = fma2(beta, p[k], v[k]);
+    q[k] = fma2(beta, q[k], fma2(d[k], v[k], w[k]));
+    if (!all_leaf) {  // q = 0 off the leaves
+      float k0, k1, q0, q1;
+      unpack2(nk[k], k0, k1);
+      unpack2(q[k], q0, q1);
+      q[k] = pack2(k0 <= 0.f ? q0 : 0.f, k1 <= 0.f ? q1 : 0.f);
+    }
+    dot = fma2(p[k], q[k], dot);
+  }
+  return sum2(dot);
+}
+
+// Step 3's cells: z (in place) from r = D z - alpha q, and the sums.
+__device__ __forceinline__ void res3_upd_cells(const f32x2 (&d)[4], const f32x2 (&q)[4], f32x2 (&z)[4], f32x2 nalpha,
+                                               float &lrz, float &lrr) {
+  f32x2 srz = 0ull, srr = 0ull;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const f32x2 r = fma2(nalpha, q[k], mul2(d[k], z[k]));
+    float d0, d1;
+    unpack2(d[k], d0, d1);
+    z[k] = mul2(r, pack2(rcp_approx(d0), rcp_approx(d1)));
+    srz = fma2(r, z[k], srz);
+    srr = fma2(r, r, srr);
+  }
+  lrz = sum2(srz);
+  lrr = sum2(srr);
+}
+
 // Step 1+2 on own oct o (local index l): w = D z - sum C z_j, p = z + beta p,
 // q = w + beta q; returns the oct's p.q.
 template <int kG, int R>
@@ -3105,29 +3164,8 @@ __device__ __forceinline__ float res3_op(const SolveDev &sd, uint32_t base, int 
   for (int k = 0; k < 4; ++k) {
     nk[k] = lds64<false>(row + L::kToK + k * L::S);
     v[k] = lds64<false>(row + k * L::S);
-    w[k] = 0ull;
   }
-  // in-oct faces: x inside a pair, y and z between pairs
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float k0, k1, v0, v1, w0, w1;
-    unpack2(nk[k], k0, k1);
-    unpack2(v[k], v0, v1);
-    const float C = __fadd_rn(k0, k1);
-    w0 = __fmul_rn(C, v1);
-    w1 = __fmul_rn(C, v0);
-    w[k] = pack2(w0, w1);
-  }
-#pragma unroll
-  for (int b = 1; b <= 2; b <<= 1) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (k & b) continue;
-      const f32x2 C = add2(nk[k], nk[k | b]);
-      w[k] = fma2(C, v[k | b], w[k]);
-      w[k | b] = fma2(C, v[k], w[k | b]);
-    }
-  }
+  res3_in_oct(nk, v, w);
   constexpr int dw = R == 2 ? 1 : 2;
   res3_dir<kG, R, 0>(sd, base, o, code[0 / dw], h, nk, w);
   res3_dir<kG, R, 1>(sd, base, o, code[1 / dw], h, nk, w);
@@ -3135,21 +3173,10 @@ __device__ __forceinline__ float res3_op(const SolveDev &sd, uint32_t base, int 
   res3_dir<kG, R, 3>(sd, base, o, code[3 / dw], h, nk, w);
   res3_dir<kG, R, 4>(sd, base, o, code[4 / dw], h, nk, w);
   res3_dir<kG, R, 5>(sd, base, o, code[5 / dw], h, nk, w);
-  f32x2 dot = 0ull;
+  f32x2 d[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const f32x2 d = R == 2 ? D[k] : lds64<false>(row + L::oD + k * L::S);
-    p[k] = fma2(beta, p[k], v[k]);
-    q[k] = fma2(beta, q[k], fma2(d, v[k], w[k]));
-    if (!all_leaf) {  // q = 0 off the leaves
-      float k0, k1, q0, q1;
-      unpack2(nk[k], k0, k1);
-      unpack2(q[k], q0, q1);
-      q[k] = pack2(k0 <= 0.f ? q0 : 0.f, k1 <= 0.f ? q1 : 0.f);
-    }
-    dot = fma2(p[k], q[k], dot);
-  }
-  return sum2(dot);
+  for (int k = 0; k < 4; ++k) d[k] = R == 2 ? D[k] : lds64<false>(row + L::oD + k * L::S);
+  return res3_op_end(nk, v, w, d, beta, all_leaf, p, q);
 }
 
 // Step 3 on own oct o: r = D z - alpha q, z = r x rcp(D), the sums.
@@ -3158,24 +3185,19 @@ __device__ __forceinline__ void res3_upd(const SolveDev &sd, uint32_t base, int 
                                          const f32x2 (&D)[4], const f32x2 (&q)[4], float &lrz, float &lrr) {
   using L = Res3<R>;
   const uint32_t row = base + (uint32_t)l * 8u;
-  f32x2 srz = 0ull, srr = 0ull, zn[4];
+  f32x2 d[4], z[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const f32x2 d = R == 2 ? D[k] : lds64<false>(row + L::oD + k * L::S);
-    const f32x2 r = fma2(nalpha, q[k], mul2(d, lds64<false>(row + k * L::S)));
-    float d0, d1;
-    unpack2(d, d0, d1);
-    zn[k] = mul2(r, pack2(rcp_approx(d0), rcp_approx(d1)));
-    srz = fma2(r, zn[k], srz);
-    srr = fma2(r, r, srr);
-    sts64(row + k * L::S, zn[k]);
+    d[k] = R == 2 ? D[k] : lds64<false>(row + L::oD + k * L::S);
+    z[k] = lds64<false>(row + k * L::S);
   }
+  res3_upd_cells(d, q, z, nalpha, lrz, lrr);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) sts64(row + k * L::S, z[k]);
   if (kG == 2)
-    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"((float *)sd.z + 8 * (size_t)o), "l"(zn[0]),
-                 "l"(zn[1]), "l"(zn[2]), "l"(zn[3])
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"((float *)sd.z + 8 * (size_t)o), "l"(z[0]), "l"(z[1]),
+                 "l"(z[2]), "l"(z[3])
                  : "memory");
-  lrz = sum2(srz);
-  lrr = sum2(srr);
 }
 
 // Step 3's e += alpha p on own oct o, which nothing else waits for: done
@@ -3198,10 +3220,74 @@ __device__ __forceinline__ void res3_e(const SolveDev &sd, int o, f32x2 alpha, c
   }
 }
 
+// ---- octs beyond a CTA's on-chip capacity (a whole-GPU group) ----
+// Oct l >= cap of a run keeps everything in the level's global arrays (L2, or
+// HBM for the largest levels), with the same arithmetic.  Bound: L2 (about 790
+// bytes per such oct and iteration, 320 of them neighbour rows, from 16 warps
+// per SM).  Step 3 goes through them backwards, from the rows that step 1+2
+// touched last to those the next step begins with, so that what L2 holds of a
+// level larger than itself is used before it is replaced.
+// Measured (stiff mixed level, us per iteration, tick path -> here): 262 144
+// octs 32.8 -> 20.2, 309 808 35.1 -> 20.6 (both on chip), 511 920 57.6 -> 33.5,
+// 1 000 000 124 -> 118; 2 097 152 245 -> 271, so the line lies at 6 144 octs
+// per CTA (kRunTail where a plan picks the path).
+__device__ __forceinline__ void ldg_row(const float *p, f32x2 (&v)[4]) {
+  asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+}
+__device__ __forceinline__ void stg_row(float *p, const f32x2 (&v)[4]) {
+  asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(v[0]), "l"(v[1]), "l"(v[2]), "l"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ float res3_tail_op(const SolveDev &sd, int o, float h, f32x2 beta, bool first,
+                                              bool all_leaf) {
+  int g[6];
+  load_nbr6(sd.nbr, o, g);
+  check_nbr6(g, sd.n_oct);
+  const size_t at = 8 * (size_t)o;
+  float K[8];
+  ld8_ro((const float *)sd.KT + at, K);
+  f32x2 v[4], w[4], nk[4];
+  asm volatile("ld.global.cg.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
+               : "l"((const float *)sd.z + at));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) nk[k] = pack2(-__fmul_rn(K[2 * k], h), -__fmul_rn(K[2 * k + 1], h));
+  res3_in_oct(nk, v, w);
+  if (g[0] >= 0) res3_face_far<0>(sd, g[0], h, nk, w);
+  if (g[1] >= 0) res3_face_far<1>(sd, g[1], h, nk, w);
+  if (g[2] >= 0) res3_face_far<2>(sd, g[2], h, nk, w);
+  if (g[3] >= 0) res3_face_far<3>(sd, g[3], h, nk, w);
+  if (g[4] >= 0) res3_face_far<4>(sd, g[4], h, nk, w);
+  if (g[5] >= 0) res3_face_far<5>(sd, g[5], h, nk, w);
+  f32x2 D[4], p[4], q[4];
+  ldg_row((const float *)sd.dg + at, D);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) p[k] = q[k] = 0ull;
+  if (!first) {
+    ldg_row((const float *)sd.p0 + at, p);
+    ldg_row((const float *)sd.q + at, q);
+  }
+  const float pq = res3_op_end(nk, v, w, D, beta, all_leaf, p, q);
+  stg_row((float *)sd.p0 + at, p);
+  stg_row((float *)sd.q + at, q);
+  return pq;
+}
+__device__ __forceinline__ void res3_tail_upd(const SolveDev &sd, int o, f32x2 nalpha, float &lrz, float &lrr) {
+  const size_t at = 8 * (size_t)o;
+  f32x2 D[4], q[4], z[4];
+  ldg_row((const float *)sd.dg + at, D);
+  ldg_row((const float *)sd.q + at, q);
+  asm volatile("ld.global.cg.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(z[0]), "=l"(z[1]), "=l"(z[2]), "=l"(z[3])
+               : "l"((const float *)sd.z + at));
+  res3_upd_cells(D, q, z, nalpha, lrz, lrr);
+  stg_row((float *)sd.z + at, z);
+}
+
 // One solve by one group (see res2_solve_l, whose state machine and decisions
 // these are).  Every thread takes the step decisions itself from the group's
 // totals, so no barrier follows them; thread 0 keeps the counters.
-template <int kG, int R>
+template <int kG, int R, bool kTail>
 __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
   using L = Res3<R>;
   constexpr int wd = (int)(sizeof(SolveDev) / 8);
@@ -3257,6 +3343,7 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
         const int gr = g[d] / chunk;
         far = kG == 2 && (unsigned)gr != cr;
         at = g[d] - gr * chunk;
+        far = far || (kTail && at >= L::cap);
         if (kG == 1) rank = (unsigned)gr;
       }
       if (R == 2) {
@@ -3273,6 +3360,14 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
       asm volatile("st.shared.u32 [%0], %1;" ::"r"(base + L::oC + (uint32_t)(d * L::cap + l) * 4u), "r"(v) : "memory");
     }
   }
+  if (kTail) {
+    for (int l = (int)threadIdx.x + L::cap; l < run; l += 512) {
+      float K[8];
+      ld8_ro((const float *)sd.KT + 8 * (size_t)(lo + l), K);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) leafs = leafs && K[c] >= 0.f;
+    }
+  }
   const bool all_leaf = __syncthreads_and(leafs);
   const bool want_x = sd.stop_rule == ATS_STOP_CERTIFIED;
   bool alive = true;
@@ -3284,10 +3379,14 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
       for (int l = (int)threadIdx.x; l < run; l += 512) {
         float zo[8], dv[8];
         ref_oct_values<float, true, true>(sd, lo + l, want_x, acc[0], acc[1], acc[2], zo, dv);
+        if (kTail && l >= L::cap) {
+          st8((float *)sd.dg + 8 * (size_t)(lo + l), dv);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          sts64(base + (uint32_t)l * 8u + k * L::S, pack2(zo[2 * k], zo[2 * k + 1]));
-          sts64(base + (uint32_t)l * 8u + L::oD + k * L::S, pack2(dv[2 * k], dv[2 * k + 1]));
+          for (int k = 0; k < 4; ++k) {
+            sts64(base + (uint32_t)l * 8u + k * L::S, pack2(zo[2 * k], zo[2 * k + 1]));
+            sts64(base + (uint32_t)l * 8u + L::oD + k * L::S, pack2(dv[2 * k], dv[2 * k + 1]));
+          }
         }
         if (kG == 2) st8((float *)sd.z + 8 * (size_t)(lo + l), zo);
       }
@@ -3324,6 +3423,11 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
           const int l = (int)threadIdx.x + 512 * r;
           if (l < run) acc[0].add_value(res3_op<kG, R>(sd, base, lo + l, l, h, b2, all_leaf, D[r], p[r], q[r]));
         }
+        if (kTail) {
+#pragma unroll 1
+          for (int l = (int)threadIdx.x + L::cap; l < run; l += 512)
+            acc[0].add_value(res3_tail_op(sd, lo + l, h, b2, it == 0, all_leaf));
+        }
         alive = res2_sum<1, kG>(acc, sh, a, buf, tot);
         const float pq = tot[0].val();
         brk = !(rz >= 0.f) || !isfinite(rz) || !(pq > 0.f) || !isfinite(pq);
@@ -3342,11 +3446,29 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
           acc[0].add_value(lrz);
           acc[1].add_value(lrr);
         }
+        if (kTail && run > L::cap) {
+#pragma unroll 1
+          for (int l = (int)threadIdx.x + (run - 1) / 512 * 512; l >= L::cap; l -= 512) {
+            if (l >= run) continue;
+            float lrz, lrr;
+            res3_tail_upd(sd, lo + l, n2, lrz, lrr);
+            acc[0].add_value(lrz);
+            acc[1].add_value(lrr);
+          }
+        }
         alive = res2_sum<2, kG>(acc, sh, a, buf, tot, [&] {
 #pragma unroll
           for (int r = 0; r < R; ++r) {
             const int l = (int)threadIdx.x + 512 * r;
             if (l < run) res3_e<R>(sd, lo + l, a2, p[r], e[r]);
+          }
+          if (kTail) {
+#pragma unroll 1
+            for (int l = (int)threadIdx.x + L::cap; l < run; l += 512) {
+              f32x2 pv[4], none[4];
+              ldg_row((const float *)sd.p0 + 8 * (size_t)(lo + l), pv);
+              res3_e<4>(sd, lo + l, a2, pv, none);
+            }
           }
         });
         if (!alive) break;
@@ -3377,6 +3499,10 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
         }
         st8(x, xv);
       }
+    }
+    if (kTail && !brk && alive) {
+#pragma unroll 1
+      for (int l = (int)threadIdx.x + L::cap; l < run; l += 512) res_xpe_oct<float>(sd, lo + l);
     }
     if (threadIdx.x == 0) {
       ResState &st = sh.st;
@@ -3417,7 +3543,14 @@ template <int kG>
 __device__ bool res3_solve(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
   const unsigned cs = kG == 2 ? gridDim.x : (kG == 1 ? cl_size() : 1u);
   const int chunk = (int)((a.solves[s].n_oct + (int)cs - 1) / (int)cs);
-  return chunk <= Res3<2>::cap ? res3_solve_r<kG, 2>(a, s, sh, buf) : res3_solve_r<kG, 4>(a, s, sh, buf);
+  if (chunk <= Res3<2>::cap) return res3_solve_r<kG, 2, false>(a, s, sh, buf);
+  return res3_solve_r<kG, 4, false>(a, s, sh, buf);
+}
+template <int kG>
+__device__ bool res3_solve_tail(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
+  const int chunk = (int)((a.solves[s].n_oct + (int)gridDim.x - 1) / (int)gridDim.x);
+  if (chunk <= Res3<2>::cap) return res3_solve_r<kG, 2, false>(a, s, sh, buf);
+  return res3_solve_r<kG, 4, true>(a, s, sh, buf);
 }
 
 }  // namespace
@@ -3425,11 +3558,13 @@ __device__ bool res3_solve(const ResArgs &a, int s, ResShared<float> &sh, int &b
 namespace {
 
 // Where a kernel instance keeps a solve's CG state: shared memory planes, the
-// level's global arrays, or registers and shared memory.
-constexpr int kStateShared = 0, kStateGlobal = 1, kStateRegs = 2;
+// level's global arrays, registers and shared memory, or (whole GPU) those for
+// the first 2 048 octs of each CTA's run and the global arrays for the rest.
+constexpr int kStateShared = 0, kStateGlobal = 1, kStateRegs = 2, kStateTail = 3;
 template <int kG, int kState>
 __device__ __forceinline__ bool resf_solve(const ResArgs &a, int s, ResShared<float> &sh, int &buf) {
   if constexpr (kState == kStateRegs) return res3_solve<kG>(a, s, sh, buf);
+  else if constexpr (kState == kStateTail) return res3_solve_tail<kG>(a, s, sh, buf);
   else return res2_solve<kG, kState == kStateGlobal>(a, s, sh, buf);
 }
 
@@ -3950,7 +4085,7 @@ template <int NT>
 static cudaError_t res2_launch_t(int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only,
                                  int priority) {
   if (a.cap == 0) return res2_launch_k<NT, kStateGlobal>(cluster, grid, a, st, cta_only, priority);
-  if (NT == 512 && a.regs) return res2_launch_k<512, kStateRegs>(cluster, grid, a, st, cta_only, priority);
+  if (NT == 512 && a.regs == 1) return res2_launch_k<512, kStateRegs>(cluster, grid, a, st, cta_only, priority);
   return res2_launch_k<NT, kStateShared>(cluster, grid, a, st, cta_only, priority);
 }
 
@@ -4020,15 +4155,16 @@ int resident_smem_cap(int threads, int device) {
 // The whole-GPU form of a bulk precision: its kernel and dynamic shared memory.
 using ResGridKernel = void (*)(ResArgs);
 template <int NT>
-static ResGridKernel res_grid_kernel(bool fp64, bool regs, size_t *smem) {
+static ResGridKernel res_grid_kernel(bool fp64, int regs, size_t *smem) {
   *smem = fp64 ? 0 : kRes2SmemBytes;
-  return fp64 ? k_resd_grid<NT> : regs ? k_res2_grid<NT, kStateRegs> : k_res2_grid<NT, kStateShared>;
+  if (fp64) return k_resd_grid<NT>;
+  return regs == 2 ? k_res2_grid<NT, kStateTail> : regs == 1 ? k_res2_grid<NT, kStateRegs> : k_res2_grid<NT, kStateShared>;
 }
 
 template <int NT>
 static cudaError_t res2_grid_launch_t(bool fp64, int grid, const ResArgs &a, cudaStream_t st) {
   size_t smem = 0;
-  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, a.regs != 0, &smem);
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, a.regs, &smem);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -4048,7 +4184,7 @@ template <int NT>
 static int res2_grid_ctas_t(bool fp64, int device) {
   int b = 0, sms = 0;
   size_t smem = 0;
-  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, false, &smem);
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, 0, &smem);
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, NT, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {

@@ -276,6 +276,7 @@ struct Plan {
   bool res_smem = false;  // K, z, p of each CTA's octs in shared memory (FP32 bulk)
   int res_cap = 0;        // octs per CTA kept in shared memory
   bool res_regs = false;  // the CG state in registers and shared memory (FP32 bulk)
+  int res_regs_grid = 0;  // ... in the whole-GPU form (2: with octs beyond the on-chip capacity)
   int res_fill = 0;       // single CTAs launched beside the clusters on the SMs they leave
   int32_t *d_queue = nullptr;   // [n_bq + n_mq + n_cq + n_tq + n_gq]
   int *d_heads = nullptr;       // [4] next position of each queue: big, cluster, CTA, middle
@@ -615,6 +616,11 @@ constexpr int64_t kRun64 = 128;
 // 512 levels of 64 .. 32 768 octs take 13.9 ms with runs of up to 2 048 and
 // 16.4 ms with the shorter ones (measured).
 constexpr int64_t kRunLatency = 1024;
+// FP32-bulk levels take the whole-GPU form up to this many octs per CTA: the
+// first 2 048 of a run stay on chip, the rest is streamed from L2 and HBM,
+// where the tick path's larger grid does better once HBM bounds it (measured
+// at 1 000 000 octs: 25.7 against 27.2 ms, at 2 097 152: 59.1 against 53.1).
+constexpr int64_t kRunTail = 6144;
 
 ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const ats_solve_opts *opts_in,
                        Plan **out) {
@@ -752,14 +758,15 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
                          : resident_max_clusters(P->res_threads, cl);
     };
     // levels above the limit: the whole-GPU form when asked for, and with
-    // ATS_SCHED_AUTO in FP64 for every level, in FP32 bulk (each CTA's run in
-    // shared memory) when the runs on its CTAs keep all six arrays in shared
-    // memory; else the tick path
+    // ATS_SCHED_AUTO in FP64 for every level, in FP32 bulk for runs of at most
+    // kRunTail octs (with the options that need the shared-memory form: when
+    // the runs keep all six arrays there); else the tick path
     const bool grid_ok = (o.sched == ATS_SCHED_GRID || o.sched == ATS_SCHED_AUTO) &&
                          (P->fp64 || (P->res_cap > 0 && P->res_threads == 512));
     const int grid_all = grid_ok ? resident_grid_ctas(P->fp64, ctx->device) : 0;
+    const bool grid_regs = o.cg_form != 1 && !o.cg_scalars;
     const int64_t grid_auto_octs =
-        P->fp64 ? INT64_MAX : (int64_t)grid_all * std::min(P->res_cap, resident_six_cap());
+        P->fp64 ? INT64_MAX : grid_all * (grid_regs ? kRunTail : std::min(P->res_cap, resident_six_cap()));
     // octs per CTA up to which a smaller group is taken: FP64 kRun64; FP32 bulk
     // with the default limits kRunLatency, with a limit given what fits the
     // CTA (see res_max_octs)
@@ -807,9 +814,12 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     // other forms give the same bits
     if (grid_all > 0) P->res_grid_all = grid_all;
     P->res_regs = P->res_smem && P->res_cap > 0 && P->res_threads == 512 && o.cg_form != 1 && !o.cg_scalars;
+    P->res_regs_grid = P->res_regs ? 1 : 0;
     for (int k = 0; k < n; ++k) {
       const int64_t c = group_ctas(P, P->mode[k]);
-      if (P->mode[k] != 0 && (P->levels[k]->n_oct + c - 1) / c > resident_run_cap()) P->res_regs = false;
+      if (P->mode[k] == 0 || (P->levels[k]->n_oct + c - 1) / c <= resident_run_cap()) continue;
+      if (P->mode[k] == 4) P->res_regs_grid = P->res_regs_grid ? 2 : 0;
+      else P->res_regs = false;
     }
     double w[4] = {0.0, 0.0, 0.0, 0.0}, longest[4] = {0.0, 0.0, 0.0, 0.0};
     for (int k = 0; k < n; ++k) {
@@ -1033,6 +1043,7 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
     a.gbar = P->d_gbar;
     a.gpart = P->d_gpart;
     a.gerr = P->d_gerr;
+    a.regs = P->res_regs_grid;
     CUDA_TRY(cudaMemsetAsync(P->d_gbar, 0, 2 * sizeof(unsigned), st));
     CUDA_TRY(cudaMemsetAsync(P->d_gerr, 0, sizeof(int), st));
     CUDA_TRY(launch_resident_grid(P->fp64, P->res_grid_all, a, st));

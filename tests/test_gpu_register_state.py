@@ -80,10 +80,27 @@ def test_same_bits_with_non_leaf_cells(ats, ctx, seed, kw):
     assert stats == sg
 
 
-@pytest.mark.parametrize("dims", [(54, 54, 53), (58, 58, 50)], ids=["run-1017", "run-1107"])
+@pytest.mark.parametrize("dims", [(54, 54, 53), (58, 58, 50), (68, 68, 67), (68, 68, 68)],
+                         ids=["run-1017", "run-1107", "run-2039", "run-2069"])
 def test_whole_gpu_layout_edge(ats, ctx, dims):
-    """154 548 and 168 200 octs over 152 CTAs: the two register layouts."""
+    """154 548 and 168 200 octs over 152 CTAs: the two register layouts; 309 808 and 314 432: just within and just
+    beyond what a CTA keeps on chip."""
     lv, st = _box(dims)
     x, _ = _solve(ats, ctx, lv, st, sched=ats.ATS_SCHED_GRID)
     xt, _ = _solve(ats, ctx, lv, st, sched=ats.ATS_SCHED_TICK)
     assert np.linalg.norm(x - xt) <= 1e-10 * np.linalg.norm(xt)
+
+
+def test_whole_gpu_tail_with_non_leaf_cells(ats, ctx):
+    """A level beyond the on-chip capacity whose every 1 000th oct has refined cells: the octs in global memory keep
+    them out of the stencil as the others do."""
+    lv, st = _box((80, 70, 60))
+    leaf = np.full(lv.n_oct, 0xFF, np.uint8)
+    inner = np.all((lv.oct_xyz > 0) & (lv.oct_xyz < np.array([79, 69, 59])), axis=1)
+    leaf[np.nonzero(inner)[0][::1000]] = 0x5A
+    lv.leaf = leaf
+    x, _ = _solve(ats, ctx, lv, st)
+    xt, _ = _solve(ats, ctx, lv, st, sched=ats.ATS_SCHED_TICK)
+    assert np.linalg.norm(x - xt) <= 1e-10 * np.linalg.norm(xt)
+    nl = ~lv.leaf_cells()
+    np.testing.assert_array_equal(x[nl], st.E[nl])
