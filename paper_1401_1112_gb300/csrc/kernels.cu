@@ -3711,190 +3711,201 @@ __global__ void __launch_bounds__(NT, 1) k_res2_grid(ResArgs a) {
 // (kRun64 where a plan picks them), and levels above the clusters take the
 // whole-GPU form.  z is the only array other threads read (ld.global.cg after
 // the step's barrier); p, q, r, e and 1 / D belong to the thread that owns the
-// oct.  Non-leaf cells: C = 0 on all their faces, and r = z = p = q = 0.
+// cell pair.  Non-leaf cells: C = 0 on all their faces, and r = z = p = q = 0.
 // Measured, certified 5e-11, build included: 128 levels of 64..2 048 octs
-// 28.6 -> 3.1 ms (one CTA of 256 threads each before), 4 096 octs 4.51 -> 1.23
-// ms and 32 736 octs 6.49 -> 2.01 ms (tick path before).
+// 27.2 -> 2.67 ms (one CTA of 256 threads each before), 4 096 octs 4.52 -> 0.90
+// ms and 32 736 octs 6.53 -> 2.03 ms (tick path before).
 
 namespace {
 
-template <int A>
-__device__ __forceinline__ void resd_axis(const SolveDev &sd, int o, const int (&nb)[6], const double *z,
-                                          const double (&v)[8], double (&w)[8]) {
-  constexpr int bit = 1 << A;
-  double Cu[8];
-  ld8_ro(sd.C64 + (3 * (size_t)o + A) * 8, Cu);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    if (c & bit) continue;
-    const int d = c | bit;
-    w[c] = fma(-Cu[c], v[d], w[c]);
-    w[d] = fma(-Cu[c], v[c], w[d]);
-  }
-  int n = nb[2 * A + 1];  // +A face: C from row A of this oct
-  if (n >= 0) {
-    double Zn[8];
-    ldc_face<A, 0>(z + 8 * (size_t)n, Zn);
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-      if (c & bit) w[c] = fma(-Cu[c], Zn[c ^ bit], w[c]);
-  }
-  n = nb[2 * A];  // -A face: C from row A of the -A neighbour
-  if (n >= 0) {
-    double Zn[8], Cn[8];
-    ldc_face<A, 1>(z + 8 * (size_t)n, Zn);
-    ld_face<A, 1>(sd.C64 + (3 * (size_t)n + A) * 8, Cn);
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-      if (!(c & bit)) w[c] = fma(-Cn[c | bit], Zn[c | bit], w[c]);
-  }
+// The work unit of a thread is a pair of cells (2k, 2k + 1) of an oct, unit
+// u = 4 o + k: a run of 32 octs then fills the four quarters of the SM's FP64
+// pipe (one quarter holds a warp for 75 cycles per instruction), where one oct
+// per thread left three of them idle up to 96 octs, and a thread's loads are
+// whole 16-byte pairs, contiguous over the warp.  Against one oct per thread,
+// us per CG iteration: 64 octs on one CTA 7.8 -> 5.9, 4 096 octs on the whole
+// GPU 12.9 -> 9.7, 32 768 octs (the pipe full either way) 15.3 -> 16.4.
+struct Pair64 {
+  double a, b;
+};
+__device__ __forceinline__ Pair64 ldp_ro(const double *p) {
+  const double2 v = __ldg(reinterpret_cast<const double2 *>(p));
+  return {v.x, v.y};
+}
+__device__ __forceinline__ Pair64 ldp_cg(const double *p) {  // written by other threads of the launch
+  Pair64 v;
+  asm volatile("ld.global" ATS_RES_LD ".v2.f64 {%0, %1}, [%2];" : "=d"(v.a), "=d"(v.b) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld1_cg(const double *p) {
+  double v;
+  asm volatile("ld.global" ATS_RES_LD ".f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ Pair64 ldp_rw(const void *base, int u) {  // this thread's own
+  Pair64 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.a), "=d"(v.b) : "l"((const double *)base + 2 * (size_t)u));
+  return v;
+}
+__device__ __forceinline__ void stp(void *base, int u, Pair64 v) {
+  asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"((double *)base + 2 * (size_t)u), "d"(v.a), "d"(v.b)
+               : "memory");
 }
 
-// Step 1 on oct o; returns the oct's p.q in the accumulator.
-__device__ __forceinline__ void resd_op_oct(const SolveDev &sd, int o, bool first, double beta, Acc<double> &pq) {
-  int nb[6];
-  load_nbr6(sd.nbr, o, nb);
-  check_nbr6(nb, sd.n_oct);
+// The neighbours of unit u and the coefficients towards them.  Upwards (+y,
+// +z) the coefficient is in the unit's own row (0 where there is no
+// neighbour), downwards in the row of the pair below.  Across y the partner
+// is pair k ^ 1, across z pair k ^ 2, of this oct or of the neighbour oct.
+struct Stencil64 {
+  Pair64 cx;                    // the face inside the pair, the +x face
+  double cxm;                   // the -x face
+  size_t xp, xm;                // cells across +x, -x
+  Pair64 cup[2], cdn[2];        // y, z
+  size_t up[2], dn[2];          // first cells of the pairs above, below
+};
+__device__ __forceinline__ Stencil64 resd_stencil(const SolveDev &sd, int u) {
+  const int o = u >> 2, k = u & 3;
+  Stencil64 s;
+  const int32_t *nbr = sd.nbr + 6 * (size_t)o;
+  const auto oct = [&](int d) {
+    const int g = __ldg(nbr + d);
+    return g >= 0 && idx_ok(g, sd.n_oct) ? g : -1;
+  };
+  const size_t c0 = 8 * (size_t)o + 2 * k;
+  const int xp = oct(1), xm = oct(0);
+  s.cx = ldp_ro(sd.C64 + 24 * (size_t)o + 2 * k);
+  s.xp = (xp >= 0 ? 8 * (size_t)xp + 2 * k : c0);
+  s.xm = (xm >= 0 ? 8 * (size_t)xm + 2 * k : c0) + 1;
+  s.cxm = xm >= 0 ? __ldg(sd.C64 + 24 * (size_t)xm + 2 * k + 1) : 0.0;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {  // y, z
+    const int bit = 1 << a, side = (k >> a) & 1, kp = k ^ bit;
+    const int n = oct(2 + 2 * a + side);  // the neighbour on the unit's outer side
+    const int ou = side ? n : o, od = side ? o : n;
+    s.cup[a] = ldp_ro(sd.C64 + 24 * (size_t)o + 8 * (a + 1) + 2 * k);
+    s.up[a] = ou >= 0 ? 8 * (size_t)ou + 2 * kp : c0;
+    s.dn[a] = od >= 0 ? 8 * (size_t)od + 2 * kp : c0;
+    s.cdn[a] = od >= 0 ? ldp_ro(sd.C64 + 24 * (size_t)od + 8 * (a + 1) + 2 * kp) : Pair64{0.0, 0.0};
+  }
+  return s;
+}
+
+// Step 1 on unit u; adds its p.q.
+__device__ __forceinline__ void resd_op(const SolveDev &sd, int u, bool first, double beta, Acc<double> &pq) {
   const double *z = (const double *)sd.z;
-  double *p = (double *)sd.p0, *q = (double *)sd.q;
-  double v[8], w[8];
-  ldc8(z + 8 * (size_t)o, v);
-  ld8_rw((const double *)sd.p1 + 8 * (size_t)o, w);  // r
-  resd_axis<0>(sd, o, nb, z, v, w);
-  resd_axis<1>(sd, o, nb, z, v, w);
-  resd_axis<2>(sd, o, nb, z, v, w);
-  if (!first) {
-    double t[8];
-    ld8_rw(p + 8 * (size_t)o, t);
+  const Stencil64 s = resd_stencil(sd, u);
+  const Pair64 v = ldp_cg(z + 2 * (size_t)u);
+  Pair64 w = ldp_rw(sd.p1, u);  // r
+  const double zp = ld1_cg(z + s.xp), zm = ld1_cg(z + s.xm);
+  Pair64 zu[2], zd[2];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = fma(beta, t[c], v[c]);
-    ld8_rw(q + 8 * (size_t)o, t);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) w[c] = fma(beta, t[c], w[c]);
+  for (int a = 0; a < 2; ++a) {
+    zu[a] = ldp_cg(z + s.up[a]);
+    zd[a] = ldp_cg(z + s.dn[a]);
   }
-  st8(p + 8 * (size_t)o, v);
-  st8(q + 8 * (size_t)o, w);
+  Pair64 p = {0.0, 0.0}, q = {0.0, 0.0};
+  if (!first) {
+    p = ldp_rw(sd.p0, u);
+    q = ldp_rw(sd.q, u);
+  }
+  w.a = fma(-s.cx.a, v.b, w.a);
+  w.b = fma(-s.cx.a, v.a, w.b);
+  w.b = fma(-s.cx.b, zp, w.b);
+  w.a = fma(-s.cxm, zm, w.a);
 #pragma unroll
-  for (int c = 0; c < 8; ++c) pq.add(v[c], w[c]);
+  for (int a = 0; a < 2; ++a) {
+    w.a = fma(-s.cup[a].a, zu[a].a, w.a);
+    w.b = fma(-s.cup[a].b, zu[a].b, w.b);
+    w.a = fma(-s.cdn[a].a, zd[a].a, w.a);
+    w.b = fma(-s.cdn[a].b, zd[a].b, w.b);
+  }
+  p.a = fma(beta, p.a, v.a);
+  p.b = fma(beta, p.b, v.b);
+  q.a = fma(beta, q.a, w.a);
+  q.b = fma(beta, q.b, w.b);
+  stp(sd.p0, u, p);
+  stp(sd.q, u, q);
+  pq.add(p.a, q.a);
+  pq.add(p.b, q.b);
 }
 
-// Step 2 on oct o.
-__device__ __forceinline__ void resd_upd_oct(const SolveDev &sd, int o, double alpha, Acc<double> &rz,
-                                             Acc<double> &rr) {
-  double a[8], b[8];
-  double *r = (double *)sd.p1 + 8 * (size_t)o, *e = (double *)sd.e + 8 * (size_t)o;
-  ld8_rw(r, a);
-  ld8_rw((const double *)sd.q + 8 * (size_t)o, b);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) a[c] = fma(-alpha, b[c], a[c]);
-  st8(r, a);
-  ld8_rw((const double *)sd.dg + 8 * (size_t)o, b);  // 1 / D
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    b[c] *= a[c];
-    rr.add(a[c], a[c]);
-    rz.add(a[c], b[c]);
-  }
-  st8((double *)sd.z + 8 * (size_t)o, b);
-  ld8_rw((const double *)sd.p0 + 8 * (size_t)o, b);
-  ld8_rw(e, a);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) a[c] = fma(alpha, b[c], a[c]);
-  st8(e, a);
+// Step 2 on unit u.
+__device__ __forceinline__ void resd_upd(const SolveDev &sd, int u, double alpha, Acc<double> &rz, Acc<double> &rr) {
+  const Pair64 q = ldp_rw(sd.q, u), inv = ldp_rw(sd.dg, u), p = ldp_rw(sd.p0, u);
+  Pair64 r = ldp_rw(sd.p1, u), e = ldp_rw(sd.e, u), z;
+  r.a = fma(-alpha, q.a, r.a);
+  r.b = fma(-alpha, q.b, r.b);
+  z.a = r.a * inv.a;
+  z.b = r.b * inv.b;
+  stp(sd.z, u, z);
+  stp(sd.p1, u, r);
+  e.a = fma(alpha, p.a, e.a);
+  e.b = fma(alpha, p.b, e.b);
+  stp(sd.e, u, e);
+  rz.add(r.a, z.a);
+  rz.add(r.b, z.b);
+  rr.add(r.a, r.a);
+  rr.add(r.b, r.b);
 }
 
 // The residual r = b - (1 + xd) x - sum C (x_i - x_j) (the form of ref_axis),
-// D = 1 + xd + sum C, z = r x (1 / D) on oct o.
-template <int A>
-__device__ __forceinline__ void resd_ref_axis(const SolveDev &sd, int o, const int (&nb)[6], const double (&xv)[8],
-                                              double (&acc)[8], double (&ds)[8]) {
-  constexpr int bit = 1 << A;
-  double Cu[8];
-  ld8_ro(sd.C64 + (3 * (size_t)o + A) * 8, Cu);
+// D = 1 + xd + sum C, z = r x (1 / D) on unit u.
+__device__ __forceinline__ void resd_ref(const SolveDev &sd, int u, bool want_x, Acc<double> &rr, Acc<double> &xx,
+                                         Acc<double> &rz) {
+  const Stencil64 s = resd_stencil(sd, u);
+  const double *x = sd.x64;
+  const Pair64 v = ldp_cg(x + 2 * (size_t)u);
+  const double df = v.a - v.b;
+  Pair64 acc = {s.cx.a * df, -s.cx.a * df}, ds = {s.cx.a + s.cxm, s.cx.a + s.cx.b};
+  acc.b = fma(s.cx.b, v.b - ld1_cg(x + s.xp), acc.b);
+  acc.a = fma(s.cxm, v.a - ld1_cg(x + s.xm), acc.a);
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    if (c & bit) continue;
-    const int d = c | bit;
-    const double df = xv[c] - xv[d];
-    acc[c] = fma(Cu[c], df, acc[c]);
-    acc[d] = fma(-Cu[c], df, acc[d]);
-    ds[c] += Cu[c];
-    ds[d] += Cu[c];
+  for (int a = 0; a < 2; ++a) {
+    const Pair64 xu = ldp_cg(x + s.up[a]), xd = ldp_cg(x + s.dn[a]);
+    acc.a = fma(s.cup[a].a, v.a - xu.a, acc.a);
+    acc.b = fma(s.cup[a].b, v.b - xu.b, acc.b);
+    acc.a = fma(s.cdn[a].a, v.a - xd.a, acc.a);
+    acc.b = fma(s.cdn[a].b, v.b - xd.b, acc.b);
+    ds.a += s.cup[a].a + s.cdn[a].a;
+    ds.b += s.cup[a].b + s.cdn[a].b;
   }
-  int n = nb[2 * A + 1];
-  if (n >= 0) {
-    double Xn[8];
-    ldc_face<A, 0>(sd.x64 + 8 * (size_t)n, Xn);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      if (!(c & bit)) continue;
-      acc[c] = fma(Cu[c], xv[c] - Xn[c ^ bit], acc[c]);
-      ds[c] += Cu[c];
-    }
-  }
-  n = nb[2 * A];
-  if (n >= 0) {
-    double Xn[8], Cn[8];
-    ldc_face<A, 1>(sd.x64 + 8 * (size_t)n, Xn);
-    ld_face<A, 1>(sd.C64 + (3 * (size_t)n + A) * 8, Cn);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      if (c & bit) continue;
-      acc[c] = fma(Cn[c | bit], xv[c] - Xn[c | bit], acc[c]);
-      ds[c] += Cn[c | bit];
-    }
-  }
-}
-
-__device__ __forceinline__ void resd_ref_oct(const SolveDev &sd, int o, bool want_x, Acc<double> &rr, Acc<double> &xx,
-                                             Acc<double> &rz) {
-  int nb[6];
-  load_nbr6(sd.nbr, o, nb);
-  check_nbr6(nb, sd.n_oct);
+  const int o = u >> 2, c = 2 * (u & 3);
   int rec = __ldg(sd.xrec + o);
   if (rec >= 0 && !idx_ok(rec, sd.n_xd)) rec = -1;
-  double xv[8], acc[8], ds[8];
-  ldc8(sd.x64 + 8 * (size_t)o, xv);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) acc[c] = ds[c] = 0.0;
-  resd_ref_axis<0>(sd, o, nb, xv, acc, ds);
-  resd_ref_axis<1>(sd, o, nb, xv, acc, ds);
-  resd_ref_axis<2>(sd, o, nb, xv, acc, ds);
-  double t[8];
+  Pair64 m = {1.0, 1.0};
   if (rec >= 0) {
-    ld8_ro(sd.xd64 + 8 * (size_t)rec, t);
-  } else {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) t[c] = 0.0;
+    const Pair64 xd = ldp_ro(sd.xd64 + 8 * (size_t)rec + c);
+    m.a += xd.a;
+    m.b += xd.b;
   }
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const double m = 1.0 + t[c];
-    acc[c] = fma(m, xv[c], acc[c]);
-    ds[c] += m;
-  }
-  ld8_ro(sd.b64 + 8 * (size_t)o, t);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) acc[c] = t[c] - acc[c];
-  ld8_ro(sd.K64 + 8 * (size_t)o, t);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const bool leaf = t[c] >= 0.0;
-    const double r = leaf ? acc[c] : 0.0;
-    const double inv = leaf ? 1.0 / ds[c] : 1.0;
-    const double z = r * inv;
-    if (leaf) {
-      rr.add(r, r);
-      rz.add(r, z);
-      if (want_x) xx.add(xv[c], xv[c]);
-    }
-    acc[c] = r;
-    ds[c] = inv;
-    t[c] = z;
-  }
-  st8((double *)sd.p1 + 8 * (size_t)o, acc);
-  st8((double *)sd.dg + 8 * (size_t)o, ds);
-  st8((double *)sd.z + 8 * (size_t)o, t);
+  const Pair64 b = ldp_ro(sd.b64 + 2 * (size_t)u), K = ldp_ro(sd.K64 + 2 * (size_t)u);
+  const bool la = K.a >= 0.0, lb = K.b >= 0.0;
+  Pair64 r, z, inv;
+  r.a = la ? b.a - fma(m.a, v.a, acc.a) : 0.0;
+  r.b = lb ? b.b - fma(m.b, v.b, acc.b) : 0.0;
+  inv.a = la ? 1.0 / (ds.a + m.a) : 1.0;
+  inv.b = lb ? 1.0 / (ds.b + m.b) : 1.0;
+  z.a = r.a * inv.a;
+  z.b = r.b * inv.b;
+  rr.add(r.a, r.a);
+  rr.add(r.b, r.b);
+  rz.add(r.a, z.a);
+  rz.add(r.b, z.b);
+  if (want_x && la) xx.add(v.a, v.a);
+  if (want_x && lb) xx.add(v.b, v.b);
+  stp(sd.p1, u, r);
+  stp(sd.dg, u, inv);
+  stp(sd.z, u, z);
+}
+
+// x += e, e = 0 on unit u.
+__device__ __forceinline__ void resd_xpe(const SolveDev &sd, int u) {
+  const Pair64 e = ldp_rw(sd.e, u);
+  Pair64 x = ldp_rw(sd.x64, u);
+  x.a += e.a;
+  x.b += e.b;
+  stp(sd.x64, u, x);
+  stp(sd.e, u, {0.0, 0.0});
 }
 
 // One FP64 solve by one group (kG: 0 one CTA, 1 a cluster, 2 every CTA of a
@@ -3920,14 +3931,14 @@ __device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &
   const int n = sd.n_oct;
   const int chunk = (int)((n + (int)cs - 1) / (int)cs);
   const int lo = min(n, (int)cr * chunk), hi = min(n, lo + chunk);
-  const int o0 = lo + (int)threadIdx.x, stride = (int)blockDim.x;
+  const int u0 = 4 * lo + (int)threadIdx.x, u1 = 4 * hi, stride = (int)blockDim.x;
   const bool want_x = sd.stop_rule == ATS_STOP_CERTIFIED;
   for (;;) {
     const int phase = sh.st.phase;
     if (phase == kDone) break;
     if (phase == kRefine) {
       Acc<double> acc[3], tot[3];
-      for (int o = o0; o < hi; o += stride) resd_ref_oct(sd, o, want_x, acc[0], acc[1], acc[2]);
+      for (int u = u0; u < u1; u += stride) resd_ref(sd, u, want_x, acc[0], acc[1], acc[2]);
       const bool ok = res2_sum<3, kG>(acc, sh, a, buf, tot);
       if (threadIdx.x == 0) {
         if (ok) refine_decision(sh.st, sd, tot[0].get(), tot[1].get(), tot[2].get());
@@ -3940,7 +3951,7 @@ __device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &
       const bool first = sh.st.first != 0;
       const double beta = sh.st.beta;
       Acc<double> acc[1], tot[1];
-      for (int o = o0; o < hi; o += stride) resd_op_oct(sd, o, first, beta, acc[0]);
+      for (int u = u0; u < u1; u += stride) resd_op(sd, u, first, beta, acc[0]);
       const bool ok = res2_sum<1, kG>(acc, sh, a, buf, tot);
       if (threadIdx.x == 0) {
         ResState &st = sh.st;
@@ -3958,7 +3969,7 @@ __device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &
     {
       const double alpha = sh.st.alpha;
       Acc<double> acc[2], tot[2];
-      for (int o = o0; o < hi; o += stride) resd_upd_oct(sd, o, alpha, acc[0], acc[1]);
+      for (int u = u0; u < u1; u += stride) resd_upd(sd, u, alpha, acc[0], acc[1]);
       const bool ok = res2_sum<2, kG>(acc, sh, a, buf, tot);
       if (threadIdx.x == 0) {
         if (ok) step_decision(sh.st, sd, cg_beta(sh.st, tot[0], tot[1], false));
@@ -3969,7 +3980,7 @@ __device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &
     if (sh.st.phase == kDone) break;
     if (sh.st.phase == kRefine) {
       // x += e, e = 0; the residual pass reads the neighbours' x
-      for (int o = o0; o < hi; o += stride) res_xpe_oct<double>(sd, o);
+      for (int u = u0; u < u1; u += stride) resd_xpe(sd, u);
       if (!res2_barrier<kG>(a, sh)) {
         if (threadIdx.x == 0) res2_timeout(sh.st);
         break;

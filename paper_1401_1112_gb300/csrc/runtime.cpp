@@ -603,10 +603,11 @@ void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
 }
 
 // FP64 resident groups: octs per CTA up to which the next smaller group is
-// taken.  An FP64 step is bound by the SM's FP64 pipe (2 100 cycles per warp
-// of octs and CG iteration, four warps side by side), a cluster's two sums
-// cost about 3 000: runs of 128 octs keep the pipe busy most of a step and
-// spread a level over as many SMs as that allows.
+// taken.  An FP64 step is bound by the SM's FP64 pipe (about 65 cycles per oct
+// and CG iteration), a cluster's two sums cost about 4 000: runs of 128 octs
+// keep the pipe busy most of a step and spread a level over as many SMs as
+// that allows (128 levels of 64 .. 2 048 octs 2.67 ms; with runs of 64 octs
+// 3.02 ms, one level of 512 octs alone 7.4 instead of 9.8 us per iteration).
 constexpr int64_t kRun64 = 128;
 // FP32-bulk resident groups with the default limits: runs of up to 1 024 octs
 // (the register layout that keeps every private array on chip).  A step's
