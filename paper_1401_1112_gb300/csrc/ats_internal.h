@@ -137,7 +137,6 @@ cudaError_t launch_coef_build_batch(const CoefArgs *args, const int32_t *blk_lev
 // 8 o + c and its +a neighbour j when both are leaves (K >= 0), else 0.
 cudaError_t launch_face_coef(int64_t n_oct, const int32_t *nbr, const double *K64, double h, double *C64,
                              cudaStream_t st);
-cudaError_t launch_gather_flags(const int *const *flags, int n, int *out, cudaStream_t st);
 
 // Device state of a planned batch, passed by value to the tick kernels.
 // Cells processed, counted when profiling: [0] k_op CG items after the first
@@ -275,8 +274,28 @@ cudaError_t launch_grid_barrier_probe(int grid, const ResArgs &a, int *out, cuda
 
 // Start of a solve: e = 0 on every cell of every item, and x64 = src[solve]
 // where src (device array of device pointers) is non-null for that solve.
+// reset (may be null): the run state that the same launch puts in place.
+struct RunReset {
+  // n_words 8-byte words of initial scalars, copied to the live and the final ones
+  const unsigned long long *init;
+  unsigned long long *sc, *fin;
+  int n_words;
+  const int *active0, *ctl0;  // initial active count and tick control block (ctl_words ints)
+  int *active, *ctl;
+  int ctl_words;
+  const int32_t *ident;  // n_list entries of the tick path's first list
+  int32_t *list;
+  int n_list;
+  int *const *flag_ptrs;  // the n levels' error flags, gathered into flags
+  int *flags;
+  int n;
+  unsigned long long *zero64[2];  // arrays set to zero: 8-byte words ...
+  int n_zero64[2];
+  int *zero32[4];                 // ... and ints
+  int n_zero32[4];
+};
 cudaError_t launch_init(bool fp64, const SolveDev *solves, const WorkItem *items, int n_items,
-                        const double *const *src, int grid, cudaStream_t st);
+                        const double *const *src, int grid, cudaStream_t st, const RunReset *reset = nullptr);
 // End of a solve: dst[solve] = x64 (2 x64 - E^n for Crank-Nicolson) where
 // dst[solve] is non-null; neg[solve] |= 1 (neg may be null) when a value of
 // the result is negative.

