@@ -143,6 +143,7 @@ cudaError_t launch_face_coef(int64_t n_oct, const int32_t *nbr, const double *K6
 // iteration of an inner solve, [1] k_ref, [2] k_upd CG items, [3] x += e at
 // the end of an inner solve, [4] k_op CG items in a first iteration.
 constexpr int kCellCounters = 5;
+constexpr int kGridBarWords = 5 * 64;  // see ResArgs::gbar; word 2 is the give-up flag
 
 struct TickArgs {
   const SolveDev *solves;
@@ -212,8 +213,9 @@ struct ResArgs {
   unsigned long long *t_solve;  // [n_solves][2] %globaltimer at a solve's start and end (profiling), or null
   int cap;                      // shared-memory form: octs per CTA kept in shared memory (0: none)
   // whole-GPU form (launch_resident_grid): every CTA of one cooperative
-  // launch works on gq[0], gq[1], ... in turn; gbar[0] = the arrivals at
-  // its grid barriers so far (zeroed before the launch; gbar[1] unused),
+  // launch works on gq[0], gq[1], ... in turn; gbar (kGridBarWords words, zeroed
+  // before the launch): [0] = the arrivals at its grid barriers so far, from
+  // word 64 on the words of its fixed-point sums,
   // gpart = [2][grid + 1][3] sums (FP32 bulk: (hi, lo) pairs): per buffer, each CTA's partial
   // sums (the last row unused); *gerr set when a barrier wait gave up
   const int32_t *gq;

@@ -276,7 +276,7 @@ struct Plan {
   std::vector<int32_t> h_queue;  // the queue order last uploaded
   unsigned *d_gbar = nullptr;
   double *d_gpart = nullptr;
-  int *d_gerr = nullptr;  // (the word behind d_gbar's two)
+  int *d_gerr = nullptr;  // (word 2 of d_gbar)
   int res_threads = 512, res_cluster = 8, res_cluster_big = 16, res_grid = 0, res_grid_big = 0;
   int res_cluster_mid = 8, res_grid_mid = 0;
   bool res_smem = false;  // K, z, p of each CTA's octs in shared memory (FP32 bulk)
@@ -863,7 +863,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       (s = dev_alloc_t(ctx, 1, &P->d_active)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 2 * kCellCounters, &P->d_cells)) != ATS_OK ||
       (s = dev_alloc_t(ctx, std::max(1, P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq), &P->d_queue)) != ATS_OK ||
-      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 3, &P->d_gbar)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_t(ctx, kGridBarWords, &P->d_gbar)) != ATS_OK) ||
       (P->n_gq > 0 && (s = dev_alloc_t(ctx, 6 * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
       (s = dev_alloc_t(ctx, 4, &P->d_heads)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 4 * (size_t)P->n_items, &P->d_lists)) != ATS_OK ||
@@ -1450,8 +1450,8 @@ ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off
   rs.n_zero32[0] = 4;
   rs.zero32[1] = ro.neg;
   rs.n_zero32[1] = n;
-  rs.zero32[2] = (int *)P->d_gbar;  // the barrier's counter (two words) and, behind it, the give-up flag
-  rs.n_zero32[2] = P->d_gbar ? 3 : 0;
+  rs.zero32[2] = (int *)P->d_gbar;  // the barrier's counter, the give-up flag, the fixed-point words
+  rs.n_zero32[2] = P->d_gbar ? kGridBarWords : 0;
   rs.zero32[3] = ro.zero;
   rs.n_zero32[3] = ro.zero ? 1 : 0;
   CUDA_TRY(launch_init(P->fp64, P->d_solves, P->d_items, P->n_items, P->d_src, P->grid, st, &rs));
