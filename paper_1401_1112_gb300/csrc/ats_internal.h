@@ -143,6 +143,7 @@ cudaError_t launch_face_coef(int64_t n_oct, const int32_t *nbr, const double *K6
 // iteration of an inner solve, [1] k_ref, [2] k_upd CG items, [3] x += e at
 // the end of an inner solve, [4] k_op CG items in a first iteration.
 constexpr int kCellCounters = 5;
+constexpr int kResLock = 16;  // levels of an FP64 whole-GPU launch in flight at once
 constexpr int kGridBarWords = 5 * 64;  // see ResArgs::gbar; word 2 is the give-up flag
 
 struct TickArgs {
@@ -216,10 +217,11 @@ struct ResArgs {
   // launch works on gq[0], gq[1], ... in turn; gbar (kGridBarWords words, zeroed
   // before the launch): [0] = the arrivals at its grid barriers so far, from
   // word 64 on the words of its fixed-point sums,
-  // gpart = [2][grid + 1][3] sums (FP32 bulk: (hi, lo) pairs): per buffer, each CTA's partial
-  // sums (the last row unused); *gerr set when a barrier wait gave up
+  // gpart = [2][grid + 1][3] sums ((hi, lo) pairs; FP64: [2][n_lock][grid][3]): per
+  // buffer, each CTA's partial sums; *gerr set when a barrier wait gave up
   const int32_t *gq;
   int n_gq;
+  int n_lock;  // FP64: levels in flight at once (at most kResLock; gpart holds as many rows)
   unsigned *gbar;
   double *gpart;
   int *gerr;

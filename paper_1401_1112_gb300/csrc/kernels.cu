@@ -4029,10 +4029,9 @@ __device__ __forceinline__ void resd_xpe(const SolveDev &sd, int u) {
 }
 
 // One FP64 solve by one group (kG: 0 one CTA, 1 a cluster, 2 every CTA of a
-// cooperative launch), the state machine of res2_solve_l.  Returns false when
-// a whole-GPU barrier wait gave up (the solve then ends with ATS_ERR_TIMEOUT).
+// cooperative launch), the state machine of res2_solve_l.
 template <int kG>
-__device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &buf) {
+__device__ void resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &buf) {
   constexpr int wd = (int)(sizeof(SolveDev) / 8);
   for (int w = threadIdx.x; w < wd; w += blockDim.x)
     reinterpret_cast<unsigned long long *>(&sh.sd)[w] = reinterpret_cast<const unsigned long long *>(a.solves + s)[w];
@@ -4107,10 +4106,217 @@ __device__ bool resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &
       }
     }
   }
-  __syncthreads();  // thread 0's last state update is seen by all
-  const bool alive = sh.st.status != ATS_ERR_TIMEOUT;
   if (threadIdx.x == 0 && cr == 0) res_finish(a, s, sh.st, n);
-  return alive;
+}
+
+// ---- the whole-GPU form: several levels in lockstep ----
+// A level alone leaves the FP64 pipes idle while its sums travel (4 096 octs:
+// 1.1 us of pipe per 9.7 us step), so the launch advances up to kLock levels
+// of its queue together: a superstep does the next pass of every level in
+// flight (residual, step 1, step 2 or x += e) on this CTA's run of that level,
+// then one grid barrier carries all their sums, which warp k merges for slot
+// k, and a level that has ended makes room for the next one.  A level's runs,
+// the order of its sums and its decisions are those of resd_solve<2> and
+// involve no other level: the pass of slot k starts at a warp of its own (short
+// runs of several levels then use different quarters of the pipe), and its
+// warps are counted from there.  resd_solve<2> stays for a level alone, whose
+// step is shorter without the slots (4 096 octs 9.7 against 11.3 us).
+// Measured: 24 levels of 2 100 .. 9 000 octs 9.0 ms (tick path 19.5), 64 of
+// 2 100 .. 16 000 29.0 (45.7), 12 of 16 500 .. 32 768 14.2 (34.2).
+constexpr int kStepRef = 0, kStepOp = 1, kStepUpd = 2, kStepXpe = 3;
+struct ResdLock {
+  SolveDev sd[kResLock];
+  ResState st[kResLock];
+  Acc<double> red[kResLock][kResMaxWarps][3];  // [slot][warp][sum]
+  int s[kResLock];     // the solve in each slot (-1: none)
+  int step[kResLock];  // its next pass
+  int rot[kResLock];   // the warp its pass starts at
+  int fresh[kResLock];
+  int live, flag;
+};
+
+// The warp's totals of a pass into row `vw` of red.
+template <int NA>
+__device__ __forceinline__ void resd_reduce(Acc<double> (&a)[3], Acc<double> (*red)[3], int vw) {
+  const int lane = threadIdx.x & 31;
+  const Acc<double> t = NA >= 2 ? warp_fold(a[0], a[1]) : warp_fold(a[0]);
+  if (lane == 0) red[vw][0] = t;
+  if (NA >= 2 && lane == 16) red[vw][1] = t;
+  if (NA == 3) {
+    const Acc<double> t2 = warp_fold(a[2]);
+    if (lane == 0) red[vw][2] = t2;
+  }
+}
+
+__device__ void resd_lockstep(const ResArgs &a, ResdLock &L) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int G = (int)gridDim.x, cta = (int)blockIdx.x, slots = a.n_lock;
+  constexpr int NT = 32 * kResMaxWarps;
+  int next = 0, buf = 0;  // (every thread counts the queue)
+  if (threadIdx.x < kResLock) L.s[threadIdx.x] = -1;
+  const auto sums_of = [](int step) { return step == kStepRef ? 3 : step == kStepOp ? 1 : step == kStepUpd ? 2 : 0; };
+  const auto run_of = [&](const SolveDev &sd, int &lo) {
+    const int chunk = (sd.n_oct + G - 1) / G;
+    lo = min(sd.n_oct, cta * chunk);
+    return min(sd.n_oct, lo + chunk) - lo;
+  };
+  for (;;) {
+    __syncthreads();
+    // free slots take the next solves of the queue
+    int live = 0;
+    for (int k = 0; k < slots; ++k) {
+      int s = L.s[k];
+      bool fresh = false;
+      while (s < 0 && next < a.n_gq) {
+        s = a.gq[next++];
+        if (!idx_ok(s, a.n_solves)) s = -1;
+        fresh = s >= 0;
+      }
+      live += s >= 0;
+      if (fresh && warp == k) {
+        for (int w = lane; w < (int)(sizeof(SolveDev) / 8); w += 32)
+          reinterpret_cast<unsigned long long *>(&L.sd[k])[w] =
+              reinterpret_cast<const unsigned long long *>(a.solves + s)[w];
+        if (lane == 0) {
+          ResState z;
+          memset(&z, 0, sizeof(z));
+          z.phase = kRefine;
+          z.status = ATS_OK;
+          L.st[k] = z;
+          L.step[k] = kStepRef;
+          L.fresh[k] = s;
+          if (a.t_solve && cta == 0) a.t_solve[2 * s] = globaltimer_ns();
+        }
+      } else if (lane == 0 && warp == k) {
+        L.fresh[k] = -1;
+      }
+    }
+    if (live == 0) return;
+    __syncthreads();
+    if (warp == 0) {  // (the slots are read above by every thread)
+      if (lane < slots && L.fresh[lane] >= 0) L.s[lane] = L.fresh[lane];
+      __syncwarp();
+      if (lane == 0) {
+        int first = 0;
+        for (int k = 0; k < slots; ++k) {
+          if (L.s[k] < 0) continue;
+          int lo;
+          L.rot[k] = first;
+          first = (first + (4 * run_of(L.sd[k], lo) + 31) / 32) % kResMaxWarps;
+        }
+      }
+    }
+    __syncthreads();
+    // the passes
+    for (int k = 0; k < slots; ++k) {
+      if (L.s[k] < 0) continue;
+      const SolveDev &sd = L.sd[k];
+      const ResState &st = L.st[k];
+      int lo;
+      const int run = run_of(sd, lo);
+      const int vt = ((int)threadIdx.x - 32 * L.rot[k]) & (NT - 1);
+      if ((vt & ~31) >= 4 * run) continue;  // (the whole warp has no unit)
+      const int u0 = 4 * lo + vt, u1 = 4 * (lo + run), vw = vt >> 5;
+      Acc<double> acc[3];
+      switch (L.step[k]) {
+        case kStepRef: {
+          const bool want_x = sd.stop_rule == ATS_STOP_CERTIFIED;
+          for (int u = u0; u < u1; u += NT) resd_ref(sd, u, want_x, acc[0], acc[1], acc[2]);
+          resd_reduce<3>(acc, L.red[k], vw);
+          break;
+        }
+        case kStepOp: {
+          const bool first = st.first != 0;
+          const double beta = st.beta;
+          for (int u = u0; u < u1; u += NT) resd_op(sd, u, first, beta, acc[0]);
+          resd_reduce<1>(acc, L.red[k], vw);
+          break;
+        }
+        case kStepUpd: {
+          const double alpha = st.alpha;
+          for (int u = u0; u < u1; u += NT) resd_upd(sd, u, alpha, acc[0], acc[1]);
+          resd_reduce<2>(acc, L.red[k], vw);
+          break;
+        }
+        default:
+          for (int u = u0; u < u1; u += NT) resd_xpe(sd, u);
+      }
+    }
+    __syncthreads();
+    // this CTA's totals, the barrier, the grid's totals and the decisions
+    const bool mine = warp < slots && L.s[warp < slots ? warp : 0] >= 0;
+    const int na = mine ? sums_of(L.step[warp]) : 0;
+    double *row = a.gpart + ((size_t)buf * slots + (mine ? warp : 0)) * G * 3;
+    if (na > 0) {
+      int lo;
+      const int nw = min(kResMaxWarps, (4 * run_of(L.sd[warp], lo) + 31) / 32);
+      for (int j = 0; j < na; j += 2) {
+        const int j2 = min(j + 1, na - 1);
+        const Acc<double> m = merge_entries<double>(L.red[warp], nw, j, j2);
+        if (lane == 0) Slot<double>::store(row + (size_t)cta * 3 + j, m);
+        if (lane == 16 && j2 > j) Slot<double>::store(row + (size_t)cta * 3 + j2, m);
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const bool ok = grid_wait(a, grid_arrive(a));
+      if (lane == 0) L.flag = ok ? 1 : 0;
+    }
+    __syncthreads();
+    if (!L.flag) break;
+    if (mine) {
+      double tot[3] = {0.0, 0.0, 0.0};
+      for (int j = 0; j < na; ++j) {
+        Acc<double> v[kGridMaxPerLane], t;
+#pragma unroll
+        for (int i = 0; i < kGridMaxPerLane; ++i) {
+          const int r = lane + 32 * i;
+          if (r < G) v[i] = Slot<double>::load(row + (size_t)r * 3 + j);
+        }
+#pragma unroll
+        for (int i = 0; i < kGridMaxPerLane; ++i) t.merge(v[i]);
+        lanes_total<16>(t);
+        tot[j] = t.get();
+      }
+      if (lane == 0) {
+        ResState &st = L.st[warp];
+        const SolveDev &sd = L.sd[warp];
+        int &step = L.step[warp];
+        Acc<double> t0, t1;
+        t0.s = tot[0];
+        t1.s = tot[1];
+        if (step == kStepRef) {
+          refine_decision(st, sd, tot[0], tot[1], tot[2]);
+          step = kStepOp;
+        } else if (step == kStepOp) {
+          st.n_op += 1;
+          st.n_first += st.first ? 1 : 0;
+          cg_alpha(st, t0, false);
+          step = kStepUpd;
+        } else if (step == kStepUpd) {
+          step_decision(st, sd, cg_beta(st, t0, t1, false));
+          step = st.phase == kRefine ? kStepXpe : kStepOp;
+        } else {
+          step = kStepRef;
+        }
+        if (st.phase == kDone) {
+          if (cta == 0) res_finish(a, L.s[warp], st, sd.n_oct);
+          L.s[warp] = -1;
+        }
+      }
+    }
+    buf ^= 1;
+  }
+  // a wait gave up: what is in flight ends with ATS_ERR_TIMEOUT, the rest is not started
+  if (cta == 0 && threadIdx.x == 0) {
+    for (int k = 0; k < slots; ++k) {
+      if (L.s[k] < 0) continue;
+      res2_timeout(L.st[k]);
+      res_finish(a, L.s[k], L.st[k], L.sd[k].n_oct);
+    }
+  }
+  for (; next < a.n_gq; ++next)
+    if (idx_ok(a.gq[next], a.n_solves)) res_never_ran(a, a.gq[next]);
 }
 
 __device__ void resd_cta_loop(const ResArgs &a, ResShared<double> &sh, int &buf) {
@@ -4161,18 +4367,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_resd_cta(ResArgs a) {
   resd_cta_loop(a, sh, buf);
 }
 
-// The whole-GPU form (see k_res2_grid).
-template <int NT>
+// The whole-GPU form: one level, or several in lockstep.
+template <int NT, bool kLockstep>
 __global__ void __launch_bounds__(NT, 1) k_resd_grid(ResArgs a) {
-  __shared__ ResShared<double> sh;
-  int buf = 0;
-  bool alive = true;
-  for (int t = 0; t < a.n_gq; ++t) {
-    const int s = a.gq[t];
-    if (!idx_ok(s, a.n_solves)) continue;
-    if (alive) alive = resd_solve<2>(a, s, sh, buf);
-    else res_never_ran(a, s);
-    __syncthreads();  // every thread has left the solve before the next one starts
+  static_assert(NT == 32 * kResMaxWarps && kResLock <= kResMaxWarps, "a warp per slot");
+  if constexpr (kLockstep) {
+    __shared__ ResdLock L;
+    resd_lockstep(a, L);
+  } else {
+    __shared__ ResShared<double> sh;
+    int buf = 0;
+    if (idx_ok(a.gq[0], a.n_solves)) resd_solve<2>(a, a.gq[0], sh, buf);
   }
 }
 
@@ -4347,16 +4552,16 @@ int resident_smem_cap(int threads, int device) {
 // The whole-GPU form of a bulk precision: its kernel and dynamic shared memory.
 using ResGridKernel = void (*)(ResArgs);
 template <int NT>
-static ResGridKernel res_grid_kernel(bool fp64, int regs, size_t *smem) {
+static ResGridKernel res_grid_kernel(bool fp64, int regs, bool lockstep, size_t *smem) {
   *smem = fp64 ? 0 : kRes2SmemBytes;
-  if (fp64) return k_resd_grid<NT>;
+  if (fp64) return lockstep ? k_resd_grid<NT, true> : k_resd_grid<NT, false>;
   return regs == 2 ? k_res2_grid<NT, kStateTail> : regs == 1 ? k_res2_grid<NT, kStateRegs> : k_res2_grid<NT, kStateShared>;
 }
 
 template <int NT>
 static cudaError_t res2_grid_launch_t(bool fp64, int grid, const ResArgs &a, cudaStream_t st) {
   size_t smem = 0;
-  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, a.regs, &smem);
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, a.regs, a.n_gq > 1, &smem);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -4376,7 +4581,7 @@ template <int NT>
 static int res2_grid_ctas_t(bool fp64, int device) {
   int b = 0, sms = 0;
   size_t smem = 0;
-  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, 0, &smem);
+  const ResGridKernel kernel = res_grid_kernel<NT>(fp64, 0, true, &smem);
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, NT, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {

@@ -140,6 +140,24 @@ ats_status dev_alloc_t(ats_context *ctx, size_t count, P **out) {
   return s;
 }
 
+// A few kilobytes of barrier and partial-sum words that a plan did not always
+// have: kept out of the context's budget, so that a solve that used to fit it
+// still does.
+template <typename P>
+ats_status dev_alloc_uncounted(ats_context *ctx, size_t bytes, P **out) {
+  void *p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    set_error(std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
+    return ATS_ERR_OOM;
+  }
+  ctx->allocs[p] = 0;
+  ++ctx->epoch;
+  *out = (P *)p;
+  return ATS_OK;
+}
+
 void dev_free(ats_context *ctx, void *p) {
   if (!p) return;
   ++ctx->epoch;
@@ -262,6 +280,7 @@ struct Plan {
   // takes these solves one after another); its barrier, partial sums and
   // give-up flag
   int n_gq = 0, res_grid_all = 0;
+  int res_lock = 1;  // FP64: levels of the whole-GPU launch in flight at once
   // the split of the device's CTA slots between the three resident launches:
   // clusters of each size that fit at once, the slots, and whether the split
   // follows measured per-class SM-time (after a completed run) or the
@@ -855,6 +874,8 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
   P->out_ts = sizeof(SolveScalars) * (size_t)n;
   P->out_flags = P->out_ts + 2 * sizeof(unsigned long long) * (size_t)n;
   P->out_bytes = P->out_flags + 2 * sizeof(int) * (size_t)n;
+  const size_t lock = (size_t)std::max(1, P->fp64 ? std::min(kResLock, P->n_gq) : 1);
+  P->res_lock = (int)lock;
   if ((s = dev_alloc_t(ctx, n, &P->d_solves)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 2 * (size_t)n, &P->d_sc)) != ATS_OK ||
       (s = dev_alloc_t(ctx, P->out_bytes, &P->d_out)) != ATS_OK ||
@@ -863,8 +884,8 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       (s = dev_alloc_t(ctx, 1, &P->d_active)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 2 * kCellCounters, &P->d_cells)) != ATS_OK ||
       (s = dev_alloc_t(ctx, std::max(1, P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq), &P->d_queue)) != ATS_OK ||
-      (P->n_gq > 0 && (s = dev_alloc_t(ctx, kGridBarWords, &P->d_gbar)) != ATS_OK) ||
-      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 6 * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_uncounted(ctx, sizeof(unsigned) * kGridBarWords, &P->d_gbar)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_uncounted(ctx, 6 * sizeof(double) * lock * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
       (s = dev_alloc_t(ctx, 4, &P->d_heads)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 4 * (size_t)P->n_items, &P->d_lists)) != ATS_OK ||
       (s = dev_alloc_t(ctx, (size_t)P->n_items, &P->d_ident)) != ATS_OK ||
@@ -1049,6 +1070,7 @@ ats_status plan_launch_resident(Plan *P, bool prof, int *neg, SolveScalars *fina
     ResArgs a = ra;
     a.gq = P->d_queue + P->n_bq + P->n_mq + P->n_cq + P->n_tq;
     a.n_gq = P->n_gq;
+    a.n_lock = P->res_lock;
     a.gbar = P->d_gbar;
     a.gpart = P->d_gpart;
     a.gerr = P->d_gerr;

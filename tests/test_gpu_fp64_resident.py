@@ -82,3 +82,34 @@ def test_irregular_levels_with_shift_match_oracle(ats, ctx, seed, form):
     kw = {"cta": dict(res_cta_octs=4096), "cluster": dict(res_cta_octs=-1, res_cluster=2),
           "grid": dict(sched=ats.ATS_SCHED_GRID, res_max_octs=8)}[form]
     _check(ats, ctx, lv, st, **kw)
+
+
+def test_levels_in_lockstep_give_their_solo_bits(ats, ctx):
+    """18 levels above the clusters' limit in one launch (16 in flight, the others as places free up), beside two small
+    ones: each gives the bits it gives alone, and one is checked against the oracle."""
+    rng = np.random.default_rng(5)
+    cases = [W.random_box_solve(rng, o, robin=True) for o in np.linspace(2100, 6000, 18).tolist() + [60, 900]]
+    levels, solo = [], []
+    opts = dict(tol=TOL, stop_rule=ats.ATS_STOP_CERTIFIED, precision=ats.ATS_PREC_FP64)
+    for lv, st in cases:
+        L = ats.Level(ctx, lv)
+        L.build(st.dt, st.K, st.E, face_K=st.face_K, face_E=st.face_E, face_F=st.face_F)
+        x = st.E.copy()
+        code, stats = L.solve(x, **opts)
+        assert code >= 0, stats
+        levels.append(L)
+        solo.append((x, stats))
+    B = ats.Batch(ctx, levels, **opts)
+    xs = [st.E.copy() for _, st in cases]
+    code, stats = B.solve(xs)
+    assert code >= 0
+    for (x, s), y, t in zip(solo, xs, stats):
+        np.testing.assert_array_equal(y, x)
+        assert s == t
+    lv, st = cases[3]
+    xr, _ = oracle.pcg(oracle.assemble(lv, st.dt, st.K, st.E, face_K=st.face_K, face_E=st.face_E, face_F=st.face_F),
+                       st.E, tol=TOL, stop_rule=oracle.STOP_CERTIFIED)
+    assert np.linalg.norm(xs[3] - xr) <= PAR * np.linalg.norm(xr)
+    B.close()
+    for L in levels:
+        L.close()
