@@ -351,7 +351,7 @@ __device__ __forceinline__ void op_face(int n, const T *__restrict__ KT, const T
   }
 }
 
-// k_ref, axis A of an oct: FP64 flux sums C (x_i - x_j) with the stored FP64
+// k_ref, axis A of an oct: acc -= the FP64 fluxes C (x_i - x_j) with the stored FP64
 // face coefficients C = h (K_i + K_j) (row A of this oct for the in-oct pairs
 // and the +A face, row A of the -A neighbour for the -A face), and the FP32
 // diagonal sums of the bulk precision.
@@ -363,6 +363,31 @@ __device__ __forceinline__ float rcp_approx(float d) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return r;
+}
+
+// FP64 -> FP32 and back on the integer pipe: the hardware's conversions run at
+// the FP64 rate (measured: 16 cycles per warp and SM, 94 for a warp alone), and
+// the residual pass, FP64-bound, makes 16 per oct and x += e 8.  With the
+// fluxes taken straight from b - (1 + xd) x: 64 octs 219 -> 177 us, 512 ragged
+// levels 14.2 -> 13.7 ms, four-level radiation step 10.9 -> 10.5 ms.  Rounds to nearest, a tie away from
+// zero; zero, subnormals, infinities, NaN and what leaves FP32's range take the
+// hardware's conversion.
+__device__ __forceinline__ float f32_of(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  if ((hi & 0x7fffffffu) - (897u << 20) >= (253u << 20)) return (float)v;
+  // the low eight exponent bits and the upper mantissa, the bias moved by -896 (+128 modulo 256)
+  const unsigned t = (__funnelshift_l(lo, hi, 3) + 0x40000000u) & 0x7fffffffu;
+  return __uint_as_float((t | (hi & 0x80000000u)) + ((lo >> 28) & 1u));
+}
+__device__ __forceinline__ double f64_of(float v) {
+  const unsigned u = __float_as_uint(v), a = u & 0x7fffffffu;
+  if (a - (1u << 23) >= (254u << 23)) return (double)v;
+  return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(u << 29));
+}
+template <typename T>
+__device__ __forceinline__ T bulk_of(double v) {
+  if constexpr (sizeof(T) == 4) return f32_of(v);
+  else return v;
 }
 
 template <int A, typename T, bool kCoh = false>
@@ -377,8 +402,8 @@ __device__ __forceinline__ void ref_axis(const SolveDev &sd, int o, const int (&
     if (c & bit) continue;
     const int d = c | bit;
     const double df = xv[c] - xv[d];
-    acc[c] = fma(Cu[c], df, acc[c]);
-    acc[d] = fma(-Cu[c], df, acc[d]);
+    acc[c] = fma(-Cu[c], df, acc[c]);
+    acc[d] = fma(Cu[c], df, acc[d]);
     if (KTo[c] >= T(0) && KTo[d] >= T(0)) {
       const T Ct = hT * (KTo[c] + KTo[d]);
       dsT[c] += Ct;
@@ -395,7 +420,7 @@ __device__ __forceinline__ void ref_axis(const SolveDev &sd, int o, const int (&
     for (int c = 0; c < 8; ++c) {
       if (!(c & bit)) continue;
       const int j = c ^ bit;
-      acc[c] = fma(Cu[c], xv[c] - Xn[j], acc[c]);
+      acc[c] = fma(-Cu[c], xv[c] - Xn[j], acc[c]);
       if (KTn[j] >= T(0)) dsT[c] += hT * (KTo[c] + KTn[j]);
     }
   }
@@ -410,7 +435,7 @@ __device__ __forceinline__ void ref_axis(const SolveDev &sd, int o, const int (&
     for (int c = 0; c < 8; ++c) {
       if (c & bit) continue;
       const int j = c | bit;
-      acc[c] = fma(Cn[j], xv[c] - Xn[j], acc[c]);
+      acc[c] = fma(-Cn[j], xv[c] - Xn[j], acc[c]);
       if (KTn[j] >= T(0)) dsT[c] += hT * (KTo[c] + KTn[j]);
     }
   }
@@ -439,32 +464,39 @@ __device__ __forceinline__ void ref_oct_values(const SolveDev &sd, int o, bool w
   T KTo[8];
   ldv8<kCoh>(sd.x64 + 8 * o, xv);
   ld8_ro(KT + 8 * o, KTo);
+  // the sum starts at b - (1 + xd) x and the fluxes are taken from it (eight
+  // FP64 subtractions fewer than a sum of their own)
   double acc[8];
-  T dsT[8];
+  T dsT[8], xdT[8];
+  ld8_ro(sd.b64 + 8 * (size_t)o, acc);
+  if (rec >= 0) {
+    double xd[8];
+    ld8_ro(sd.xd64 + 8 * (size_t)rec, xd);
+    if (mixed) ld8_ro((const T *)sd.xdT + 8 * (size_t)rec, xdT);
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    acc[c] = 0.0;
-    dsT[c] = T(0);
+    for (int c = 0; c < 8; ++c) {
+      acc[c] = fma(-(1.0 + xd[c]), xv[c], acc[c]);
+      if (!mixed) xdT[c] = (T)xd[c];
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      acc[c] -= xv[c];
+      xdT[c] = T(0);
+    }
   }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) dsT[c] = T(0);
   ref_axis<0, T, kCoh>(sd, o, nb, KT, hT, KTo, xv, acc, dsT);
   ref_axis<1, T, kCoh>(sd, o, nb, KT, hT, KTo, xv, acc, dsT);
   ref_axis<2, T, kCoh>(sd, o, nb, KT, hT, KTo, xv, acc, dsT);
-  double xd[8], b[8];
-  T xdT[8];
-  if (rec >= 0) {
-    ld8_ro(sd.xd64 + 8 * rec, xd);
-    if (mixed) ld8_ro((const T *)sd.xdT + 8 * rec, xdT);
-  }
-  ld8_ro(sd.b64 + 8 * o, b);
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const bool leaf = KTo[c] >= T(0);
-    const double base = rec >= 0 ? fma(-(1.0 + xd[c]), xv[c], b[c]) : b[c] - xv[c];
-    const double r = base - acc[c];
-    const T rT = (T)r;
+    const T rT = bulk_of<T>(acc[c]);
     // D in the bulk precision, kept for the CG kernels of the following
     // inner solve
-    const T dT = T(1) + (rec >= 0 ? (mixed ? xdT[c] : (T)xd[c]) : T(0)) + dsT[c];
+    const T dT = T(1) + xdT[c] + dsT[c];
     T zc;
     if constexpr (kRcp && sizeof(T) == 4) zc = rT * rcp_approx(dT);
     else zc = rT / dT;
@@ -474,7 +506,7 @@ __device__ __forceinline__ void ref_oct_values(const SolveDev &sd, int o, bool w
       rr.add(rT, rT);
       rz.add(rT, zc);
       if (want_x) {
-        const T xT = (T)xv[c];
+        const T xT = bulk_of<T>(xv[c]);
         xx.add(xT, xT);
       }
     }
@@ -1720,8 +1752,9 @@ int tick_blocks_per_sm(bool fp64, bool paper) {
 // later one (z, p, D, x) is read with ld.global.cg after the step's cluster
 // barrier (release / acquire at cluster scope); arrays no step writes (K, the
 // neighbour table, face coefficients, b, diagonal extras) take the read-only
-// path.  The FP32 bulk keeps its CG state in shared memory, the FP64 bulk in
-// global memory (L2); each has its own section below.
+// path.  The FP32 bulk keeps its CG state in registers and shared memory (or in
+// shared memory alone, for the options that need it), the FP64 bulk in global
+// memory (L2); each has its own section below.
 
 namespace {
 
@@ -2085,7 +2118,8 @@ __device__ __forceinline__ void res_xpe_oct(const SolveDev &sd, int o) {
   ldc8(sd.x64 + 8 * o, xv);
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    xv[c] += (double)ev[c];
+    if constexpr (sizeof(T) == 4) xv[c] += f64_of(ev[c]);
+    else xv[c] += ev[c];
     ev[c] = T(0);
   }
   st8(sd.x64 + 8 * o, xv);
@@ -2586,7 +2620,7 @@ __device__ __forceinline__ void res2_xpe_oct(const Cx &cx, const SolveDev &sd, i
   ldc8(sd.x64 + 8 * o, xv);
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    xv[c] += (double)e[c];
+    xv[c] += f64_of(e[c]);
     z0[c] = 0.f;
   }
   st8(sd.x64 + 8 * o, xv);
@@ -3674,8 +3708,8 @@ __device__ bool res3_solve_r(const ResArgs &a, int s, ResShared<float> &sh, int 
         for (int k = 0; k < 4; ++k) {
           float e0, e1;
           unpack2(e[r][k], e0, e1);
-          xv[2 * k] += (double)e0;
-          xv[2 * k + 1] += (double)e1;
+          xv[2 * k] += f64_of(e0);
+          xv[2 * k + 1] += f64_of(e1);
         }
         st8(x, xv);
       }
