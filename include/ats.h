@@ -176,18 +176,17 @@ typedef struct {
                      /* distributed shared memory; default), 1 = global      */
                      /* memory (L2).  The FP64 bulk always uses global.      */
   int res_cluster_big; /* resident solver: CTAs per cluster for the levels    */
-                     /* whose runs on res_cluster_mid CTAs would not fit     */
-                     /* their shared memory (ATS_PREC_FP64: would exceed     */
-                     /* 128 octs per CTA), or whose estimated work         */
+                     /* whose runs on res_cluster_mid CTAs would exceed the   */
+                     /* groups' limit (see res_max_octs; ATS_PREC_FP64: 128  */
+                     /* octs per CTA), or whose estimated work         */
                      /* exceeds res_big_work (0 = 16; < 0 = none)           */
   int res_big_work;  /* resident solver: a level of more than res_cta_octs   */
                      /* octs also takes the larger clusters when its        */
                      /* estimated work n_oct min(sqrt(1 + 8 h), 4 n_oct^(1/3)),*/
                      /* h = dt / (2 dx^2), exceeds this (0 = no work rule)   */
   int res_cluster_mid; /* resident solver: CTAs per cluster for the levels    */
-                     /* whose runs on res_cluster CTAs would not fit their   */
-                     /* shared memory (ATS_PREC_FP64: 128 octs per CTA)      */
-                     /* but whose runs on this many would     */
+                     /* whose runs on res_cluster CTAs would exceed the       */
+                     /* groups' limit but whose runs on this many would not   */
                      /* (0 = 8; < 0 = none: they take res_cluster_big);     */
                      /* used only between res_cluster and res_cluster_big   */
   int cg_form;       /* resident solver, mixed precision: how each CG step    */
@@ -212,14 +211,17 @@ typedef struct {
  *   certificate inside one persistent launch, on one thread-block cluster of
  *   res_cluster CTAs (per-step sums exchanged through distributed shared
  *   memory, steps ordered by the hardware cluster barrier); a level whose
- *   runs on res_cluster CTAs would not fit their shared memory takes the
- *   smallest of res_cluster_mid and res_cluster_big CTAs whose runs fit (or
+ *   runs on res_cluster CTAs would be longer than the groups' limit (1024 or
+ *   2048 octs, see res_max_octs; ATS_PREC_FP64: 128) takes the smallest of
+ *   res_cluster_mid and res_cluster_big CTAs whose runs are not (or
  *   res_cluster_big when its estimated work exceeds res_big_work, when
- *   set); a level of at most res_cta_octs octs runs on one CTA; clusters and CTAs take solves from work queues ordered
- *   by estimated work (largest first; after a completed run of a batch, by
- *   the measured durations); the cluster sizes and the single CTAs run as
- *   concurrent launches sharing the SMs in proportion to their queues'
- *   estimated work (after a completed run, their measured SM-time).  Not for the paper stopping rule (ATS_STOP_PAPER
+ *   set); a level of at most res_cta_octs octs runs on one CTA; clusters and
+ *   CTAs take solves from work queues ordered by estimated work (largest
+ *   first; after a completed run of a batch, by the measured durations); the
+ *   cluster sizes and the single CTAs run as
+ *   concurrent launches sharing the SMs in shares that let the class that ends
+ *   last end earliest, by their queues' estimated work (after a completed run,
+ *   their measured SM-time).  Not for the paper stopping rule (ATS_STOP_PAPER
  *   takes the tick path). */
 #define ATS_SCHED_AUTO 0     /* resident solver for levels up to res_max_octs octs; */
         /* above it the whole-GPU form (see ATS_SCHED_GRID): FP64 for every level,   */
