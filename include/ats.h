@@ -621,6 +621,16 @@ ats_status ats_bounds_violations(int device, long long *count);
  * ATS_ERR_INVALID_ARG (null outputs, negative counts, more CTAs than SMs),
  * ATS_ERR_CUDA (also when the flag disagrees with the waits). */
 ats_status ats_grid_barrier_selftest(int device, int ctas, int extra, int *n_normal, int *n_gave_up, double *ms);
+/* Self-test of that solver's sums over its CTAs (at most one per SM), in the
+ * order a CG step takes them: n rounds (at most 4096) of the p.q sum, which
+ * scales by a reference value, and of the sum that publishes z.  values:
+ * [n][ctas], the value each CTA adds; refs: [n].  totals: [n][2], the two sums
+ * rounded to FP32; buffers: [n], which of the two sets of partial sums (0, 1)
+ * the second sum used.  Host arrays.  Errors: ATS_ERR_INVALID_ARG (null
+ * arrays, counts out of range), ATS_ERR_CUDA (also when the CTAs' totals
+ * differ or a wait gave up). */
+ats_status ats_grid_sum_selftest(int device, int ctas, int n, const float *values, const float *refs, float *totals,
+                                 int *buffers);
 
 #ifdef __cplusplus
 }

@@ -187,6 +187,7 @@ _SIGS = [
     ("ats_bounds_violations", ctypes.c_int, [ctypes.c_int, ctypes.POINTER(ctypes.c_longlong)]),
     ("ats_grid_barrier_selftest", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
                                                  ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_double)]),
+    ("ats_grid_sum_selftest", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, P, P, P, P]),
 ]
 
 ATS_NOALLOC_MAX_CELLS = 262144
@@ -510,6 +511,19 @@ def ats_grid_barrier_selftest(device: int = 0, ctas: int = 0, extra: int = 0):
     _check(lib().ats_grid_barrier_selftest(device, ctas, extra, ctypes.byref(a), ctypes.byref(b), ctypes.byref(t)),
            "ats_grid_barrier_selftest")
     return {"normal": a.value, "gave_up": b.value, "ms": t.value}
+
+
+def ats_grid_sum_selftest(values, refs, device: int = 0):
+    """The whole-GPU solver's sums over its CTAs alone: values [n][CTAs], refs
+    [n].  Returns ([n][2] totals, [n] sets of partial sums used)."""
+    v = np.ascontiguousarray(values, np.float32)
+    r = np.ascontiguousarray(refs, np.float32)
+    if v.ndim != 2 or r.shape != v.shape[:1]:
+        raise ValueError("values [n][CTAs] and refs [n]")
+    tot, buf = np.zeros((len(v), 2), np.float32), np.zeros(len(v), np.int32)
+    _check(lib().ats_grid_sum_selftest(device, v.shape[1], len(v), v.ctypes.data, r.ctypes.data, tot.ctypes.data,
+                                       buf.ctypes.data), "ats_grid_sum_selftest")
+    return tot, buf
 
 
 def ats_bounds_violations(device: int = 0) -> int:

@@ -275,6 +275,10 @@ int resident_run_cap();
 // threads) waiting for a.g_expect arrivals: out[cta] = 1 when its wait ended
 // normally, 0 when it gave up (and *a.gerr = 1).  a.gbar, a.gerr zeroed first.
 cudaError_t launch_grid_barrier_probe(int grid, const ResArgs &a, int *out, cudaStream_t st);
+// n rounds of that form's two sums alone (cooperative launch of `grid` CTAs);
+// a.gbar (kGridBarWords words) zeroed first, a.gpart as for a solve.
+cudaError_t launch_grid_sum_probe(int grid, const ResArgs &a, int n, const float *value, const float *ref,
+                                  float *total, int *slot, cudaStream_t st);
 
 // Start of a solve: e = 0 on every cell of every item, and x64 = src[solve]
 // where src (device array of device pointers) is non-null for that solve.

@@ -2698,8 +2698,10 @@ __device__ bool grid_sync(const ResArgs &a, int *flag) {
 // in rank order -- lane j takes ranks j, j + 32, ..., every load issued before
 // the merges -- with a butterfly, so all CTAs hold bitwise the same totals.
 // Every thread ends with them in `out`, and with false when the CTA's wait
-// gave up.  The slots alternate between two buffers: a buffer is written
-// again only two sums later, after a barrier that every reader has passed.
+// gave up.  `buf`: bit 0 alternates the CTA's own arrays (as in group_sum), bit
+// 1 the slots.  Bit 1 turns here alone: a slot buffer is written again only two
+// of these sums later, after a barrier (release and acquire) that every reader
+// of its previous contents has passed.
 // `work`: what each thread does between its arrival and its wait; `after`:
 // what the other warps do, once the barrier is complete, while warp 0 merges.
 constexpr int kGridMaxPerLane = 8;  // up to 256 CTAs in the launch
@@ -2708,15 +2710,16 @@ __device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, i
                          const Work &work, const After &after) {
   constexpr bool kAfter = !std::is_same<After, NoWork>::value;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  warps_to_red<T, NA>(a, sh.red[buf]);
+  const int cb = buf & 1;
+  warps_to_red<T, NA>(a, sh.red[cb]);
   __syncthreads();
   if (warp == 0) {
     const unsigned G = gridDim.x;
-    double *slots = ra.gpart + (size_t)buf * (G + 1) * 3;  // [G] CTA slots of 3 sums (FP32 bulk: (hi, lo) pairs)
+    double *slots = ra.gpart + (size_t)(buf >> 1) * (G + 1) * 3;  // [G] CTA slots of 3 sums (FP32 bulk: (hi, lo) pairs)
 #pragma unroll
     for (int k = 0; k < NA; k += 2) {
       const int k2 = k + 1 < NA ? k + 1 : k;
-      const Acc<T> m = merge_entries<T>(sh.red[buf], nw, k, k2);
+      const Acc<T> m = merge_entries<T>(sh.red[cb], nw, k, k2);
       if (lane == 0) Slot<T>::store(slots + blockIdx.x * 3 + k, m);
       if (k2 > k && lane == 16) Slot<T>::store(slots + blockIdx.x * 3 + k2, m);
     }
@@ -2738,7 +2741,7 @@ __device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, i
 #pragma unroll
         for (int i = 0; i < kGridMaxPerLane; ++i) t.merge(v[i]);
         lanes_total<16>(t);
-        if (lane == 0) sh.inbox[buf][0][k] = t;
+        if (lane == 0) sh.inbox[cb][0][k] = t;
       }
     }
   } else {
@@ -2751,8 +2754,8 @@ __device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, i
   __syncthreads();
   const bool ok = sh.task != 0;
 #pragma unroll
-  for (int k = 0; k < NA; ++k) out[k] = sh.inbox[buf][0][k];
-  buf ^= 1;
+  for (int k = 0; k < NA; ++k) out[k] = sh.inbox[cb][0][k];
+  buf ^= 3;
   return ok;
 }
 
@@ -2761,10 +2764,12 @@ __device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, i
 // every CTA adds its total as a fixed-point number to two 64-bit words whose
 // low ten bits count the CTAs, and polls them until the count is complete.
 // Integer additions commute, so every CTA reads the same bits whatever the
-// order.  The words only grow (fx_old: their last complete values), two sets
-// used in turn as the sums' other buffers.  Nothing else is published by this
-// sum, so no fence is needed (each costs 0.6 us): only a sum that makes z
-// visible keeps the barrier.  Measured alone on 152 CTAs: 1.81 -> 1.13 us.
+// order.  The words only grow (fx_old: their last complete values).  Nothing is
+// published by this sum, so it has no fence (each costs 0.6 us) and orders no
+// other memory: only a sum that makes z visible keeps the barrier, and such a
+// barrier lies between any two of these sums on the same words.  So this sum
+// turns the CTA's own arrays (bit 0 of `buf`) and leaves the slots of
+// grid_sum (bit 1) alone.  Measured alone on 152 CTAs: 1.81 -> 1.13 us.
 // Fixed point: `ref`, a positive value every CTA holds (the current r.z), is
 // scaled into [2^24, 2^25); the first word sums the integer part (up to 2^44 per CTA),
 // the second the fraction in units of 2^-35 (offset by 2^36 to stay positive):
@@ -2782,16 +2787,17 @@ __device__ bool grid_sum_fx(Acc<float> (&a)[1], ResShared<float> &sh, const ResA
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const bool fx = ref > 1e-37f && ref < 1e37f;  // the same in every CTA
   if (fx) {
+    const int cb = buf & 1;
     Acc<float> t[1] = {a[0]};
-    warps_to_red<float, 1>(t, sh.red[buf]);
+    warps_to_red<float, 1>(t, sh.red[cb]);
     __syncthreads();
     if (warp == 0) {
-      const Acc<float> m = merge_entries<float>(sh.red[buf], nw, 0, 0);
+      const Acc<float> m = merge_entries<float>(sh.red[cb], nw, 0, 0);
       const int E = 24 - ((int)(__float_as_uint(ref) >> 23) - 127), e1 = E / 2, e2 = E - e1;
       const float fs = m.s * pow2f(e1) * pow2f(e2), fc = m.c * pow2f(e1) * pow2f(e2);
       const unsigned long long G = gridDim.x;
       unsigned long long *word =
-          reinterpret_cast<unsigned long long *>(ra.gbar + kFxWord * (1 + 2 * buf + (lane & 1)));
+          reinterpret_cast<unsigned long long *>(ra.gbar + kFxWord * (1 + 2 * cb + (lane & 1)));
       if (lane < 2) {
         unsigned long long v = lane == 0 ? 0ull : 1ull << 45;
         if (fabsf(fs) < pow2f(44) && fabsf(fc) < pow2f(44)) {
@@ -2802,7 +2808,7 @@ __device__ bool grid_sum_fx(Acc<float> (&a)[1], ResShared<float> &sh, const ResA
         }
         asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"((v << 10) + 1ull) : "memory");
       }
-      const unsigned long long old = sh.fx_old[buf][lane & 1];
+      const unsigned long long old = sh.fx_old[cb][lane & 1];
       unsigned long long d = 0;
       unsigned ns = 16;
       bool ok = true;
@@ -2820,7 +2826,7 @@ __device__ bool grid_sum_fx(Acc<float> (&a)[1], ResShared<float> &sh, const ResA
         __nanosleep(ns);
         if (ns < 64) ns <<= 1;
       }
-      if (lane < 2) sh.fx_old[buf][lane] = old + d;
+      if (lane < 2) sh.fx_old[cb][lane] = old + d;
       const unsigned long long w1 = __shfl_sync(kFull, d, 1) >> 10;
       if (lane == 0) {
         const long long hi = (long long)d >> 10, lo = (long long)w1 - (long long)(G << 36);
@@ -2828,13 +2834,13 @@ __device__ bool grid_sum_fx(Acc<float> (&a)[1], ResShared<float> &sh, const ResA
         const float c = __fadd_rn(__ll2float_rn(hi - __float2ll_rn(f)), __fmul_rn(__ll2float_rn(lo), pow2f(-35)));
         Acc<float> r;
         r.s = __fadd_rn(f, c) * pow2f(-e1) * pow2f(-e2);
-        sh.inbox[buf][0][0] = r;
+        sh.inbox[cb][0][0] = r;
         sh.task = !ok ? 0 : (w1 >> 45) != 0 ? 2 : 1;
       }
     }
     __syncthreads();
     const int got = sh.task;
-    out = sh.inbox[buf][0][0].s;
+    out = sh.inbox[cb][0][0].s;
     buf ^= 1;
     if (got != 2) return got == 1;
     __syncthreads();  // the flag is read before the sum below writes it
@@ -4681,6 +4687,51 @@ cudaError_t launch_grid_barrier_probe(int grid, const ResArgs &a, int *out, cuda
   return cudaLaunchKernelEx(&cfg, k_grid_barrier_probe, a, out);
 }
 
+// Sums of the whole-GPU form in the order a CG step takes them: per round the
+// fixed-point sum of one value per CTA, scaled by ref[i], then the slot sum of
+// the same values.  total: [n][CTAs][2], slot: [n][CTAs], the slot buffer that
+// the second sum used.
+__global__ void __launch_bounds__(512, 1)
+    k_grid_sum_probe(ResArgs a, int n, const float *__restrict__ value, const float *__restrict__ ref, float *total,
+                     int *slot) {
+  __shared__ ResShared<float> sh;
+  if (threadIdx.x < 4) sh.fx_old[threadIdx.x >> 1][threadIdx.x & 1] = 0;
+  __syncthreads();
+  int buf = 0;
+  for (int i = 0; i < n; ++i) {
+    const size_t at = (size_t)i * gridDim.x + blockIdx.x;
+    Acc<float> v[1], w[1], tot[1];
+    if (threadIdx.x == 0) {
+      v[0].add_value(value[at]);
+      w[0] = v[0];
+    }
+    float t;
+    if (!grid_sum_fx(v, sh, a, buf, ref[i], t)) break;
+    const int sb = buf >> 1;
+    if (!grid_sum<float, 1>(w, sh, a, buf, tot, NoWork(), NoWork())) break;
+    if (threadIdx.x == 0) {
+      total[2 * at] = t;
+      total[2 * at + 1] = tot[0].val();
+      slot[at] = sb;
+    }
+  }
+}
+
+cudaError_t launch_grid_sum_probe(int grid, const ResArgs &a, int n, const float *value, const float *ref,
+                                  float *total, int *slot, cudaStream_t st) {
+  if (grid <= 0 || grid > 32 * kGridMaxPerLane || !a.gbar || !a.gpart || !a.gerr) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(512);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_grid_sum_probe, a, n, value, ref, total, slot);
+}
+
 cudaError_t launch_resident(int threads, int cluster, int grid, const ResArgs &a, cudaStream_t st, bool cta_only) {
   if (a.n_cq + a.n_tq <= 0) return cudaSuccess;
   if (cluster < 1 || cluster > kMaxCluster || grid <= 0) return cudaErrorInvalidValue;
@@ -4786,4 +4837,72 @@ extern "C" ats_status ats_grid_barrier_selftest(int device, int ctas, int extra,
   *ms = (double)t;
   // every wait that gave up must have raised the flag
   return (gave_up > 0) == (flag != 0) ? ATS_OK : ATS_ERR_CUDA;
+}
+
+// The sums of the whole-GPU solver alone, on chosen values (see
+// k_grid_sum_probe).  Every CTA must end with the same bits.
+extern "C" ats_status ats_grid_sum_selftest(int device, int ctas, int n, const float *values, const float *refs,
+                                            float *totals, int *buffers) {
+  if (ctas < 1 || n < 1 || n > 4096 || !values || !refs || !totals || !buffers) return ATS_ERR_INVALID_ARG;
+  int sms = 0;
+  if (cudaSetDevice(device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    cudaGetLastError();
+    return ATS_ERR_CUDA;
+  }
+  if (ctas > sms) return ATS_ERR_INVALID_ARG;
+  const size_t m = (size_t)n * ctas;
+  const size_t b_bar = sizeof(unsigned) * ats::kGridBarWords, b_part = 6 * sizeof(double) * ((size_t)ctas + 1);
+  unsigned *bar = nullptr;
+  double *part = nullptr;
+  float *val = nullptr, *ref = nullptr, *tot = nullptr;
+  int *slot = nullptr;
+  cudaStream_t st = nullptr;
+  cudaError_t err = cudaMalloc(&bar, b_bar);
+  if (err == cudaSuccess) err = cudaMalloc(&part, b_part);
+  if (err == cudaSuccess) err = cudaMalloc(&val, sizeof(float) * m);
+  if (err == cudaSuccess) err = cudaMalloc(&ref, sizeof(float) * n);
+  if (err == cudaSuccess) err = cudaMalloc(&tot, 2 * sizeof(float) * m);
+  if (err == cudaSuccess) err = cudaMalloc(&slot, sizeof(int) * m);
+  if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (err == cudaSuccess) err = cudaMemsetAsync(bar, 0, b_bar, st);
+  if (err == cudaSuccess) err = cudaMemsetAsync(slot, 0xFF, sizeof(int) * m, st);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(val, values, sizeof(float) * m, cudaMemcpyHostToDevice, st);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(ref, refs, sizeof(float) * n, cudaMemcpyHostToDevice, st);
+  ats::ResArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.gbar = bar;
+  a.gerr = (int *)(bar + 2);
+  a.gpart = part;
+  if (err == cudaSuccess) err = ats::launch_grid_sum_probe(ctas, a, n, val, ref, tot, slot, st);
+  std::vector<float> h(2 * m);
+  std::vector<int> hs(m);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(h.data(), tot, 2 * sizeof(float) * m, cudaMemcpyDeviceToHost, st);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(hs.data(), slot, sizeof(int) * m, cudaMemcpyDeviceToHost, st);
+  if (st) {
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (err == cudaSuccess) err = e;
+    cudaStreamDestroy(st);
+  }
+  cudaFree(bar);
+  cudaFree(part);
+  cudaFree(val);
+  cudaFree(ref);
+  cudaFree(tot);
+  cudaFree(slot);
+  if (err != cudaSuccess) {
+    cudaGetLastError();
+    return ATS_ERR_CUDA;
+  }
+  bool same = true;
+  for (int i = 0; i < n; ++i) {
+    const float *row = h.data() + 2 * (size_t)i * ctas;
+    const int *srow = hs.data() + (size_t)i * ctas;
+    for (int c = 0; c < ctas; ++c)
+      same = same && std::memcmp(row + 2 * c, row, 2 * sizeof(float)) == 0 && srow[c] == srow[0] && srow[c] >= 0;
+    totals[2 * i] = row[0];
+    totals[2 * i + 1] = row[1];
+    buffers[i] = srow[0];
+  }
+  return same ? ATS_OK : ATS_ERR_CUDA;
 }

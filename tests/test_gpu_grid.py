@@ -19,6 +19,8 @@ kind split over more CTAs than octs (idle CTAs in every barrier and sum),
 bitwise equality alone / in a batch / run to run, a batch mixing every
 resident form, and the barrier's bounded wait.
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -204,3 +206,46 @@ def test_grid_barrier_waits_are_bounded(ats):
     assert 1.0 < bad["ms"] < 5000.0
     again = ats.ats_grid_barrier_selftest(0, 0, 0)
     assert again["gave_up"] == 0
+
+
+@pytest.mark.parametrize("ctas", [1, 3, 0])
+def test_sums_over_the_launch(ats, ctas):
+    """The whole-GPU solver's two sums on chosen values: both within FP32
+    rounding of the exact total (the p.q sum also within its quantum of 2^-60
+    of the reference value per CTA), the p.q sum by its slow way where the
+    reference or a value is out of range, and each slot sum on the other set
+    of partial sums than the one before it -- also with p.q sums between them
+    -- so that a barrier lies between reading a set and writing it again."""
+    import torch
+
+    ctas = ctas or torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(ctas)
+    values, refs, slow = [], [], []
+    for i in range(96):
+        v = (rng.standard_normal(ctas) * 10.0 ** rng.integers(-3, 4)).astype(np.float32)
+        ref, far = np.float32(abs(v).max() * 2.0 ** rng.integers(-12, 20)), False
+        if i % 8 == 5:  # the reference out of range
+            small = i % 16 == 5
+            v, ref, far = v * np.float32(1e-38 if small else 1e33), np.float32(1e-38 if small else 2e37), True
+        elif i % 8 == 6:  # one CTA's value beyond 2^20 of it
+            ref, far = np.float32(abs(v).max() * 2.0 ** -21), True
+        elif i % 8 == 7:
+            v = abs(v)
+        values.append(v)
+        refs.append(ref)
+        slow.append(far)
+    tot, buf = ats.ats_grid_sum_selftest(values, refs)
+    pos = 0
+    for v, ref, far, (fx, plain), b in zip(values, refs, slow, tot, buf):
+        exact = math.fsum(v.tolist())
+        rnd = 1.01 * 2.0 ** -24 * abs(exact) + 2.0 ** -149  # (one rounding to FP32, subnormals included)
+        # pairs merged over at most 13 levels, each level's errors at most 2^-24 of sum |v| and rounded to 2^-24 of
+        # what has gathered: 2 * 13^2 * 2^-48 sum |v|
+        assert abs(float(plain) - exact) <= rnd + ctas * 2.0 ** -39 * float(abs(v).max())
+        if far:
+            assert fx.tobytes() == plain.tobytes()
+        else:
+            assert abs(float(fx) - exact) <= rnd + ctas * 2.0 ** -60 * float(ref)
+        pos ^= int(far)
+        assert b == pos
+        pos ^= 1
