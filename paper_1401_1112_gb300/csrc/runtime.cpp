@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "ats_internal.h"
+#include "host_range.h"
 
 namespace ats {
 
@@ -251,11 +252,8 @@ struct Plan {
   std::vector<const double *> h_src;
   std::vector<double *> h_dst, h_rdst;
   bool any_dst = false;  // k_final has a result to write
-  // host-memory solves: the last host x pointers seen, whether the device
-  // can write each directly (pinned), and the pointers copy_runs copies back
-  // (null where the resident kernel wrote the host array itself)
-  std::vector<double *> h_xhost, h_xdev;
-  std::vector<char> h_xdirect;
+  // host-memory solves: the pointers copy_runs copies back (null where the
+  // resident kernel wrote the host array itself)
   std::vector<double *> h_copyback;
   bool profiling = false;
   // two sets (by poll slot) of: chunk start, then kTickEvents per tick of a
@@ -1375,23 +1373,15 @@ ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off
   // x directly when the device can write it (pinned), else into the staging
   // buffer -- and k_final writes the others; copy_runs brings back the staged
   // host results
-  if (!dev) {
-    std::vector<double *> hx(x_inout, x_inout + n);
-    if (hx != P->h_xhost) {
-      P->h_xhost = hx;
-      P->h_xdev.assign(n, nullptr);
-      P->h_xdirect.assign(n, 0);
-      for (int k = 0; k < n; ++k) {
-        cudaPointerAttributes pa;
-        if (cudaPointerGetAttributes(&pa, hx[k]) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
-            pa.devicePointer) {
-          P->h_xdev[k] = (double *)pa.devicePointer;
-          P->h_xdirect[k] = 1;
-        }
-        cudaGetLastError();
-      }
-    }
-  }
+  std::vector<double *> xdev(n, nullptr);
+  if (!dev && P->res_smem)
+    host_targets(x_inout, n, xdev.data(), [](double *p, void **d) {
+      cudaPointerAttributes pa = {};
+      const bool ok = cudaPointerGetAttributes(&pa, p) == cudaSuccess;
+      cudaGetLastError();
+      *d = pa.devicePointer;
+      return ok && pa.type == cudaMemoryTypeHost && pa.devicePointer;
+    });
   std::vector<double *> rdst(n, nullptr);
   P->h_copyback.assign(n, nullptr);
   for (int k = 0; k < n; ++k) {
@@ -1399,9 +1389,9 @@ ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off
     src[k] = x0_e ? P->levels[k]->E_dev : stage;
     const int m = P->mode[k];
     const bool res_out = P->res_smem && (m == 1 || m == 2 || m == 3 || m == 5);
-    const bool direct = !dev && res_out && P->h_xdirect[k];
+    const bool direct = !dev && res_out && xdev[k];
     dst[k] = res_out ? nullptr : stage;
-    rdst[k] = res_out ? (direct ? P->h_xdev[k] : stage) : nullptr;
+    rdst[k] = res_out ? (direct ? xdev[k] : stage) : nullptr;
     if (!dev && !direct) P->h_copyback[k] = x_inout[k];
   }
   if (src != P->h_src || dst != P->h_dst || rdst != P->h_rdst) {
