@@ -1,5 +1,6 @@
 // Host runtime of the level-solve library: context, levels, operator build,
 // solve plans (single and batched), CUDA-graph replay and convergence polling.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -385,6 +386,38 @@ int choose_tile(int64_t n_oct, int requested, int grid) {
   const int64_t per_cta = (n_oct + g - 1) / g;
   const int64_t t = (per_cta + 127) / 128 * 128;
   return (int)std::min<int64_t>(8 * kThreads, std::max<int64_t>(2 * kThreads, t));
+}
+
+// The pinned host memory around p that the device can write (managed memory is
+// not: its pages move).  The runtime tells whether p is pinned, only the driver
+// how far the allocation or registration reaches.
+HostRange pinned_range(const void *p) {
+  using Fn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+  static const Fn fn = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (Fn)f;
+  }();
+  unsigned type = 0, managed = 0;
+  CUdeviceptr dev = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute at[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                               CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                               CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void *out[5] = {&type, &managed, &dev, &start, &size};
+  HostRange r;
+  if (!fn || fn(5, at, out, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed ||
+      !dev || !start || start > (uintptr_t)p)
+    return r;
+  r.lo = start;
+  r.hi = start + size;
+  r.dev = dev - ((uintptr_t)p - start);
+  return r;
 }
 
 // Copy per-level host arrays into (h2d) or out of one device buffer at the
@@ -1374,14 +1407,11 @@ ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off
   // buffer -- and k_final writes the others; copy_runs brings back the staged
   // host results
   std::vector<double *> xdev(n, nullptr);
-  if (!dev && P->res_smem)
-    host_targets(x_inout, n, xdev.data(), [](double *p, void **d) {
-      cudaPointerAttributes pa = {};
-      const bool ok = cudaPointerGetAttributes(&pa, p) == cudaSuccess;
-      cudaGetLastError();
-      *d = pa.devicePointer;
-      return ok && pa.type == cudaMemoryTypeHost && pa.devicePointer;
-    });
+  if (!dev && P->res_smem) {
+    std::vector<size_t> len(n);
+    for (int k = 0; k < n; ++k) len[k] = (size_t)P->levels[k]->N;
+    host_targets(x_inout, len.data(), n, xdev.data(), pinned_range);
+  }
   std::vector<double *> rdst(n, nullptr);
   P->h_copyback.assign(n, nullptr);
   for (int k = 0; k < n; ++k) {
