@@ -142,24 +142,6 @@ ats_status dev_alloc_t(ats_context *ctx, size_t count, P **out) {
   return s;
 }
 
-// A few kilobytes of barrier and partial-sum words that a plan did not always
-// have: kept out of the context's budget, so that a solve that used to fit it
-// still does.
-template <typename P>
-ats_status dev_alloc_uncounted(ats_context *ctx, size_t bytes, P **out) {
-  void *p = nullptr;
-  const cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    set_error(std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
-    return ATS_ERR_OOM;
-  }
-  ctx->allocs[p] = 0;
-  ++ctx->epoch;
-  *out = (P *)p;
-  return ATS_OK;
-}
-
 void dev_free(ats_context *ctx, void *p) {
   if (!p) return;
   ++ctx->epoch;
@@ -915,8 +897,8 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
       (s = dev_alloc_t(ctx, 1, &P->d_active)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 2 * kCellCounters, &P->d_cells)) != ATS_OK ||
       (s = dev_alloc_t(ctx, std::max(1, P->n_bq + P->n_mq + P->n_cq + P->n_tq + P->n_gq), &P->d_queue)) != ATS_OK ||
-      (P->n_gq > 0 && (s = dev_alloc_uncounted(ctx, sizeof(unsigned) * kGridBarWords, &P->d_gbar)) != ATS_OK) ||
-      (P->n_gq > 0 && (s = dev_alloc_uncounted(ctx, 6 * sizeof(double) * lock * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_t(ctx, kGridBarWords, &P->d_gbar)) != ATS_OK) ||
+      (P->n_gq > 0 && (s = dev_alloc_t(ctx, 6 * lock * ((size_t)P->res_grid_all + 1), &P->d_gpart)) != ATS_OK) ||
       (s = dev_alloc_t(ctx, 4, &P->d_heads)) != ATS_OK ||
       (s = dev_alloc_t(ctx, 4 * (size_t)P->n_items, &P->d_lists)) != ATS_OK ||
       (s = dev_alloc_t(ctx, (size_t)P->n_items, &P->d_ident)) != ATS_OK ||
