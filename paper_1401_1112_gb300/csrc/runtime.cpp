@@ -15,6 +15,7 @@
 
 #include "ats_internal.h"
 #include "host_range.h"
+#include "split.h"
 
 namespace ats {
 
@@ -557,47 +558,19 @@ ats_status plan_upload_queues(Plan *P) {
 // The CTA slots of the device, shared by the resident launches by their
 // queues' work w[0] (big clusters), w[1] (middle clusters), w[2] (clusters),
 // w[3] (single CTAs) in SM-time, and by the longest solve's work in each,
-// longest[]: the counts of clusters that make the class that ends last end
-// earliest (each class ends after its work over its slots, and not before its
-// longest solve), out of every combination that fits.  The single CTAs get
-// their share first (so the largest of them start at once) and every slot
-// left over; a cluster that has emptied its queue goes on with single-CTA
-// solves.  Rounding each class's share to whole clusters, largest first, left
-// the smallest clusters 16 of 152 SMs on a batch of 512 levels: they ended
-// after 27.1 ms, the other classes after 14.4 and 11.6 ms (measured).
+// longest[] (see split.h).
 void plan_split(Plan *P, const double (&w)[4], const double (&longest)[4]) {
   const int slots = P->res_slots;
   const int size[3] = {P->res_cluster_big, P->res_cluster_mid, P->res_cluster};
-  const int lim[3] = {P->res_clA, P->res_clM, P->res_clB};
-  const int cnt[3] = {P->n_bq, P->n_mq, P->n_cq};
-  const double wsum = std::max(1e-300, w[0] + w[1] + w[2] + w[3]);
-  const int c_min = P->n_tq > 0 ? std::max(1, (int)std::ceil(slots * w[3] / wsum)) : 0;
-  int lo[3], hi[3], k[3] = {0, 0, 0};
-  for (int q = 0; q < 3; ++q) {
-    lo[q] = cnt[q] > 0 ? 1 : 0;
-    hi[q] = cnt[q] > 0 ? std::max(1, std::min(lim[q], cnt[q])) : 0;
-    k[q] = lo[q];
-  }
-  const auto end_of = [&](int q, int n) {
-    return cnt[q] > 0 ? std::max(w[q] / ((double)n * size[q]), longest[q] / size[q]) : 0.0;
-  };
-  // (the first combination stands when not even one cluster of each class fits)
-  double best = HUGE_VAL;
-  int best_used = 0;
-  for (int i = lo[0]; i <= hi[0]; ++i)
-    for (int j = lo[1]; j <= hi[1]; ++j)
-      for (int l = lo[2]; l <= hi[2]; ++l) {
-        const int used = i * size[0] + j * size[1] + l * size[2];
-        if (used + c_min > slots) break;
-        const double t = std::max(end_of(0, i), std::max(end_of(1, j), end_of(2, l)));
-        if (t < best || (t == best && used < best_used)) {
-          best = t;
-          best_used = used;
-          k[0] = i;
-          k[1] = j;
-          k[2] = l;
-        }
-      }
+  const SplitIn in = {slots,
+                      {size[0], size[1], size[2]},
+                      {P->res_clA, P->res_clM, P->res_clB},
+                      {P->n_bq, P->n_mq, P->n_cq},
+                      {w[0], w[1], w[2], w[3]},
+                      {longest[0], longest[1], longest[2]},
+                      P->n_tq};
+  int k[3];
+  split_clusters(in, k);
   P->res_grid_big = k[0] * size[0];
   P->res_grid_mid = k[1] * size[1];
   const bool clusters = P->n_bq + P->n_mq + P->n_cq > 0;
