@@ -155,17 +155,15 @@ typedef struct {
   int res_cluster;   /* resident solver: CTAs per thread-block cluster, 1..16 */
                      /* (0 = 4)                                              */
   int res_cta_octs;  /* resident solver: a level of at most this many octs is */
-                     /* solved by one CTA alone (0 = 1024 for ATS_PREC_MIXED, */
-                     /* 2048 when res_max_octs is given, 128 for              */
-                     /* ATS_PREC_FP64; < 0 = never)                          */
+                     /* solved by one CTA alone (0 = 2048 for ATS_PREC_MIXED, */
+                     /* 128 for ATS_PREC_FP64; < 0 = never)                  */
   int res_max_octs;  /* ATS_SCHED_AUTO: levels above this many octs take the  */
                      /* whole-GPU form or the tick path (see ATS_SCHED_AUTO) */
                      /* (0 = 16384 for ATS_PREC_MIXED, 2048 for              */
-                     /* ATS_PREC_FP64).  Mixed precision: 0 here and in       */
-                     /* res_cta_octs sizes the groups for the shortest solve  */
-                     /* (at most 1024 octs per CTA where a cluster size       */
-                     /* allows it); a limit given in either sizes them for    */
-                     /* the most solves per SM (2048 octs per CTA)            */
+                     /* ATS_PREC_FP64).  Mixed precision: also the limit of a */
+                     /* cluster's octs per CTA, 1536 (a larger cluster is     */
+                     /* taken above it, which solves a lone level sooner), or */
+                     /* 2048 (the most solves per SM) when more than 16384    */
   int cg_scalars;    /* resident solver, mixed precision: the CG step's alpha,  */
                      /* beta and inner convergence test from the error-free   */
                      /* dot totals, 0 = rounded to FP32 (the tick path's form, */
@@ -211,7 +209,7 @@ typedef struct {
  *   certificate inside one persistent launch, on one thread-block cluster of
  *   res_cluster CTAs (per-step sums exchanged through distributed shared
  *   memory, steps ordered by the hardware cluster barrier); a level whose
- *   runs on res_cluster CTAs would be longer than the groups' limit (1024 or
+ *   runs on res_cluster CTAs would be longer than the groups' limit (1536 or
  *   2048 octs, see res_max_octs; ATS_PREC_FP64: 128) takes the smallest of
  *   res_cluster_mid and res_cluster_big CTAs whose runs are not (or
  *   res_cluster_big when its estimated work exceeds res_big_work, when

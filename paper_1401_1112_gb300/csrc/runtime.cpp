@@ -617,14 +617,29 @@ void plan_adapt_split(Plan *P, const unsigned long long *ts) {
 // that allows (128 levels of 64 .. 2 048 octs 2.67 ms; with runs of 64 octs
 // 3.02 ms, one level of 512 octs alone 7.4 instead of 9.8 us per iteration).
 constexpr int64_t kRun64 = 128;
-// FP32-bulk resident groups with the default limits: runs of up to 1 024 octs
-// (the register layout that keeps every private array on chip).  A step's
-// sums cost 2 to 3 us whatever the run, so the longest runs give the most
-// solves per SM and the shorter ones the shorter solve: 5 832 octs take 1.75
-// ms on 8 CTAs and 2.61 ms on 4 (7.6 and 5.7 SM-ns per oct and iteration);
-// 512 levels of 64 .. 32 768 octs take 13.9 ms with runs of up to 2 048 and
-// 16.4 ms with the shorter ones (measured).
-constexpr int64_t kRunLatency = 1024;
+// FP32-bulk resident groups: octs per CTA up to which the next smaller cluster
+// is taken (one CTA alone: kCta32).  A step's sums cost 2 to 3 us whatever the
+// run, so long runs give the most solves per SM and short ones the shortest
+// solve; one rule serves a level alone and a full batch, because the order of
+// a level's sums follows its group.  Where the line lies, ms with the smaller
+// and the larger group:
+//   octs           one level alone        a full GPU (levels)
+//   1 100  1 / 4   0.93 / 0.58       (456) 1.96 / 3.48
+//   2 000  1 / 4   1.50 / 0.74       (456) 2.78 / 4.42
+//   5 832  4 / 8   1.66 / 1.09       (152) 3.18 / 4.63
+//   6 783  4 / 8   2.05 / 1.15       (152) 3.80 / 4.92
+//   8 400  8 / 16  1.59 / 1.10        (76) 4.13 / 5.74
+//   12 000 8 / 16  1.85 / 1.14        (76) 3.80 / 4.73
+// Runs above 1 536 octs are where the larger cluster costs a full GPU no more
+// than the shared-memory form did on the smaller one (5 832 octs 4.28, 6 200
+// octs 5.35 against 5.08 on 8 CTAs); below it the larger group would buy the
+// lone level's time with the batch's.
+constexpr int64_t kRun32 = 1536;
+constexpr int64_t kCta32 = 2048;
+// res_max_octs above its default keeps larger levels, hence batches that fill
+// the GPU, on the clusters: the longest runs that stay on chip (512 levels of
+// 64 .. 32 768 octs 9.1 ms, with runs of 1 536 octs 10.3 ms).
+constexpr int64_t kMaxOcts32 = 16384;
 // FP32-bulk levels take the whole-GPU form up to this many octs per CTA: the
 // first 2 048 of a run stay on chip, the rest is streamed from L2 and HBM,
 // where the tick path's larger grid does better once HBM bounds it (measured
@@ -751,7 +766,7 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     // FP64 (the global-memory form) 2048
     const int64_t max_octs = o.sched == ATS_SCHED_RESIDENT
                                  ? INT64_MAX
-                                 : (o.res_max_octs > 0 ? o.res_max_octs : (P->fp64 ? 2048 : 16384));
+                                 : (o.res_max_octs > 0 ? o.res_max_octs : (P->fp64 ? 2048 : kMaxOcts32));
     const double big_work = o.res_big_work > 0 ? (double)o.res_big_work : HUGE_VAL;  // 0: no work rule
     // FP32 bulk: the shared-memory kernel, its CG state in shared memory
     // (res_state 0, where the device has room) or in global memory (cap 0);
@@ -776,14 +791,11 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     const bool grid_regs = o.cg_form != 1 && !o.cg_scalars;
     const int64_t grid_auto_octs =
         P->fp64 ? INT64_MAX : grid_all * (grid_regs ? kRunTail : std::min(P->res_cap, resident_six_cap()));
-    // octs per CTA up to which a smaller group is taken: FP64 kRun64; FP32 bulk
-    // with the default limits kRunLatency, with a limit given what fits the
-    // CTA (see res_max_octs)
-    const bool throughput = o.res_max_octs > 0 || o.res_cta_octs > 0;
-    // (the same groups wherever the state is kept, so that the results are the same)
+    // octs per CTA up to which a smaller group is taken (the same groups
+    // wherever the state is kept, so that the results are the same)
     const int64_t fit = P->res_smem ? std::max(0, resident_smem_cap(P->res_threads, ctx->device)) : 0;
-    const int64_t run = P->fp64 ? kRun64 : throughput ? fit : std::min<int64_t>(kRunLatency, fit);
-    const int64_t cta_octs = o.res_cta_octs != 0 ? o.res_cta_octs : P->fp64 ? kRun64 : throughput ? 2048 : kRunLatency;
+    const int64_t run = P->fp64 ? kRun64 : std::min(o.res_max_octs > kMaxOcts32 ? fit : kRun32, fit);
+    const int64_t cta_octs = o.res_cta_octs != 0 ? o.res_cta_octs : P->fp64 ? kRun64 : kCta32;
     P->mode.assign(n, 0);
     for (int k = 0; k < n; ++k) {
       const int64_t no = P->levels[k]->n_oct;
