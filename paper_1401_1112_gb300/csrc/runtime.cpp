@@ -2658,7 +2658,8 @@ ats_status ats_batch_autotune(ats_batch *B, double *const *x_inout, const int *t
         static const int kShapes[][4] = {{512, 4, 2048, 16}, {512, 8, 2048, 16}, {512, 8, 2048, -1},
                                          {256, 4, 2048, 16}, {512, 4, 1024, 16}, {512, 2, 2048, 16},
                                          {512, 4, 2048, 8}, {512, 16, 2048, -1}};
-        const int base_cta = base.res_cta_octs ? base.res_cta_octs : 2048;
+        // (the batch's own shape, timed above, is left out)
+        const int base_cta = base.res_cta_octs ? base.res_cta_octs : (int)(P->fp64 ? kRun64 : kCta32);
         const int base_big = P->res_cluster_big > 0 ? P->res_cluster_big : -1;
         for (const auto &sh : kShapes) {
           if (sh[0] == P->res_threads && sh[1] == P->res_cluster && sh[2] == base_cta && sh[3] == base_big) continue;

@@ -75,3 +75,26 @@ def test_same_bits_with_the_state_in_global_memory(ats, ctx, dims, kw):
     y, h = _run(ats, ctx, dims, res_state=1, **kw)
     assert g == h
     np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("prec,limit,shapes", [("mixed", 0, 8), ("mixed", 1024, 8), ("mixed", 512, 9), ("fp64", 0, 9),
+                                               ("fp64", 2048, 8)])
+def test_autotuner_leaves_out_the_batchs_own_shape_alone(ats, ctx, prec, limit, shapes):
+    """Eight resident shapes and the batch's own: the one that is its own, by
+    the default limit or the given one, is not timed twice, and no other is
+    left out (FP64 by default: 256 threads, 4 CTAs, 128 octs on one CTA)."""
+    rng = np.random.default_rng(1)
+    levels = []
+    for o in (90, 1500):
+        lv, st = W.random_box_solve(rng, o, dt_hi=1.0)
+        L = ats.Level(ctx, lv)
+        L.build(st.dt, st.K, st.E, face_E=st.face_E, face_F=st.face_F)
+        levels.append((L, st))
+    precision = ats.ATS_PREC_MIXED if prec == "mixed" else ats.ATS_PREC_FP64
+    B = ats.Batch(ctx, [L for L, _ in levels], tol=5e-11, stop_rule=ats.ATS_STOP_CERTIFIED, precision=precision,
+                  res_cta_octs=limit)
+    r = B.autotune([st.E.copy() for _, st in levels], reps=1)
+    assert r["candidates"] == shapes
+    B.close()
+    for L, _ in levels:
+        L.close()
