@@ -234,7 +234,9 @@ typedef struct {
         /* in global memory), the faces across runs and the per-step sums through   */
         /* global memory, steps ordered by a grid barrier whose waits give up after */
         /* a bounded number of polls (the solve then ends with ATS_ERR_TIMEOUT);    */
-        /* such levels run one after another, after the other resident solves.     */
+        /* such levels run after the other resident solves, one after another      */
+        /* (FP64: up to 16 of them advance together, each with the bits it has     */
+        /* alone).                                                                  */
 
 /* initial guess of a solve (ats_solve_opts.x0) */
 #define ATS_X0_GIVEN 0 /* x_inout holds the initial guess on entry (default) */

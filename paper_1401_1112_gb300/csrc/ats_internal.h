@@ -256,8 +256,10 @@ int resident_smem_clusters(int threads, int cluster, int cap);
 int resident_smem_cap(int threads, int device);
 // The whole-GPU form of the resident solver of either bulk precision
 // (512-thread CTAs): one cooperative launch of `grid` CTAs (at most
-// resident_grid_ctas) solves gq[0, n_gq) one level at a time, each level split into `grid` contiguous runs; sums and
-// steps go through global memory and a grid barrier whose waits end after a
+// resident_grid_ctas) solves gq[0, n_gq), each level split into `grid`
+// contiguous runs, one level at a time (FP64: up to a.n_lock together, a
+// barrier carrying the sums of all of them); sums and steps go through global
+// memory and a grid barrier whose waits end after a
 // bounded number of polls (then *gerr is set and the solve ends with
 // ATS_ERR_TIMEOUT).
 cudaError_t launch_resident_grid(bool fp64, int grid, const ResArgs &a, cudaStream_t st);
@@ -280,9 +282,7 @@ cudaError_t launch_grid_barrier_probe(int grid, const ResArgs &a, int *out, cuda
 cudaError_t launch_grid_sum_probe(int grid, const ResArgs &a, int n, const float *value, const float *ref,
                                   float *total, int *slot, cudaStream_t st);
 
-// Start of a solve: e = 0 on every cell of every item, and x64 = src[solve]
-// where src (device array of device pointers) is non-null for that solve.
-// reset (may be null): the run state that the same launch puts in place.
+// The state of a run that launch_init puts in place.
 struct RunReset {
   // n_words 8-byte words of initial scalars, copied to the live and the final ones
   const unsigned long long *init;
@@ -302,6 +302,9 @@ struct RunReset {
   int *zero32[4];                 // ... and ints
   int n_zero32[4];
 };
+// Start of a solve: e = 0 on every cell of every item, and x64 = src[solve]
+// where src (device array of device pointers) is non-null for that solve.
+// reset (may be null): the run state that the same launch puts in place.
 cudaError_t launch_init(bool fp64, const SolveDev *solves, const WorkItem *items, int n_items,
                         const double *const *src, int grid, cudaStream_t st, const RunReset *reset = nullptr);
 // End of a solve: dst[solve] = x64 (2 x64 - E^n for Crank-Nicolson) where

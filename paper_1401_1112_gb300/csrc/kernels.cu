@@ -351,10 +351,6 @@ __device__ __forceinline__ void op_face(int n, const T *__restrict__ KT, const T
   }
 }
 
-// k_ref, axis A of an oct: acc -= the FP64 fluxes C (x_i - x_j) with the stored FP64
-// face coefficients C = h (K_i + K_j) (row A of this oct for the in-oct pairs
-// and the +A face, row A of the -A neighbour for the -A face), and the FP32
-// diagonal sums of the bulk precision.
 // The approximate reciprocal of the hardware (PTX rcp.approx, within one
 // ulp): for the Jacobi step z = D^-1 r of the resident solver's FP32 bulk, one
 // fixed value per cell for a whole inner solve, so the preconditioner stays
@@ -367,11 +363,12 @@ __device__ __forceinline__ float rcp_approx(float d) {
 
 // FP64 -> FP32 and back on the integer pipe: the hardware's conversions run at
 // the FP64 rate (measured: 16 cycles per warp and SM, 94 for a warp alone), and
-// the residual pass, FP64-bound, makes 16 per oct and x += e 8.  With the
-// fluxes taken straight from b - (1 + xd) x: 64 octs 219 -> 177 us, 512 ragged
-// levels 14.2 -> 13.7 ms, four-level radiation step 10.9 -> 10.5 ms.  Rounds to nearest, a tie away from
-// zero; zero, subnormals, infinities, NaN and what leaves FP32's range take the
-// hardware's conversion.
+// the residual pass, FP64-bound, makes 16 per oct and x += e 8.  Together with
+// the fluxes taken straight from b - (1 + xd) x (ref_axis) they save 4 % of a
+// batch of 512 ragged levels and of the four-level radiation step, a fifth of
+// a solve of 64 octs.  Rounds to nearest, a tie away from zero; zero,
+// subnormals, infinities, NaN and what leaves FP32's range take the hardware's
+// conversion.
 __device__ __forceinline__ float f32_of(double v) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
   if ((hi & 0x7fffffffu) - (897u << 20) >= (253u << 20)) return (float)v;
@@ -390,6 +387,10 @@ __device__ __forceinline__ T bulk_of(double v) {
   else return v;
 }
 
+// k_ref, axis A of an oct: acc -= the FP64 fluxes C (x_i - x_j) with the stored FP64
+// face coefficients C = h (K_i + K_j) (row A of this oct for the in-oct pairs
+// and the +A face, row A of the -A neighbour for the -A face), and the FP32
+// diagonal sums of the bulk precision.
 template <int A, typename T, bool kCoh = false>
 __device__ __forceinline__ void ref_axis(const SolveDev &sd, int o, const int (&nb)[6], const T *__restrict__ KT,
                                          T hT, const T (&KTo)[8], const double (&xv)[8], double (&acc)[8],
@@ -1585,10 +1586,10 @@ __device__ __forceinline__ bool oct_aligned(const void *p) { return ((uintptr_t)
 // of the half-step root (x + E^n) / 2) where src is given.  The caller's
 // arrays take 32-byte vectors when aligned, else one cell per access.
 // With a RunReset the launch also puts the run's state in place (scalars,
-// counters, queue heads, flags) and gathers the error flags: a dozen copies
-// and memsets of a few bytes each before, 2 to 4 us apiece on the host and the
-// stream.  With the results read back in one copy, a solve of 64 octs takes
-// 219 instead of 268 us, its operator build and the call included.
+// counters, queue heads, flags) and gathers the error flags: as copies and
+// memsets of a few bytes each they are a dozen operations of 2 to 4 us on the
+// host and the stream, about 50 us of a solve with the results read back in
+// one copy instead of four.
 template <typename T>
 __global__ void k_init(const SolveDev *__restrict__ solves, const WorkItem *__restrict__ items,
                        int n_items, const double *const *__restrict__ src, RunReset rs) {
@@ -2773,7 +2774,10 @@ __device__ bool grid_sum(Acc<T> (&a)[NA], ResShared<T> &sh, const ResArgs &ra, i
 // Fixed point: `ref`, a positive value every CTA holds (the current r.z), is
 // scaled into [2^24, 2^25); the first word sums the integer part (up to 2^44 per CTA),
 // the second the fraction in units of 2^-35 (offset by 2^36 to stay positive):
-// the quantum is 2^-59 of ref.  A total out of range or not finite adds 2^45
+// the quantum is 2^-59 of ref.  So 152 CTAs' rounding is coarser than that of
+// the (hi, lo) pairs of grid_sum once p.q falls below about r.z / 16, and below
+// the FP32 rounding that follows either down to about r.z / 2^29 (1 / alpha
+// there: a diagonal of 5e8).  A total out of range or not finite adds 2^45
 // to the second word; then every CTA takes grid_sum instead.
 constexpr int kFxWord = 64;  // 32-bit words between the fixed-point words (and before the first)
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }
@@ -3103,7 +3107,8 @@ __device__ bool res2_solve(const ResArgs &a, int s, ResShared<float> &sh, int &b
 // Measured (us per CG iteration of one level, refinement passes and call
 // included, shared-memory form -> this one): 512 octs on one CTA 4.0 -> 3.1,
 // 2 028 on one CTA 11.2 -> 8.3, 4 096 on 4 CTAs 6.8 -> 5.1, 8 000 on 8 CTAs
-// 7.3 -> 5.7, 32 768 on 16 CTAs 13.0 -> 9.3, on the whole GPU 11.2 -> 7.5.
+// 7.3 -> 5.7, 32 768 on 16 CTAs 13.0 -> 9.3, on the whole GPU 11.2 -> 6.2 (with
+// the staged rows and the sums of that form).
 
 namespace {
 
@@ -3394,7 +3399,7 @@ __device__ __forceinline__ void res3_e(const SolveDev &sd, int o, f32x2 alpha, c
 // Measured (stiff mixed level, us per iteration, tick path -> here): 262 144
 // octs 32.8 -> 20.2, 309 808 35.1 -> 20.6 (both on chip), 511 920 57.6 -> 33.5,
 // 1 000 000 124 -> 118; 2 097 152 245 -> 271, so the line lies at 6 144 octs
-// per CTA (kRunTail where a plan picks the path).
+// per CTA, below the size at which they meet (kRunTail where a plan picks the path).
 __device__ __forceinline__ void ldg_row(const float *p, f32x2 (&v)[4]) {
   asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
 }
@@ -3865,16 +3870,19 @@ __global__ void __launch_bounds__(NT, 1) k_res2_grid(ResArgs a) {
 // q = (I + dt A) z + beta q_prev, which needs no barrier after p:
 //   1. w = r - sum C z_j, p = z + beta p, q = w + beta q, the sum p.q;
 //   2. r -= alpha q, e += alpha p, z = r x (1 / D), the sums r.z and r.r.
-// The vectors come from L1 / L2 (14 rows of 64 bytes per oct and iteration
-// against 112 x 18 / 32 = 63 cycles of the pipe), so shared memory would not
-// pay.  What counts is the octs per SM: the groups are chosen for small runs
+// The vectors come from L1 / L2 (per oct and iteration 17 rows of 64 bytes of
+// its own -- 3 of C64, z, r, p, q read and p, q written; q, 1 / D, p, r, e read
+// and r, z, e written -- and the neighbours' z and coefficients, against
+// 112 x 18 / 32 = 63 cycles of the pipe), so shared memory would not pay.  What counts is the octs per SM: the groups are chosen for small runs
 // (kRun64 where a plan picks them), and levels above the clusters take the
 // whole-GPU form.  z is the only array other threads read (ld.global.cg after
 // the step's barrier); p, q, r, e and 1 / D belong to the thread that owns the
 // cell pair.  Non-leaf cells: C = 0 on all their faces, and r = z = p = q = 0.
 // Measured, certified 5e-11, build included: 128 levels of 64..2 048 octs
-// 27.2 -> 2.67 ms (one CTA of 256 threads each before), 4 096 octs 4.52 -> 0.90
-// ms and 32 736 octs 6.53 -> 2.03 ms (tick path before).
+// 2.67 ms (27.2 with one CTA of 256 threads each and no stored 1 / D), 4 096
+// octs 0.87 ms (tick path 4.52), 32 736 octs 2.0 ms (6.53), solves alone of
+// 262 144 octs 9.2 ms (25.7), 1 000 000 octs 32.3 (96.8), 2 000 000 octs 64.5
+// (187.7): no size at which the tick path is the better one.
 
 namespace {
 
@@ -3902,7 +3910,9 @@ __device__ __forceinline__ double ld1_cg(const double *p) {
   asm volatile("ld.global" ATS_RES_LD ".f64 %0, [%1];" : "=d"(v) : "l"(p));
   return v;
 }
-__device__ __forceinline__ Pair64 ldp_rw(const void *base, int u) {  // this thread's own
+// ... by a thread of this CTA, behind a barrier (the unit's own thread, except
+// in lockstep, where the thread of a unit changes from step to step)
+__device__ __forceinline__ Pair64 ldp_rw(const void *base, int u) {
   Pair64 v;
   asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.a), "=d"(v.b) : "l"((const double *)base + 2 * (size_t)u));
   return v;
@@ -4008,8 +4018,8 @@ __device__ __forceinline__ void resd_upd(const SolveDev &sd, int u, double alpha
   rr.add(r.b, r.b);
 }
 
-// The residual r = b - (1 + xd) x - sum C (x_i - x_j) (the form of ref_axis),
-// D = 1 + xd + sum C, z = r x (1 / D) on unit u.
+// The residual r = b - ((1 + xd) x + sum C (x_i - x_j)), the fluxes summed
+// first, D = 1 + xd + sum C, z = r x (1 / D) on unit u.
 __device__ __forceinline__ void resd_ref(const SolveDev &sd, int u, bool want_x, Acc<double> &rr, Acc<double> &xx,
                                          Acc<double> &rz) {
   const Stencil64 s = resd_stencil(sd, u);
@@ -4151,7 +4161,7 @@ __device__ void resd_solve(const ResArgs &a, int s, ResShared<double> &sh, int &
 
 // ---- the whole-GPU form: several levels in lockstep ----
 // A level alone leaves the FP64 pipes idle while its sums travel (4 096 octs:
-// 1.1 us of pipe per 9.7 us step), so the launch advances up to kLock levels
+// 1.1 us of pipe per 9.7 us step), so the launch advances up to kResLock levels
 // of its queue together: a superstep does the next pass of every level in
 // flight (residual, step 1, step 2 or x += e) on this CTA's run of that level,
 // then one grid barrier carries all their sums, which warp k merges for slot

@@ -259,8 +259,8 @@ struct Plan {
   int n_bq = 0, n_cq = 0, n_tq = 0, n_tick = 0, n_tick_items = 0;
   int n_mq = 0;  // mode 5: the middle clusters (res_cluster_mid CTAs)
   // mode 4: the whole-GPU form (one cooperative launch of res_grid_all CTAs
-  // takes these solves one after another); its barrier, partial sums and
-  // give-up flag
+  // takes these solves one after another, FP64 up to res_lock of them
+  // together); its barrier, partial sums and give-up flag
   int n_gq = 0, res_grid_all = 0;
   int res_lock = 1;  // FP64: levels of the whole-GPU launch in flight at once
   // the split of the device's CTA slots between the three resident launches:
@@ -642,8 +642,11 @@ constexpr int64_t kCta32 = 2048;
 constexpr int64_t kMaxOcts32 = 16384;
 // FP32-bulk levels take the whole-GPU form up to this many octs per CTA: the
 // first 2 048 of a run stay on chip, the rest is streamed from L2 and HBM,
-// where the tick path's larger grid does better once HBM bounds it (measured
-// at 1 000 000 octs: 25.7 against 27.2 ms, at 2 097 152: 59.1 against 53.1).
+// where the tick path's larger grid does better once HBM bounds it.  Measured,
+// this form and the tick path (ms, stiff level): 697 048 octs 14.7 / 24.0,
+// 903 264 21.8 / 25.9, 1 000 000 24.8 / 27.7, 1 202 252 31.5 / 30.9, 1 494 540
+// 39.8 / 40.6, 2 097 152 56.2 / 52.8.  The line lies below the sizes at which
+// the two are equal, so that every size that takes this form gains by it.
 constexpr int64_t kRunTail = 6144;
 
 ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const ats_solve_opts *opts_in,
@@ -761,9 +764,10 @@ ats_status plan_create(ats_context *ctx, ats_level *const *levels, int n, const 
     P->res_cluster_mid = 0;
   {
     const bool res_ok = o.sched != ATS_SCHED_TICK && o.stop_rule != ATS_STOP_PAPER;
-    // default limit: mixed precision 16384 octs (the shared-memory form
-    // beats a whole-GPU tick loop up to about there for one solve alone);
-    // FP64 (the global-memory form) 2048
+    // default limit: the octs that the largest clusters take at about a
+    // thousand (FP64: 128) octs per CTA; above it the whole-GPU form, whose
+    // solves run one after another (16 000 octs 1.28 ms on 16 CTAs, seven
+    // such clusters at once)
     const int64_t max_octs = o.sched == ATS_SCHED_RESIDENT
                                  ? INT64_MAX
                                  : (o.res_max_octs > 0 ? o.res_max_octs : (P->fp64 ? 2048 : kMaxOcts32));
@@ -1279,6 +1283,14 @@ void plan_bytes(const Plan *P, const unsigned long long cells[kCellCounters], do
   *upd_b = 7 * w * cells[2] + (16 + 2 * w) * cells[3];
 }
 
+// Where a run of the plan puts what its caller reads: the final scalars, the
+// levels' error flags and the negative-result flags (one per solve), and an
+// int set to zero at the start (or null).
+struct RunOut {
+  SolveScalars *fin;
+  int *flags, *neg, *zero;
+};
+
 // Enqueue the start of a run: refresh the solve descriptors of levels
 // rebuilt since the plan was made, copy x in (device x is read in place,
 // host x goes through one staging buffer, one copy per run of levels whose
@@ -1288,14 +1300,6 @@ void plan_bytes(const Plan *P, const unsigned long long cells[kCellCounters], do
 // holds; the reset itself is device to device.  capture: st is under stream
 // capture, so nothing may come from the host (device x only, and every
 // upload already resident, else ATS_ERR_INVALID_ARG).
-// Where a run of the plan puts what its caller reads: the final scalars, the
-// levels' error flags and the negative-result flags (one per solve), and an
-// int set to zero at the start (or null).
-struct RunOut {
-  SolveScalars *fin;
-  int *flags, *neg, *zero;
-};
-
 ats_status plan_begin(Plan *P, double *const *x_inout, std::vector<int64_t> &off, const RunOut &ro,
                       bool capture = false) {
   ats_context *ctx = P->ctx;
